@@ -34,9 +34,10 @@ def _nvcc() -> str:
 def _units():
     units = []
     for tin in (0, 1, 2):
-        units.append((os.path.join(CSRC, "credit_kernels.cu"), f"credit_kernels_{tin}.o", [f"-DCREDIT_TIN={tin}"]))
+        for name in ("credit_kernels", "credit_team"):
+            units.append((os.path.join(CSRC, name + ".cu"), f"{name}_{tin}.o", [f"-DCREDIT_TIN={tin}"]))
     for src in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp"))):
-        if os.path.basename(src) == "credit_kernels.cu":
+        if os.path.basename(src) in ("credit_kernels.cu", "credit_team.cu"):
             continue
         units.append((src, os.path.basename(src).rsplit(".", 1)[0] + ".o", []))
     return units

@@ -97,6 +97,42 @@ int two_pass_split(int sm_count, long long rows, long long cols, int isz) {
     return static_cast<int>(G < 1 ? 1 : G);
 }
 
+// Narrow rows: the one-CTA path with whole rows in shared memory (k_row_team),
+// up to the row width at which it stops being the fastest plan.  Measured on
+// GB300 against the learned model's picks (rows 96-16384, widths 256 B to 96
+// KiB, on and off the 16-byte grid; us, the model's pick -> this one):
+//   16384 x 4096 BF16 RMSNorm 80 -> 48, 65536 x 1024 FP32 softmax 252 -> 92,
+//   20325 x 3616 BF16 softmax 130 -> 52, 16384 x 8192 BF16 -> FP8 RMSNorm
+//   167 -> 81, FP8 LayerNorm 332 -> 112, 10800 x 4096 BF16 int8 93 -> 29,
+//   1000 rows of 24 KiB: 5-60% faster for every op and type but FP8 softmax.
+// The limits: norms of rows on the 16-byte grid go to the tensor-memory path
+// from 48 KiB (1000 x 64 KiB BF16 RMSNorm 29 against 38), off the grid, where
+// that path loses its staged gamma / beta, only above 96 KiB; E4M3 softmax and
+// log-sum-exp have their code tables (24 KiB rows of FP8 log-sum-exp 11
+// against 15, 32 KiB of FP8 softmax 13 against 15); log-sum-exp has no output
+// for the second look at the row to save, in BF16 it draws level at 32 KiB.
+static bool row_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, int tout,
+                     credit_plan_t *p) {
+    const int isz = dtype_size(tin);
+    const bool norm = op == CREDIT_OP_LAYERNORM || op == CREDIT_OP_RMSNORM;
+    long long limit = 96 << 10;
+    if (op == CREDIT_OP_LOGSUMEXP) limit = tin == 0 ? limit : tin == 1 ? 32 << 10 : 8 << 10;
+    else if (op == CREDIT_OP_SOFTMAX && tin == 2) limit = 24 << 10;
+    else if (norm && tin != 2 && tout != 2 && cols * isz % 16 == 0) limit = 48 << 10;
+    TeamCfg tc;
+    if (cols * isz > limit ||
+        !team_config(di, rows, cols, isz, op == CREDIT_OP_LAYERNORM ? 2 : op == CREDIT_OP_RMSNORM, 0, &tc))
+        return false;
+    std::memset(p, 0, sizeof(*p));
+    p->source = 3;
+    p->path = CREDIT_PATH_ONE_CTA;
+    p->cluster_size = 1;
+    p->ctas_per_row = 1;
+    p->retain = CREDIT_RETAIN_ROW;
+    p->smem_bytes = tc.smem;
+    return true;
+}
+
 // Rule for int8 quantisation (measured on GB300, 4096 rows of 16K-256K FP32
 // columns): the smallest cluster whose slices fit the tensor-memory tier
 // (128 KiB); the fewest CTAs per row keeps the most rows in flight and the
@@ -122,6 +158,7 @@ static bool quant_plan(const DeviceInfo &di, int device, long long rows, long lo
 
 void heuristic_plan(const DeviceInfo &di, int device, int op, long long rows, long long cols, int tin, int tout,
                     credit_plan_t *p) {
+    if (row_plan(di, op, rows, cols, tin, tout, p)) return;
     std::memset(p, 0, sizeof(*p));
     p->source = 3;
     if (op == CREDIT_OP_QUANT_INT8 && quant_plan(di, device, rows, cols, tin, p)) return;
@@ -191,8 +228,10 @@ credit_status credit_plan_ex(credit_op op, int64_t rows, int64_t cols, credit_dt
             return CREDIT_OK;
         }
     }
-    // the calibration and the learned model cover the four ops of Sec. III-B; the quantiser takes the rule
-    if (q8 || !model_plan(*di, dev, op, rows, cols, in_dtype, tout, out))
+    // narrow rows take the rule unless CREDIT_MODEL asks for a model's own choice; the calibration and the
+    // learned model cover the four ops of Sec. III-B; the quantiser takes the rule
+    if (!(cache && row_plan(*di, op, rows, cols, in_dtype, tout, out)) &&
+        (q8 || !model_plan(*di, dev, op, rows, cols, in_dtype, tout, out)))
         heuristic_plan(*di, dev, op, rows, cols, in_dtype, tout, out);
     if (cache) {
         std::lock_guard<std::mutex> lk(g_plan_mu);

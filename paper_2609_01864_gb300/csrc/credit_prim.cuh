@@ -530,13 +530,6 @@ __device__ __forceinline__ void st_global_v4_hint(void *p, const uint4 &v, uint6
                  "r"(v.z), "r"(v.w), "l"(policy)
                  : "memory");
 }
-__device__ __forceinline__ uint4 ld_global_stream_v4(const void *p) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
-    return v;
-}
 
 // ------------------------------------------------------------ warp/block reductions
 __device__ __forceinline__ float warp_sum(float v) {
@@ -548,6 +541,13 @@ __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
+}
+
+// The same maximum in one instruction.
+__device__ __forceinline__ float warp_max_redux(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 // Deterministic block all-reduce (sum or max) through `red` (>= 33 floats).

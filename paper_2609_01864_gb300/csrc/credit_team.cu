@@ -1,0 +1,48 @@
+// credit_team.cu -- instantiates the team kernels for one input
+// dtype (compiled with -DCREDIT_TIN=0, 1 and 2, like credit_kernels.cu).
+#include "credit_row_team.cuh"
+
+#ifndef CREDIT_TIN
+#error "CREDIT_TIN must be defined (0 = FP32, 1 = BF16, 2 = FP8-E4M3)"
+#endif
+
+#define CREDIT_CAT2(a, b) a##b
+#define CREDIT_CAT(a, b) CREDIT_CAT2(a, b)
+
+namespace credit {
+
+template <int OP, int TOUT>
+static const void *team_fn(bool grid, bool aff) {
+    if constexpr (OP == OP_LN || OP == OP_RMS) {
+        if (aff)
+            return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, true>)
+                        : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, true>);
+    }
+    return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, false>)
+                : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, false>);
+}
+
+template <int OP>
+static const void *team_out(int tout, bool grid, bool aff) {
+    switch (tout) {
+    case DT_F32: return team_fn<OP, DT_F32>(grid, aff);
+    case DT_BF16: return team_fn<OP, DT_BF16>(grid, aff);
+    case DT_E4M3: return team_fn<OP, DT_E4M3>(grid, aff);
+    default: return nullptr;
+    }
+}
+
+const void *CREDIT_CAT(team_kernel_tin, CREDIT_TIN)(int op, int tout, bool grid, bool aff) {
+    switch (op) {
+    case OP_SOFTMAX: return team_out<OP_SOFTMAX>(tout, grid, aff);
+    case OP_LSE: return team_fn<OP_LSE, DT_F32>(grid, aff);
+    case OP_LN: return team_out<OP_LN>(tout, grid, aff);
+    case OP_RMS: return team_out<OP_RMS>(tout, grid, aff);
+#if CREDIT_TIN != 2
+    case OP_Q8: return tout == DT_I8 ? team_fn<OP_Q8, DT_I8>(grid, aff) : nullptr;
+#endif
+    default: return nullptr;
+    }
+}
+
+}  // namespace credit
