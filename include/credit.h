@@ -376,8 +376,10 @@ typedef struct {
  *       CREDIT_ERR_UNSUPPORTED, with nothing launched.
  *   TWO_PASS (G = ctas_per_row >= 1)  a statistics sweep over HBM and a
  *       second sweep that rereads a and dy; G > 1 splits a row over G CTAs
- *       whose partials go through the device workspace between two launches.
- *       Any alignment.
+ *       whose partials go through the device workspace between two launches;
+ *       G = 1 keeps rows of up to 96 KiB per array that fit in shared memory
+ *       between the two looks.  Any alignment (fastest where a, dy and dx
+ *       start at the same offset from a 16-byte boundary).
  * fill_share and retain must be 0.  Asynchronous on `stream`; the statuses
  * of credit_run_ex.
  */
@@ -386,12 +388,13 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
 /*
  * credit_plan_bwd -- a plan for (op, rows, cols, dtype) of the backward ops,
  * assuming 16-byte aligned rows (credit_run_bwd falls back to TWO_PASS for
- * unaligned rows when planning itself): the fused two-pass path for rows of
- * at most 16 KiB per array, else the staged path with the smallest cluster
- * size whose slices (two row buffers of a and dy, and gamma for the norms)
- * fit, else the split two-pass path.  The logits and pair ops, whose per-row
- * merges grow with the cluster size, are staged only for P <= 4 with slices
- * of at most 64 KiB per array.  source = 3 (built-in rule).
+ * unaligned rows when planning itself): the one-CTA two-pass path for rows of
+ * at most 16 KiB per array (pair ops 24 KiB, logits ops 64 KiB), else the
+ * staged path with the smallest cluster size whose slices (two row buffers of
+ * a and dy, and gamma for the norms) fit, else the split two-pass path.  The
+ * logits and pair ops, whose per-row merges grow with the cluster size, are
+ * staged only for P <= 4 with slices of at most 64 KiB per array (pair ops at
+ * P = 4: the largest that fit).  source = 3 (built-in rule).
  */
 credit_status credit_plan_bwd(int32_t op, int64_t rows, int64_t cols, credit_dtype dtype, credit_plan_t *out);
 

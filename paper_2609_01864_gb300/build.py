@@ -1,6 +1,6 @@
 """Build libcredit.so in-tree with nvcc for sm_103a (GB300).
 
-Every translation unit compiles in parallel; the kernel TU compiles once per
+Every translation unit compiles in parallel; the kernel TUs compile once per
 input dtype.  The result lands in ``paper_2609_01864_gb300/_build/``.  No
 cmake, no torch C++ extension: the library exposes a plain C ABI and is
 loaded with ctypes.
@@ -36,6 +36,8 @@ def _units():
     for tin in (0, 1, 2):
         for name in ("credit_kernels", "credit_team"):
             units.append((os.path.join(CSRC, name + ".cu"), f"{name}_{tin}.o", [f"-DCREDIT_TIN={tin}"]))
+    for dt in (0, 1):
+        units.append((os.path.join(CSRC, "credit_bwd.cu"), f"credit_bwd_{dt}.o", [f"-DCREDIT_BWD_DT={dt}"]))
     for src in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp"))):
         if os.path.basename(src) in ("credit_kernels.cu", "credit_team.cu"):
             continue

@@ -58,10 +58,17 @@
 
 #include "../../include/credit.h"
 #include "credit_host.h"
-#include "credit_rows.cuh"
+#include "credit_row_team.cuh"
 
 namespace credit {
 extern std::atomic<long long> g_launch_count;
+
+// Kernel table of one (op, dtype).
+struct BwdKernels {
+    const void *staged;
+    const void *fused[2], *stats[2], *apply[2];  // [rows off the 16-byte grid]
+    const void *team[2][2];  // [rows on the 16-byte grid][gamma in shared memory]
+};
 
 namespace {
 
@@ -78,7 +85,16 @@ constexpr int kBwdThreads = 512;
 constexpr int kBwdCtrl = 1792;             // control area before the row buffers (bytes)
 constexpr int kBwdMaxChunks = 8;           // chunks (mbarriers) per row buffer
 constexpr uint32_t kBwdPiece = 32768;      // bytes per bulk copy instruction
-constexpr long long kBwdFusedMaxBytes = 16384;  // planner: fused two-pass up to this many bytes per array row
+constexpr long long kBwdTeamMaxBytes = 98304;  // bytes per array row up to which k_bwd_team is used (G = 1)
+// Planner: rows of at most this many bytes per array on the 16-byte grid take
+// the one-CTA two-pass path (k_bwd_team), wider ones the staged path.
+// Measured (GB300, 1000 and 6000 rows, staged -> k_bwd_team): up to 16 KiB the
+// team kernel is ahead for every op (1.05-2.6x); at 24 KiB the plain sums are
+// level (0.9-1.1x), the pair ops 1.1-1.6x, the logits ops 1.2-1.7x and still
+// 1.03-1.26x at 64 KiB.
+inline long long bwd_team_bytes(int op) {
+    return op == BOP_SMLOGITS || op == BOP_XENT ? 65536 : op == BOP_WVAR || op == BOP_PEARSON ? 24576 : 16384;
+}
 
 struct BwdArgs {
     const unsigned char *a, *dy;
@@ -763,29 +779,41 @@ __global__ void __launch_bounds__(kBwdThreads, 1) k_bwd_staged(const BwdArgs p) 
 }
 
 // ------------------------------------------------------------------ two-pass
-// Units of CTA j of G for one row: 16-byte groups when the row's three
-// arrays are 16-byte aligned (plus the tail elements, by CTA G - 1), single
-// elements otherwise.
+// Units of CTA j of G for one row: where the row's arrays share their phase
+// on the 16-byte grid, the full 16-byte groups after the head (plus the head
+// elements, by CTA 0, and the tail elements, by CTA G - 1); single elements
+// otherwise.
 struct BwdSpan {
     bool vec;
-    long long lo, hi;        // groups (vec) or elements
-    long long t_lo, t_hi;    // tail elements handled here (vec only)
+    int h0;                // head elements of the row (OFF only)
+    long long lo, hi;      // groups (vec) or elements
+    long long t_lo, t_hi;  // tail elements handled here (vec only)
+    bool first;            // CTA 0 (OFF only)
 };
 
-template <int DT>
+template <int DT, bool OFF>
 __device__ __forceinline__ BwdSpan bwd_span(const BwdArgs &p, long long row, int j, int G) {
     constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V;
-    const size_t off = static_cast<size_t>(row * p.ld) * isz;
-    const bool vec = ((reinterpret_cast<uintptr_t>(p.a + off) | reinterpret_cast<uintptr_t>(p.dy + off) |
-                       reinterpret_cast<uintptr_t>(p.dx + off) |
-                       (p.dx2 ? reinterpret_cast<uintptr_t>(p.dx2 + off) : 0)) & 15u) == 0;
     BwdSpan s;
-    s.vec = vec;
-    if (vec) {
-        const long long Gq = p.cols / V;
+    s.h0 = 0;
+    s.first = j == 0;
+    if constexpr (OFF) {
+        const uint32_t u = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.a));
+        auto diff = [&](const unsigned char *q) { return static_cast<uint32_t>(reinterpret_cast<uintptr_t>(q)) ^ u; };
+        s.vec = ((diff(p.dy) | diff(p.dx) | (p.dx2 ? diff(p.dx2) : 0u)) & 15u) == 0 && u % isz == 0;
+        const uint32_t mis = (u + static_cast<uint32_t>(row * p.ld) * isz) & 15u;
+        if (s.vec) s.h0 = static_cast<int>(min(static_cast<long long>(((16u - mis) & 15u) / isz), p.cols));
+    } else {
+        const size_t off = static_cast<size_t>(row * p.ld) * isz;
+        s.vec = ((reinterpret_cast<uintptr_t>(p.a + off) | reinterpret_cast<uintptr_t>(p.dy + off) |
+                  reinterpret_cast<uintptr_t>(p.dx + off) | (p.dx2 ? reinterpret_cast<uintptr_t>(p.dx2 + off) : 0)) &
+                 15u) == 0;
+    }
+    if (s.vec) {
+        const long long Gq = (p.cols - s.h0) / V;
         s.lo = group_split(Gq, j, G);
         s.hi = group_split(Gq, j + 1, G);
-        s.t_lo = j == G - 1 ? Gq * V : p.cols;
+        s.t_lo = j == G - 1 ? s.h0 + Gq * V : p.cols;
         s.t_hi = p.cols;
     } else {
         s.lo = group_split(p.cols, j, G);
@@ -795,58 +823,88 @@ __device__ __forceinline__ BwdSpan bwd_span(const BwdArgs &p, long long row, int
     return s;
 }
 
-template <int OP, int DT>
+// The elements outside the groups of a span (vec: head and tail; else all of it): fn(element).
+template <bool OFF, class F>
+__device__ __forceinline__ void bwd_singles(const BwdSpan &s, F &&fn) {
+    if (OFF && s.first && static_cast<int>(threadIdx.x) < s.h0) fn(static_cast<long long>(threadIdx.x));
+    const long long e_lo = s.vec ? s.t_lo : s.lo, e_hi = s.vec ? s.t_hi : s.hi;
+    for (long long i = e_lo + threadIdx.x; i < e_hi; i += blockDim.x) fn(i);
+}
+
+// fn(first element, a, dy, gamma) on every group of a span.  OFF: rows off the
+// 16-byte grid, whose gamma lies at any phase (ldg_shift) and whose two groups
+// of each array in flight repay the registers (1440 x 46161 FP32 LayerNorm dx
+// 220 us with two, 227 with one; on the grid the plain loop with one is 3%
+// ahead, its 32-36 registers leave room for four CTAs of 512 threads).
+template <int OP, int DT, bool OFF, class F>
+__device__ __forceinline__ void bwd_groups(const BwdArgs &p, long long row, const BwdSpan &s, F &&fn) {
+    constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V, U = OFF ? 2 : 1;
+    if (!s.vec) return;
+    const bool g_vec = p.gamma == nullptr || (reinterpret_cast<uintptr_t>(p.gamma) & 15u) == 0;
+    const size_t off = static_cast<size_t>(row * p.ld + s.h0) * isz;
+    const float *gam = kNorm<OP> ? p.gamma : nullptr;
+    for (long long k0 = s.lo + threadIdx.x; k0 < s.hi; k0 += U * blockDim.x) {
+        uint4 wa[U], wd[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long k = k0 + u * blockDim.x;
+            if (u == 0 || k < s.hi) {
+                wa[u] = ld_global_v4(p.a + off + 16 * k);
+                wd[u] = ld_global_v4(p.dy + off + 16 * k);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long k = k0 + u * blockDim.x;
+            if (u > 0 && k >= s.hi) continue;
+            float fa[V], fd[V], fg[V];
+            decode_group<DT>(wa[u], fa, 1.0f);
+            decode_group<DT>(wd[u], fd, 1.0f);
+            if constexpr (OFF) ldg_shift<V>(gam, s.h0 + k * V, p.cols, 1.0f, fg);
+            else load_affine<V>(gam, k * V, g_vec, 1.0f, fg);
+            fn(s.h0 + k * V, fa, fd, fg);
+        }
+    }
+}
+
+template <int OP, int DT, bool OFF>
 __device__ __forceinline__ BwdState<OP> bwd_sums(const BwdArgs &p, long long row, const BwdRow<OP> &R,
                                                  const BwdSpan &s) {
     constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V;
     const size_t off = static_cast<size_t>(row * p.ld) * isz;
-    const bool g_vec = p.gamma == nullptr || (reinterpret_cast<uintptr_t>(p.gamma) & 15u) == 0;
     const float *gam = kNorm<OP> ? p.gamma : nullptr;
     BwdState<OP> st;
-    if (s.vec) {
-        for (long long k = s.lo + threadIdx.x; k < s.hi; k += blockDim.x) {
-            float fa[V], fd[V], fg[V];
-            decode_group<DT>(ld_global_v4(p.a + off + 16 * k), fa, 1.0f);
-            decode_group<DT>(ld_global_v4(p.dy + off + 16 * k), fd, 1.0f);
-            load_affine<V>(gam, k * V, g_vec, 1.0f, fg);
-            st.template add<V>(R, fa, fd, fg);
-        }
-    }
-    const long long e_lo = s.vec ? s.t_lo : s.lo, e_hi = s.vec ? s.t_hi : s.hi;
-    for (long long i = e_lo + threadIdx.x; i < e_hi; i += blockDim.x)
+    bwd_groups<OP, DT, OFF>(p, row, s, [&](long long, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
+        st.template add<V>(R, fa, fd, fg);
+    });
+    bwd_singles<OFF>(s, [&](long long i) {
         st.add1(R, decode_one<DT>(p.a + off + i * isz, 1.0f), decode_one<DT>(p.dy + off + i * isz, 1.0f),
                 gam ? gam[i] : 1.0f);
+    });
     return st;
 }
 
-template <int OP, int DT>
+template <int OP, int DT, bool OFF>
 __device__ __forceinline__ void bwd_apply(const BwdArgs &p, long long row, const BwdRow<OP> &R, const BwdSpan &s,
                                           const Coef &kc) {
     constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V;
     const size_t off = static_cast<size_t>(row * p.ld) * isz;
-    const bool g_vec = p.gamma == nullptr || (reinterpret_cast<uintptr_t>(p.gamma) & 15u) == 0;
     const float *gam = kNorm<OP> ? p.gamma : nullptr;
-    if (s.vec) {
-        for (long long k = s.lo + threadIdx.x; k < s.hi; k += blockDim.x) {
-            float fa[V], fd[V], fg[V], y[V];
-            decode_group<DT>(ld_global_v4(p.a + off + 16 * k), fa, 1.0f);
-            decode_group<DT>(ld_global_v4(p.dy + off + 16 * k), fd, 1.0f);
-            load_affine<V>(gam, k * V, g_vec, 1.0f, fg);
-            if constexpr (kPair<OP>) {
-                float y2[V];
+    bwd_groups<OP, DT, OFF>(p, row, s, [&](long long i, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
+        float y[V];
+        if constexpr (kPair<OP>) {
+            float y2[V];
 #pragma unroll
-                for (int v = 0; v < V; ++v) R.dx_pair(fa[v], fd[v], kc, y[v], y2[v]);
-                store_group<DT, V>(p.dx + off + 16 * k, y, true);
-                store_group<DT, V>(p.dx2 + off + 16 * k, y2, true);
-            } else {
+            for (int v = 0; v < V; ++v) R.dx_pair(fa[v], fd[v], kc, y[v], y2[v]);
+            store_group<DT, V>(p.dx + off + i * isz, y, true);
+            store_group<DT, V>(p.dx2 + off + i * isz, y2, true);
+        } else {
 #pragma unroll
-                for (int v = 0; v < V; ++v) y[v] = R.dx(fa[v], fd[v], fg[v], kc);
-                store_group<DT, V>(p.dx + off + 16 * k, y, true);
-            }
+            for (int v = 0; v < V; ++v) y[v] = R.dx(fa[v], fd[v], fg[v], kc);
+            store_group<DT, V>(p.dx + off + i * isz, y, true);
         }
-    }
-    const long long e_lo = s.vec ? s.t_lo : s.lo, e_hi = s.vec ? s.t_hi : s.hi;
-    for (long long i = e_lo + threadIdx.x; i < e_hi; i += blockDim.x) {
+    });
+    bwd_singles<OFF>(s, [&](long long i) {
         const float av = decode_one<DT>(p.a + off + i * isz, 1.0f), dv = decode_one<DT>(p.dy + off + i * isz, 1.0f);
         if constexpr (kPair<OP>) {
             float o1, o2;
@@ -856,18 +914,18 @@ __device__ __forceinline__ void bwd_apply(const BwdArgs &p, long long row, const
         } else {
             store_one<DT>(p.dx + off + i * isz, R.dx(av, dv, gam ? gam[i] : 1.0f, kc));
         }
-    }
+    });
 }
 
 // G = 1: one CTA per row, both sweeps.
-template <int OP, int DT>
+template <int OP, int DT, bool OFF>
 __global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_fused(const BwdArgs p) {
     __shared__ float red[128];
     const long long row = p.row0 + blockIdx.x;
     BwdRow<OP> R;
     R.load(p, row);
-    const BwdSpan s = bwd_span<DT>(p, row, 0, 1);
-    const BwdState<OP> t = bwd_sums<OP, DT>(p, row, R, s);
+    const BwdSpan s = bwd_span<DT, OFF>(p, row, 0, 1);
+    const BwdState<OP> t = bwd_sums<OP, DT, OFF>(p, row, R, s);
     Coef kc;
     if constexpr (kPair<OP>) {
         float tot[kPairState<OP>];
@@ -880,20 +938,20 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_fused(const BwdArgs p) {
         const float2 tot = block_sum2(t.s0, t.s1, red);
         kc = row_coeffs<OP>(tot.x, tot.y, p.cols);
     }
-    bwd_apply<OP, DT>(p, row, R, s, kc);
+    bwd_apply<OP, DT, OFF>(p, row, R, s, kc);
 }
 
 // G > 1, launch 1: partial sums of CTA j of row lr into ws[lr][j][0..1] (logits ops: the state into
 // ws[lr][j][0..2] of a 4-float record; pair ops: the sums into an 8-float record).
-template <int OP, int DT>
+template <int OP, int DT, bool OFF>
 __global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_stats(const BwdArgs p) {
     __shared__ float red[128];
     const int G = p.G, j = blockIdx.x % G;
     const long long lr = blockIdx.x / G, row = p.row0 + lr;
     BwdRow<OP> R;
     R.load(p, row);
-    const BwdSpan s = bwd_span<DT>(p, row, j, G);
-    const BwdState<OP> t = bwd_sums<OP, DT>(p, row, R, s);
+    const BwdSpan s = bwd_span<DT, OFF>(p, row, j, G);
+    const BwdState<OP> t = bwd_sums<OP, DT, OFF>(p, row, R, s);
     if constexpr (kPair<OP>) {
         float tot[kPairState<OP>];
         block_merge_pair<OP>(t, red, tot);
@@ -918,8 +976,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_stats(const BwdArgs p) {
 }
 
 // G > 1, launch 2: the row totals (partials in the fixed order j = 0..G-1), then dx.
-template <int OP, int DT>
-__global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_apply(const BwdArgs p) {
+template <int OP, int DT, bool OFF>
+__global__ void __launch_bounds__(kBwdThreads, kPair<OP> && !OFF ? 4 : 1) k_bwd_tp_apply(const BwdArgs p) {
     const int G = p.G, j = blockIdx.x % G;
     const long long lr = blockIdx.x / G, row = p.row0 + lr;
     BwdRow<OP> R;
@@ -947,38 +1005,397 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_tp_apply(const BwdArgs p) {
         }
         kc = row_coeffs<OP>(S0, S1, p.cols);
     }
-    bwd_apply<OP, DT>(p, row, R, bwd_span<DT>(p, row, j, G), kc);
+    bwd_apply<OP, DT, OFF>(p, row, R, bwd_span<DT, OFF>(p, row, j, G), kc);
 }
 
-struct BwdKernels {
-    const void *staged, *fused, *stats, *apply;
-};
+// ------------------------------------------------------------------ rows in shared memory (TWO_PASS, G = 1)
+// The one-CTA-per-row two-pass path for rows that fit shared memory: the same
+// two looks at the row, the second one at shared memory.  The scheme of
+// k_row_team: one persistent CTA per SM, teams of T threads on rows of their
+// own, S stages of (a row, dy row) per team filled by bulk copies, gamma in
+// planes (AFF), rows cut on the 16-byte grid of a's address (GRID: all rows
+// start and end on it), edge elements one per thread, loaded one row ahead
+// with the row's saved statistics.  Shared memory makes a further look at the
+// row cheap, so the logits ops take the maximum first and the pair ops the
+// means first (plain sums; no online states and no Chan merges).
+constexpr int kBwdTeamRed = 4 * 96;  // floats of reduction scratch per team: 4 arrays of 3 sums x 32 warps
 
-template <int OP, int DT>
+__host__ __device__ constexpr int bwd_team_ctrl(int T, int teams) {
+    return kTeamMaxTeams * kTeamMaxStages * 8 + (T > 32 ? teams * kBwdTeamRed * 4 : 0);
+}
+
+// K sums over a team's T threads (the tree of team_reduce).
+template <int K>
+__device__ __forceinline__ void team_sums(float (&v)[K], float *red, int bar, int T) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = warp_sum(v[k]);
+    if (T == 32) return;
+    const int lane = threadIdx.x & 31, nw = T >> 5;
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) red[32 * k + (threadIdx.x >> 5)] = v[k];
+    }
+    named_bar_sync(bar, T);
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = warp_sum(lane < nw ? red[32 * k + lane] : 0.0f);
+}
+
+__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+
+template <int OP, int DT, bool GRID, bool AFF>
+__global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V, NP = V / 4;
+    const int T = blockDim.x, t = threadIdx.x, team = threadIdx.y, teams = blockDim.y, S = p.nbuf;
+    const int N = static_cast<int>(p.cols), gmax = N / V;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem) + team * kTeamMaxStages;
+    float *red = reinterpret_cast<float *>(smem + kTeamMaxTeams * kTeamMaxStages * 8) + (T > 32 ? team * kBwdTeamRed : 0);
+    const int np = affine_np<NP>(N);
+    float *gsm = reinterpret_cast<float *>(smem + bwd_team_ctrl(T, teams));
+    const AffinePlanes gp{gsm, np};
+    const uint32_t arr = gmax * 16u;  // bytes of one array's stage
+    unsigned char *stages = reinterpret_cast<unsigned char *>(gsm + (AFF ? NP * np * 4 : 0)) +
+                            static_cast<size_t>(team) * S * 2 * arr;
+    const long long stride = static_cast<long long>(gridDim.x) * teams;
+    const long long row_first = static_cast<long long>(blockIdx.x) * teams + team;
+
+    struct Geo {
+        int h0, G, t0;
+    };
+    auto offset = [&](long long row) { return static_cast<size_t>(row * p.ld) * isz; };
+    auto geo = [&](size_t off) {
+        if constexpr (GRID) return Geo{0, gmax, 0};
+        Geo g;
+        g.h0 = min(static_cast<int>((0u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.a) + off)) & 15u) / isz, N);
+        g.G = (N - g.h0) / V;
+        g.t0 = (N - g.h0) % V;
+        return g;
+    };
+    auto issue = [&](long long row, int slot) {  // thread 0: both arrays' groups into a stage
+        const size_t off = offset(row);
+        const Geo g = geo(off);
+        if (!GRID && g.G == 0) return;
+        const uint32_t bytes = static_cast<uint32_t>(g.G) * 16u;
+        unsigned char *da = stages + static_cast<uint32_t>(slot) * 2u * arr;
+        const size_t src = off + g.h0 * isz;
+        mbar_arrive_expect_tx(&full[slot], 2 * bytes);
+        for (uint32_t o = 0; o < bytes; o += kMaxChunkBytes) {
+            const uint32_t n = min(bytes - o, static_cast<uint32_t>(kMaxChunkBytes));
+            bulk_g2s(da + o, p.a + src + o, n, &full[slot]);
+            bulk_g2s(da + arr + o, p.dy + src + o, n, &full[slot]);
+        }
+    };
+    auto edge_index = [&](const Geo &g) -> int {
+        if constexpr (GRID) return -1;
+        return t < g.h0 ? t : (T - 1 - t < g.t0 ? g.h0 + g.G * V + (T - 1 - t) : -1);
+    };
+
+    if (t == 0) {
+        for (int k = 0; k < S; ++k) mbar_init(&full[k], 1);
+        fence_mbar_init();
+        for (int k = 0; k < S; ++k)
+            if (row_first + k * stride < p.rows) issue(row_first + k * stride, k);
+    }
+    if constexpr (AFF) planes_fill<NP>(gsm, np, p.gamma, 1.0f, N, team * T + t, T * teams);
+    __syncthreads();
+
+    BwdRow<OP> Rn;  // the next row's saved statistics and edge elements
+    float ean = 0.0f, edn = 0.0f;
+    auto fetch_next = [&](long long row) {
+        Rn.load(p, row);
+        if constexpr (!GRID) {
+            const size_t off = offset(row);
+            const int i = edge_index(geo(off));
+            if (i >= 0) {
+                ean = decode_one<DT>(p.a + off + i * isz, 1.0f);
+                edn = decode_one<DT>(p.dy + off + i * isz, 1.0f);
+            }
+        }
+    };
+    if (row_first < p.rows) fetch_next(row_first);
+
+    int slot = 0;
+    uint32_t lap = 0;
+    bool odd = false;  // row parity: the one reduction of the plain sums alternates between two arrays
+    for (long long row = row_first; row < p.rows; row += stride, odd = !odd) {
+        const size_t off = offset(row);
+        const Geo g = geo(off);
+        const int ie = edge_index(g);
+        const bool edge = !GRID && ie >= 0;
+        const BwdRow<OP> R = Rn;
+        const float ea = ean, ed = edn;
+        if (row + stride < p.rows) fetch_next(row + stride);
+        const unsigned char *da = stages + static_cast<uint32_t>(slot) * 2u * arr, *dd = da + arr;
+        if (GRID || g.G > 0) mbar_wait_bounded(&full[slot], lap & 1u, p.err);
+
+        auto each = [&](auto &&fn) {  // this thread's groups
+#pragma unroll 1
+            for (int gi = t; gi < g.G; gi += T) {
+                float fa[V], fd[V];
+                decode_group<DT>(*reinterpret_cast<const uint4 *>(da + 16 * gi), fa, 1.0f);
+                decode_group<DT>(*reinterpret_cast<const uint4 *>(dd + 16 * gi), fd, 1.0f);
+                fn(gi, fa, fd);
+            }
+        };
+        // dy gamma of a group
+        auto times_gamma = [&](int gi, float (&fd)[V]) {
+            if constexpr (kNorm<OP>) {
+                float fg[V];
+                if constexpr (AFF && GRID) planes_group<NP>(gp, gi, 0, fg);
+                else if constexpr (AFF) planes_load<NP>(gp, g.h0 + gi * V, fg);
+                else ldg_shift<V>(p.gamma, g.h0 + gi * V, N, 1.0f, fg);
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const float2 x = __fmul2_rn(make_float2(fd[v], fd[v + 1]), make_float2(fg[v], fg[v + 1]));
+                    fd[v] = x.x;
+                    fd[v + 1] = x.y;
+                }
+            }
+        };
+        const float eg = kNorm<OP> && edge && p.gamma ? p.gamma[ie] : 1.0f;
+        // after the row's first reduction: every thread is done with the previous row
+        auto refill = [&]() {
+            if (T == 32) __syncwarp();
+            const long long nr = row + (S - 1) * stride;
+            if (t == 0 && S > 1 && row != row_first && nr < p.rows) {
+                fence_proxy_async_smem();
+                issue(nr, (slot ? slot : S) - 1);
+            }
+        };
+
+        Coef kc;
+        if constexpr (!kLogits<OP> && !kPair<OP>) {
+            float2 s0 = f2(0.0f), s1 = f2(0.0f);
+            each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+                times_gamma(gi, fd);
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const float2 d = make_float2(fd[v], fd[v + 1]);
+                    float2 x = make_float2(fa[v], fa[v + 1]);
+                    if constexpr (OP == BOP_LN) {
+                        x = __fadd2_rn(x, f2(-R.mean));
+                        s0 = __fadd2_rn(s0, d);
+                    }
+                    s1 = __ffma2_rn(x, d, s1);
+                }
+            });
+            float v[2] = {s1.x + s1.y, s0.x + s0.y};
+            if (edge) {
+                const float d = ed * eg;
+                v[0] = fmaf(OP == BOP_LN ? ea - R.mean : ea, d, v[0]);
+                v[1] += d;
+            }
+            if constexpr (OP == BOP_LN) {
+                team_sums(v, red + (odd ? 96 : 0), team, T);
+            } else {
+                float v1[1] = {v[0]};
+                team_sums(v1, red + (odd ? 96 : 0), team, T);
+                v[0] = v1[0];
+            }
+            kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0] * R.rstd, N);
+        } else if constexpr (kLogits<OP>) {
+            GroupMax<DT, false> gm;
+#pragma unroll 1
+            for (int gi = t; gi < g.G; gi += T) gm.add(*reinterpret_cast<const uint4 *>(da + 16 * gi));
+            float m = gm.value();
+            if (edge) m = fmaxf(m, ea);
+            m = team_reduce<true>(m, red, team, T);
+            refill();
+            const float mz = m == -INFINITY ? 0.0f : m;
+            float2 sS = f2(0.0f), sT = f2(0.0f);
+            each([&](int, float (&fa)[V], float (&fd)[V]) {
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const float2 x = __fmul2_rn(__fadd2_rn(make_float2(fa[v], fa[v + 1]), f2(-mz)), f2(kLog2e));
+                    const float2 e = make_float2(ex2_ftz(x.x), ex2_ftz(x.y)), d = make_float2(fd[v], fd[v + 1]);
+                    sS = __fadd2_rn(sS, e);
+                    sT = OP == BOP_SMLOGITS ? __ffma2_rn(e, d, sT) : __fadd2_rn(sT, d);
+                }
+            });
+            float v[2] = {sS.x + sS.y, sT.x + sT.y};
+            if (edge) {
+                const float e = ex2_ftz((ea - mz) * kLog2e);
+                v[0] += e;
+                v[1] = OP == BOP_SMLOGITS ? fmaf(e, ed, v[1]) : v[1] + ed;
+            }
+            team_sums(v, red + 96, team, T);
+            kc = logit_coeffs<OP>(m, v[0], v[1]);
+        } else {
+            // means about the row's first group's first elements, then the centred sums
+            const float ka = GRID || g.G > 0 ? decode_one<DT>(da, 1.0f) : decode_one<DT>(p.a + off, 1.0f);
+            const float kd = GRID || g.G > 0 ? decode_one<DT>(dd, 1.0f) : decode_one<DT>(p.dy + off, 1.0f);
+            float2 u0 = f2(0.0f), u1 = f2(0.0f);
+            each([&](int, float (&fa)[V], float (&fd)[V]) {
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const float2 x = __fadd2_rn(make_float2(fa[v], fa[v + 1]), f2(-ka));
+                    const float2 d = make_float2(fd[v], fd[v + 1]);
+                    if constexpr (OP == BOP_WVAR) {
+                        u0 = __fadd2_rn(u0, d);
+                        u1 = __ffma2_rn(d, x, u1);
+                    } else {
+                        u0 = __fadd2_rn(u0, x);
+                        u1 = __fadd2_rn(u1, __fadd2_rn(d, f2(-kd)));
+                    }
+                }
+            });
+            float v[2] = {u0.x + u0.y, u1.x + u1.y};
+            if (edge) {
+                v[0] += OP == BOP_WVAR ? ed : ea - ka;
+                v[1] += OP == BOP_WVAR ? ed * (ea - ka) : ed - kd;
+            }
+            team_sums(v, red, team, T);
+            refill();
+            const float n = static_cast<float>(N);
+            const float xb = ka + (OP == BOP_WVAR ? v[1] / v[0] : v[0] / n);
+            const float yb = OP == BOP_WVAR ? 0.0f : kd + v[1] / n;
+            float2 q0 = f2(0.0f), q1 = f2(0.0f), q2 = f2(0.0f);
+            each([&](int, float (&fa)[V], float (&fd)[V]) {
+#pragma unroll
+                for (int k = 0; k < V; k += 2) {
+                    const float2 x = __fadd2_rn(make_float2(fa[k], fa[k + 1]), f2(-xb));
+                    const float2 d = make_float2(fd[k], fd[k + 1]);
+                    if constexpr (OP == BOP_WVAR) {
+                        q0 = __ffma2_rn(__fmul2_rn(d, x), x, q0);
+                    } else {
+                        const float2 y = __fadd2_rn(d, f2(-yb));
+                        q0 = __ffma2_rn(x, x, q0);
+                        q1 = __ffma2_rn(y, y, q1);
+                        q2 = __ffma2_rn(x, y, q2);
+                    }
+                }
+            });
+            float q[3] = {q0.x + q0.y, q1.x + q1.y, q2.x + q2.y};
+            if (edge) {
+                const float x = ea - xb, y = ed - yb;
+                q[0] = fmaf(OP == BOP_WVAR ? ed * x : x, x, q[0]);
+                q[1] = fmaf(y, y, q[1]);
+                q[2] = fmaf(x, y, q[2]);
+            }
+            if constexpr (OP == BOP_WVAR) {
+                float q1s[1] = {q[0]};
+                team_sums(q1s, red + 96, team, T);
+                const float c[3] = {v[0], xb, q1s[0]};
+                kc = pair_coeffs<OP>(c, R);
+            } else {
+                team_sums(q, red + 96, team, T);
+                const float c[6] = {n, xb, yb, q[0], q[1], q[2]};
+                kc = pair_coeffs<OP>(c, R);
+            }
+        }
+        if constexpr (!kLogits<OP> && !kPair<OP>) refill();
+
+        // ---- gradients
+        const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
+        unsigned char *xr = p.dx + off + g.h0 * isz;
+        unsigned char *xr2 = kPair<OP> ? p.dx2 + off + g.h0 * isz : nullptr;
+        const bool vec = GRID || ((reinterpret_cast<uintptr_t>(xr) | reinterpret_cast<uintptr_t>(xr2)) & 15u) == 0;
+        each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+            float y[V];
+            if constexpr (kPair<OP>) {
+                float y2[V];
+#pragma unroll
+                for (int v = 0; v < V; ++v) R.dx_pair(fa[v], fd[v], kc, y[v], y2[v]);
+                store_group<DT, V>(xr2 + 16 * gi, y2, vec);
+            } else {
+                times_gamma(gi, fd);
+#pragma unroll
+                for (int v = 0; v < V; v += 2) {
+                    const float2 x = make_float2(fa[v], fa[v + 1]), d = make_float2(fd[v], fd[v + 1]);
+                    float2 r;
+                    if constexpr (OP == BOP_SOFTMAX) {
+                        r = __fmul2_rn(x, __fadd2_rn(d, f2(-kc.c0)));
+                    } else if constexpr (kLogits<OP>) {
+                        const float2 z = __fmul2_rn(__fadd2_rn(x, f2(-kc.c0)), f2(kLog2e));
+                        const float2 e = make_float2(ex2_ftz(z.x), ex2_ftz(z.y));
+                        if constexpr (OP == BOP_SMLOGITS) {
+                            r = __fmul2_rn(__fmul2_rn(e, f2(kc.c1)), __fadd2_rn(d, f2(-kc.c2)));
+                        } else {
+                            r = __fmul2_rn(f2(R.w), __ffma2_rn(e, f2(kc.c1), make_float2(-d.x, -d.y)));
+                        }
+                    } else {
+                        const float2 xm = OP == BOP_LN ? __fadd2_rn(x, f2(-R.mean)) : x;
+                        r = __ffma2_rn(d, f2(R.rstd), __ffma2_rn(xm, f2(k1), f2(k0)));
+                    }
+                    y[v] = r.x;
+                    y[v + 1] = r.y;
+                }
+            }
+            store_group<DT, V>(xr + 16 * gi, y, vec);
+        });
+        if (edge) {
+            if constexpr (kPair<OP>) {
+                float o1, o2;
+                R.dx_pair(ea, ed, kc, o1, o2);
+                store_one<DT>(p.dx + off + ie * isz, o1);
+                store_one<DT>(p.dx2 + off + ie * isz, o2);
+            } else {
+                store_one<DT>(p.dx + off + ie * isz, R.dx(ea, ed, eg, kc));
+            }
+        }
+        if (S == 1 && row + stride < p.rows) {
+            if (T == 32) __syncwarp();
+            else named_bar_sync(team, T);
+            if (t == 0) {
+                fence_proxy_async_smem();
+                issue(row + stride, 0);
+            }
+        }
+        if (++slot == S) {
+            slot = 0;
+            ++lap;
+        }
+    }
+}
+
+
+#ifdef CREDIT_BWD_DT
+template <int OP>
 BwdKernels bwd_kernels_of() {
-    return {reinterpret_cast<const void *>(&k_bwd_staged<OP, DT>), reinterpret_cast<const void *>(&k_bwd_tp_fused<OP, DT>),
-            reinterpret_cast<const void *>(&k_bwd_tp_stats<OP, DT>),
-            reinterpret_cast<const void *>(&k_bwd_tp_apply<OP, DT>)};
+    constexpr int DT = CREDIT_BWD_DT;
+    constexpr bool A = kNorm<OP>;  // the other ops have no gamma
+    return {reinterpret_cast<const void *>(&k_bwd_staged<OP, DT>),
+            {reinterpret_cast<const void *>(&k_bwd_tp_fused<OP, DT, false>),
+             reinterpret_cast<const void *>(&k_bwd_tp_fused<OP, DT, true>)},
+            {reinterpret_cast<const void *>(&k_bwd_tp_stats<OP, DT, false>),
+             reinterpret_cast<const void *>(&k_bwd_tp_stats<OP, DT, true>)},
+            {reinterpret_cast<const void *>(&k_bwd_tp_apply<OP, DT, false>),
+             reinterpret_cast<const void *>(&k_bwd_tp_apply<OP, DT, true>)},
+            {{reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, false>),
+              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, A>)},
+             {reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, false>),
+              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, A>)}}};
 }
+#endif
+}  // namespace
 
-bool bwd_kernels(int op, int dt, BwdKernels *k) {
-    switch (op * 4 + dt) {
-    case BOP_SOFTMAX * 4 + DT_F32: *k = bwd_kernels_of<BOP_SOFTMAX, DT_F32>(); return true;
-    case BOP_SOFTMAX * 4 + DT_BF16: *k = bwd_kernels_of<BOP_SOFTMAX, DT_BF16>(); return true;
-    case BOP_LN * 4 + DT_F32: *k = bwd_kernels_of<BOP_LN, DT_F32>(); return true;
-    case BOP_LN * 4 + DT_BF16: *k = bwd_kernels_of<BOP_LN, DT_BF16>(); return true;
-    case BOP_RMS * 4 + DT_F32: *k = bwd_kernels_of<BOP_RMS, DT_F32>(); return true;
-    case BOP_RMS * 4 + DT_BF16: *k = bwd_kernels_of<BOP_RMS, DT_BF16>(); return true;
-    case BOP_SMLOGITS * 4 + DT_F32: *k = bwd_kernels_of<BOP_SMLOGITS, DT_F32>(); return true;
-    case BOP_SMLOGITS * 4 + DT_BF16: *k = bwd_kernels_of<BOP_SMLOGITS, DT_BF16>(); return true;
-    case BOP_XENT * 4 + DT_F32: *k = bwd_kernels_of<BOP_XENT, DT_F32>(); return true;
-    case BOP_XENT * 4 + DT_BF16: *k = bwd_kernels_of<BOP_XENT, DT_BF16>(); return true;
-    case BOP_WVAR * 4 + DT_F32: *k = bwd_kernels_of<BOP_WVAR, DT_F32>(); return true;
-    case BOP_WVAR * 4 + DT_BF16: *k = bwd_kernels_of<BOP_WVAR, DT_BF16>(); return true;
-    case BOP_PEARSON * 4 + DT_F32: *k = bwd_kernels_of<BOP_PEARSON, DT_F32>(); return true;
-    case BOP_PEARSON * 4 + DT_BF16: *k = bwd_kernels_of<BOP_PEARSON, DT_BF16>(); return true;
+// The file is compiled three times: with CREDIT_BWD_DT = 0 (FP32) and 1 (BF16)
+// for the kernels of one type, and without it for the host side.
+bool bwd_kernels_dt0(int op, BwdKernels *k);
+bool bwd_kernels_dt1(int op, BwdKernels *k);
+
+#ifdef CREDIT_BWD_DT
+#define CREDIT_CAT2(a, b) a##b
+#define CREDIT_CAT(a, b) CREDIT_CAT2(a, b)
+bool CREDIT_CAT(bwd_kernels_dt, CREDIT_BWD_DT)(int op, BwdKernels *k) {
+    switch (op) {
+    case BOP_SOFTMAX: *k = bwd_kernels_of<BOP_SOFTMAX>(); return true;
+    case BOP_LN: *k = bwd_kernels_of<BOP_LN>(); return true;
+    case BOP_RMS: *k = bwd_kernels_of<BOP_RMS>(); return true;
+    case BOP_SMLOGITS: *k = bwd_kernels_of<BOP_SMLOGITS>(); return true;
+    case BOP_XENT: *k = bwd_kernels_of<BOP_XENT>(); return true;
+    case BOP_WVAR: *k = bwd_kernels_of<BOP_WVAR>(); return true;
+    case BOP_PEARSON: *k = bwd_kernels_of<BOP_PEARSON>(); return true;
     default: return false;
     }
+}
+
+}  // namespace credit
+#else
+namespace {
+
+bool bwd_kernels(int op, int dt, BwdKernels *k) {
+    return dt == DT_F32 ? bwd_kernels_dt0(op, k) : dt == DT_BF16 ? bwd_kernels_dt1(op, k) : false;
 }
 
 // ------------------------------------------------------------------ host
@@ -1040,6 +1457,51 @@ bool bwd_config(const DeviceInfo &di, long long N, int isz, int P, int req_nbuf,
     return false;
 }
 
+// Geometry of k_bwd_team; false where it does not apply: the arrays' rows at
+// different phases of the 16-byte grid, or no room for a row of both arrays.
+struct BwdTeamCfg {
+    int threads, teams, stages, grid;
+    bool grid_rows, gamma_smem;
+    long long smem;
+};
+bool bwd_team_config(const DeviceInfo &di, const credit_bwd_args *a, BwdTeamCfg *out) {
+    const int isz = dtype_size(a->dtype), V = 16 / isz;
+    const uintptr_t ua = reinterpret_cast<uintptr_t>(a->a), ud = reinterpret_cast<uintptr_t>(a->dy);
+    if (((ua ^ ud) & 15u) != 0 || ua % isz != 0) return false;
+    const long long groups = a->cols / V, per_sm = (a->rows + di.sm_count - 1) / di.sm_count;
+    if (a->cols * isz > kBwdTeamMaxBytes) return false;
+    const bool norm = a->op == BOP_LN || a->op == BOP_RMS;
+    auto warps = [](long long n) { return n < 1 ? 32 : (n + 31) / 32 * 32; };
+    BwdTeamCfg r;
+    // teams of four 16-byte groups of each array per thread, as many as have a row and fit shared memory with
+    // one stage; where that leaves threads over, each team takes more of them
+    const long long T4 = warps((groups + kTeamGroups - 1) / kTeamGroups);
+    long long teams = kTeamMaxThreads / (T4 < kTeamMaxThreads ? T4 : kTeamMaxThreads);
+    const long long fit = groups > 0 ? (di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16)) / (groups * 32) : teams;
+    if (teams > fit) teams = fit;
+    if (teams > per_sm) teams = per_sm;
+    if (teams < 1) return false;
+    long long T = T4;
+    if (teams * T4 <= kTeamMaxThreads / 2 || T4 > kTeamMaxThreads) {
+        const long long most = kTeamMaxThreads / teams / 32 * 32, want = warps(groups);
+        T = want < most ? want : most;
+    }
+    r.teams = static_cast<int>(teams);
+    r.threads = static_cast<int>(T);
+    const long long np4 = (a->cols + 3) / 4, NP = V / 4, aff = norm ? NP * ((np4 + NP - 1) / NP + 1) * 16 : 0;
+    const long long stage = groups * 32 * r.teams, room = di.smem_optin - bwd_team_ctrl(r.threads, r.teams);
+    r.gamma_smem = norm && aff + stage <= room && per_sm > r.teams;
+    const long long left = room - (r.gamma_smem ? aff : 0);
+    r.stages = stage == 0 || 2 * stage <= left ? 2 : stage <= left ? 1 : 0;
+    if (r.stages == 0) return false;
+    r.smem = bwd_team_ctrl(r.threads, r.teams) + (r.gamma_smem ? aff : 0) + r.stages * stage;
+    const long long ctas = (a->rows + r.teams - 1) / r.teams;
+    r.grid = static_cast<int>(ctas < di.sm_count ? ctas : di.sm_count);
+    r.grid_rows = a->cols % V == 0 && rows_aligned(a);
+    *out = r;
+    return true;
+}
+
 // gamma is staged in shared memory by the norms when present and 16-byte aligned.
 bool stage_gamma(int op, const float *gamma) {
     return (op == BOP_LN || op == BOP_RMS) && gamma != nullptr && (reinterpret_cast<uintptr_t>(gamma) & 15u) == 0;
@@ -1077,7 +1539,7 @@ credit_status plan_bwd_for(int dev, int op, long long cols, int dtype, credit_pl
     out->threads = kBwdThreads;
     const int isz = dtype_size(dtype);
     const DeviceInfo *di = dev >= 0 ? device_info(dev) : nullptr;
-    if (di != nullptr && cols * isz > kBwdFusedMaxBytes) {
+    if (di != nullptr && cols * isz > bwd_team_bytes(op)) {
         BwdKernels k;
         if (!bwd_kernels(op, dtype, &k)) return CREDIT_ERR_UNSUPPORTED;
         const bool merge_heavy = op == BOP_SMLOGITS || op == BOP_XENT || kPairOp(op);
@@ -1085,10 +1547,12 @@ credit_status plan_bwd_for(int dev, int op, long long cols, int dtype, credit_pl
             // the logits ops carry a per-row merge of (max, sum, dot) states, the pair ops Chan merges of
             // centred moments, whose cost and exchange latency grow with P: staged only while a CTA's slice is
             // at most 64 KiB per array and P <= 4 (measured: P = 4 beats two-pass at 64K FP32 columns, P = 8
-            // and 16 lose at 128K), either buffering
+            // and 16 lose at 128K), either buffering; the pair ops, with four arrays to move, at P = 4 up to
+            // the largest slice that fits (1000 x 200000 BF16 Pearson 312 us against 373, 3200 x 74752 FP32
+            // weighted variance 745 against 856)
             for (int P = 1; P <= 4; P *= 2) {
                 BwdCfg cfg;
-                if (cols * isz > 65536LL * P) continue;
+                if (cols * isz > 65536LL * P && !(kPairOp(op) && P == 4)) continue;
                 if (!bwd_config(*di, cols, isz, P, 0, false, &cfg)) continue;
                 if (prepare_staged_kernel(dev, k.staged) != CREDIT_OK) continue;
                 if (staged_max_clusters(dev, k.staged, P, cfg.threads, cfg.smem, false) <= 0) continue;
@@ -1219,6 +1683,19 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
         return CREDIT_OK;
     }
     const int G = chosen.ctas_per_row;
+    BwdTeamCfg tc;
+    if (G == 1 && bwd_team_config(*device_info(dev), args, &tc)) {
+        const void *fn = k.team[tc.grid_rows][tc.gamma_smem];
+        if ((st = prepare_staged_kernel(dev, fn)) != CREDIT_OK) return st;
+        BwdArgs r = base;
+        r.nbuf = tc.stages;
+        void *kargs[] = {&r};
+        e = launch_kernel(fn, dim3(tc.grid), dim3(tc.threads, tc.teams), static_cast<size_t>(tc.smem), 1, stream, kargs);
+        if (e != cudaSuccess) return cuda_st(e);
+        g_launch_count.fetch_add(1);
+        return CREDIT_OK;
+    }
+    const int off = !rows_aligned(args);
     const size_t rec = (args->op == BOP_SMLOGITS || args->op == BOP_XENT) ? 4
                        : (args->op == BOP_WVAR || args->op == BOP_PEARSON) ? 8 : 2;  // floats per partial
     const long long cap = G == 1 ? 0x7FFFFFFFLL : static_cast<long long>(ws_floats / (static_cast<size_t>(G) * rec));
@@ -1231,16 +1708,16 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
         r.G = G;
         void *kargs[] = {&r};
         if (G == 1) {
-            e = launch_kernel(k.fused, dim3(static_cast<unsigned>(n)), dim3(kBwdThreads), 0, 1, stream, kargs);
+            e = launch_kernel(k.fused[off], dim3(static_cast<unsigned>(n)), dim3(kBwdThreads), 0, 1, stream, kargs);
             if (e != cudaSuccess) return cuda_st(e);
             g_launch_count.fetch_add(1);
             continue;
         }
         const dim3 grid(static_cast<unsigned>(G * n));
-        e = launch_kernel(k.stats, grid, dim3(kBwdThreads), 0, 1, stream, kargs);
+        e = launch_kernel(k.stats[off], grid, dim3(kBwdThreads), 0, 1, stream, kargs);
         if (e != cudaSuccess) return cuda_st(e);
         g_launch_count.fetch_add(1);
-        e = launch_kernel(k.apply, grid, dim3(kBwdThreads), 0, 1, stream, kargs);
+        e = launch_kernel(k.apply[off], grid, dim3(kBwdThreads), 0, 1, stream, kargs);
         if (e != cudaSuccess) return cuda_st(e);
         g_launch_count.fetch_add(1);
     }
@@ -1248,3 +1725,5 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
 }
 
 }  // extern "C"
+
+#endif  // CREDIT_BWD_DT

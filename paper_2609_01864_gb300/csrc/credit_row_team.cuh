@@ -105,7 +105,7 @@ __device__ __forceinline__ void planes_load(const AffinePlanes &a, int i0, float
 // is all dflt), the same way: no vector that reaches outside it is read (such a group loads its
 // elements one by one).
 template <int V>
-__device__ __forceinline__ void ldg_shift(const float *p, int i0, int N, float dflt, float (&v)[V]) {
+__device__ __forceinline__ void ldg_shift(const float *p, long long i0, long long N, float dflt, float (&v)[V]) {
     if (p == nullptr) {
 #pragma unroll
         for (int k = 0; k < V; ++k) v[k] = dflt;
