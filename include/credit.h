@@ -94,11 +94,12 @@ typedef enum {
  *         be staged in shared memory beside the ring (rows off the 16-byte
  *         grid) runs on the SMEM tier instead, also under an explicit TMEM
  *         plan.
- *   ROW   whole rows in shared memory, several teams of threads per SM, each
- *         on its own row (ONE_CTA plans; any op, type and alignment).  Where a
- *         row does not fit, or the plan sets threads, chunk_bytes or
- *         cluster_size > 1, ROW means AUTO; ring_chunks is the number of rows
- *         in flight per team (0 = default).
+ *   ROW   whole rows (CLUSTER: whole slices, cluster_size a power of two) in
+ *         shared memory, several teams of threads per SM, each on its own
+ *         row; any op, type and alignment.  Where they do not fit, or the
+ *         plan sets threads, chunk_bytes or fill_share, ROW means AUTO;
+ *         ring_chunks is the number of rows in flight per team (0 =
+ *         default).
  *   AUTO  TMEM where it applies and a slice exceeds 32 KiB, else SMEM
  *         (CREDIT_RETAIN=smem in the environment makes AUTO mean SMEM,
  *         CREDIT_RETAIN=tmem TMEM wherever it applies).  The planners set

@@ -22,9 +22,9 @@ namespace credit {
 bool kernels_tin0(int op, int tout, KernelSet *ks);
 bool kernels_tin1(int op, int tout, KernelSet *ks);
 bool kernels_tin2(int op, int tout, KernelSet *ks);
-const void *team_kernel_tin0(int op, int tout, bool grid, bool aff);
-const void *team_kernel_tin1(int op, int tout, bool grid, bool aff);
-const void *team_kernel_tin2(int op, int tout, bool grid, bool aff);
+const void *team_kernel_tin0(int op, int tout, bool grid, bool aff, bool cluster);
+const void *team_kernel_tin1(int op, int tout, bool grid, bool aff, bool cluster);
+const void *team_kernel_tin2(int op, int tout, bool grid, bool aff, bool cluster);
 }  // namespace credit
 
 using namespace credit;
@@ -58,12 +58,12 @@ bool kernel_set(int op, int tin, int tout, KernelSet *ks) {
     }
 }
 
-const void *team_kernel(int op, int tin, int tout, bool grid, bool aff) {
+const void *team_kernel(int op, int tin, int tout, bool grid, bool aff, bool cluster) {
     if (op == OP_LSE) tout = DT_F32;
     switch (tin) {
-    case DT_F32: return team_kernel_tin0(op, tout, grid, aff);
-    case DT_BF16: return team_kernel_tin1(op, tout, grid, aff);
-    case DT_E4M3: return team_kernel_tin2(op, tout, grid, aff);
+    case DT_F32: return team_kernel_tin0(op, tout, grid, aff, cluster);
+    case DT_BF16: return team_kernel_tin1(op, tout, grid, aff, cluster);
+    case DT_E4M3: return team_kernel_tin2(op, tout, grid, aff, cluster);
     default: return nullptr;
     }
 }
@@ -263,55 +263,70 @@ bool ring_config_tm(const DeviceInfo &di, long long N, int isz, int P, int req_r
     return true;
 }
 
-// Geometry of k_row_team.  Threads per row: four 16-byte groups each up to
-// 16 KiB rows and eight above, so that rows of 24-64 KiB still leave an SM
-// several teams (4096 x 24K FP32 LayerNorm off the grid: 146 us with eight,
-// 206 with four); an SM with fewer rows than that gives each more threads.
-bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int nab, int req_stages, TeamCfg *out) {
-    const long long groups = N * isz / 16;  // at any phase of the row
-    if (N <= 0 || groups * 16 > di.smem_optin) return false;
+// Geometry of k_row_team for rows split over P CTAs.  Threads per slice: four
+// 16-byte groups each up to 16 KiB slices and eight above, so that slices of
+// 24-64 KiB still leave an SM several teams (16384 x 6K FP32 LayerNorm off the
+// grid: 146 us with eight, 206 with four); an SM with fewer rows than that, or
+// without room for a stage per team, gives each team more threads.
+bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int nab, int P, int req_stages,
+                 TeamCfg *out) {
+    if (N <= 0 || P < 1 || P > kMaxCluster || (P & (P - 1)) != 0) return false;
+    const long long V = 16 / isz, groups = (N / V + P - 1) / P;  // of a slice, at any phase of the row
+    if (groups * 16 > di.smem_optin || (P > 1 && N / V < 32 * P)) return false;
     TeamCfg r;
+    r.P = P;
     const int per_thread = groups > 256 * kTeamGroups ? 2 * kTeamGroups : kTeamGroups;
     auto warps = [](long long n) { return n < 1 ? 32 : (n + 31) / 32 * 32; };
     long long T = warps((groups + per_thread - 1) / per_thread);
     if (T > kTeamMaxThreads) T = kTeamMaxThreads;
-    const long long per_sm = (rows + di.sm_count - 1) / di.sm_count;
-    r.teams = static_cast<int>(kTeamMaxThreads / T);
-    if (r.teams > per_sm) {
-        r.teams = static_cast<int>(per_sm < 1 ? 1 : per_sm);
-        const long long most = kTeamMaxThreads / r.teams / 32 * 32, want = warps(groups);
+    const long long walkers = di.sm_count / P, per_sm = (rows + walkers - 1) / walkers;
+    long long teams = kTeamMaxThreads / T;
+    // gamma / beta planes (AffinePlanes) of the columns a slice can cover
+    const long long cols = P == 1 ? N : (groups + 3) * V < N ? (groups + 3) * V : N, NP = V / 4;
+    const long long aff = nab * NP * (((cols + 3) / 4 + NP - 1) / NP + 1) * 16;
+    const long long ctrl = team_ctrl_bytes(static_cast<int>(teams), P > 1);
+    if (P > 1 && groups > 0) {  // gamma / beta always resident; as many teams as that leaves room for
+        const long long fit = (di.smem_optin - ctrl - aff) / (groups * 16);
+        if (fit < 1) return false;
+        if (teams > fit) teams = fit;
+    }
+    if (teams > per_sm) teams = per_sm;
+    if (teams < 1) teams = 1;
+    if (teams * T <= kTeamMaxThreads / 2 || teams == per_sm) {
+        const long long most = kTeamMaxThreads / teams / 32 * 32, want = warps(groups);
         T = want < most ? want : most;
     }
+    r.teams = static_cast<int>(teams);
     r.threads = static_cast<int>(T);
-    const long long stage = groups * 16 * r.teams;
-    const long long np4 = (N + 3) / 4, NP = 4 / isz;  // gamma / beta planes (AffinePlanes)
-    const long long aff = nab * NP * ((np4 + NP - 1) / NP + 1) * 16;
-    long long room = di.smem_optin - team_ctrl_bytes(r.teams);
+    const long long stage = groups * 16 * teams;
+    long long room = di.smem_optin - team_ctrl_bytes(r.teams, P > 1);
     // gamma / beta in shared memory unless a team has one row only, which would wait for the copy
-    r.affine_resident = nab > 0 && aff + stage <= room && per_sm > r.teams;
+    r.affine_resident = nab > 0 && aff + stage <= room && (P > 1 || per_sm > teams);
     if (r.affine_resident) room -= aff;
     long long S = req_stages > 0 ? req_stages : 2;  // a third stage measures the same
     if (stage > 0 && S > room / stage) S = room / stage;
     if (S < 1 || S > kTeamMaxStages) return false;
     r.stages = static_cast<int>(S);
-    r.smem = team_ctrl_bytes(r.teams) + (r.affine_resident ? aff : 0) + S * stage;
-    const long long ctas = (rows + r.teams - 1) / r.teams;
-    r.grid = static_cast<int>(ctas < di.sm_count ? ctas : di.sm_count);
+    r.smem = team_ctrl_bytes(r.teams, P > 1) + (r.affine_resident ? aff : 0) + S * stage;
+    const long long ctas = (rows + teams - 1) / teams;
+    r.grid = static_cast<int>(ctas < walkers ? ctas : walkers);
     r.grid_rows = false;
     *out = r;
     return true;
 }
 
 bool team_plan_config(const DeviceInfo &di, const credit_args *a, const credit_plan_t *p, TeamCfg *out) {
-    if (p->path != CREDIT_PATH_ONE_CTA || p->retain != CREDIT_RETAIN_ROW || p->threads || p->reducer_threads ||
-        p->chunk_bytes || p->ring_chunks < 0 || p->ring_chunks > kTeamMaxStages)
+    if ((p->path != CREDIT_PATH_ONE_CTA && p->path != CREDIT_PATH_CLUSTER) || p->retain != CREDIT_RETAIN_ROW ||
+        p->threads || p->reducer_threads || p->chunk_bytes || p->fill_share > 0.0f || p->ring_chunks < 0 ||
+        p->ring_chunks > kTeamMaxStages)
         return false;
     const int isz = dtype_size(a->in_dtype), osz = dtype_size(a->op == OP_LSE ? DT_F32 : a->out_dtype), V = 16 / isz;
     const int nab = a->op == OP_LN ? 2 : a->op == OP_RMS ? 1 : 0;
-    if (!team_config(di, a->rows, a->cols, isz, nab, p->ring_chunks, out)) return false;
+    const int P = p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size;
+    if (!team_config(di, a->rows, a->cols, isz, nab, P, p->ring_chunks, out)) return false;
     const long long ld_in = a->ld_in ? a->ld_in : a->cols, ld_out = a->ld_out ? a->ld_out : a->cols;
     const int vb = V * osz < 16 ? V * osz : 16;
-    out->grid_rows = a->cols % V == 0 && reinterpret_cast<uintptr_t>(a->in) % 16 == 0 && ld_in * isz % 16 == 0 &&
+    out->grid_rows = P == 1 && a->cols % V == 0 && reinterpret_cast<uintptr_t>(a->in) % 16 == 0 && ld_in * isz % 16 == 0 &&
                      (a->op == OP_LSE || (reinterpret_cast<uintptr_t>(a->out) % vb == 0 && ld_out * osz % vb == 0));
     return true;
 }
@@ -600,7 +615,7 @@ credit_status check_plan(int device, const credit_args *a, const credit_plan_t *
         if (p->path == CREDIT_PATH_CLUSTER && P < 2) return CREDIT_ERR_UNSUPPORTED;
         TeamCfg gc;
         if (team_plan_config(*di, a, p, &gc))
-            return staged_max_clusters(device, team_kernel(a->op, a->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0), 1, gc.threads * gc.teams, gc.smem,
+            return staged_max_clusters(device, team_kernel(a->op, a->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
                                        false) > 0
                        ? CREDIT_OK
                        : CREDIT_ERR_UNSUPPORTED;
@@ -729,16 +744,22 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
         TeamCfg gc;
         if (team_plan_config(d.info, a, p, &gc)) {
             if (g_test_extra_tx.load() > 0) return CREDIT_ERR_UNSUPPORTED;  // the wait test's ring kernel only
-            const void *fn = team_kernel(a->op, tin, tout, gc.grid_rows, gc.affine_resident != 0);
+            const void *fn = team_kernel(a->op, tin, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1);
             if (fn == nullptr) return CREDIT_ERR_UNSUPPORTED;
             const credit_status st = prepare_kernel(d, fn, true);
             if (st != CREDIT_OK) return st;
+            int grid = gc.grid;
+            if (P > 1) {  // every cluster resident
+                const int maxc = staged_max_clusters(device, fn, P, gc.threads * gc.teams, gc.smem, false);
+                if (maxc <= 0) return CREDIT_ERR_UNSUPPORTED;
+                if (grid > maxc) grid = maxc;
+            }
             RowArgs r = base;
             r.ring = gc.stages;
             r.affine_resident = gc.affine_resident;
             void *args[] = {&r};
-            const cudaError_t e = launch(fn, dim3(gc.grid), dim3(gc.threads, gc.teams),
-                                         static_cast<size_t>(gc.smem), 1, s, args);
+            const cudaError_t e = launch(fn, dim3(static_cast<unsigned>(grid * P)), dim3(gc.threads, gc.teams),
+                                         static_cast<size_t>(gc.smem), P, s, args);
             if (e != cudaSuccess) return cuda_status(e);
             g_launch_count.fetch_add(1);
             return CREDIT_OK;
@@ -921,7 +942,7 @@ int32_t credit_max_clusters(const credit_args *args, const credit_plan_t *plan) 
     const int tout = args->op == OP_LSE ? DT_F32 : args->out_dtype;
     TeamCfg gc;
     if (team_plan_config(*di, args, plan, &gc))
-        return staged_max_clusters(dev, team_kernel(args->op, args->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0), 1, gc.threads * gc.teams, gc.smem,
+        return staged_max_clusters(dev, team_kernel(args->op, args->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
                                    false);
     RingCfg rc;
     if (!ring_config_for(*di, args, dtype_size(args->in_dtype), P, plan, &rc)) return 0;

@@ -1137,12 +1137,12 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                 fn(gi, fa, fd);
             }
         };
+        const AffineRow<NP> ar(gp, GRID || !AFF ? 0 : g.h0);
         // dy gamma of a group
         auto times_gamma = [&](int gi, float (&fd)[V]) {
             if constexpr (kNorm<OP>) {
                 float fg[V];
-                if constexpr (AFF && GRID) planes_group<NP>(gp, gi, 0, fg);
-                else if constexpr (AFF) planes_load<NP>(gp, g.h0 + gi * V, fg);
+                if constexpr (AFF) affine_pair<GRID, false>(ar, gp, gp, g.h0 + gi * V, gi, 0, fg, fg);
                 else ldg_shift<V>(p.gamma, g.h0 + gi * V, N, 1.0f, fg);
 #pragma unroll
                 for (int v = 0; v < V; v += 2) {

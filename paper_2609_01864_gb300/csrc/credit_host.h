@@ -47,16 +47,18 @@ constexpr long long kTmAutoMinSlice = 32768;
 bool ring_config_tm(const DeviceInfo &di, long long N, int isz, int P, int req_ring, int req_chunk, int nab,
                     RingCfg *out);
 // Geometry of k_row_team: teams of `threads` threads, `teams` of them in the
-// SM's one CTA, `stages` rows in flight per team.
+// SM's one CTA, `stages` rows in flight per team; rows split over clusters of
+// P CTAs, `grid` of them.
 struct TeamCfg {
-    int threads, teams, stages, grid;
+    int P, threads, teams, stages, grid;
     int affine_resident;  // gamma / beta staged in shared memory
     bool grid_rows;       // every row starts and ends on the 16-byte grid of both tensors
     long long smem;
 };
 // nab: gamma / beta arrays of the op (0, 1 or 2).  False where a row does not fit.
-bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int nab, int req_stages, TeamCfg *out);
-// A ONE_CTA plan that asks for whole rows, and a row that allows it.
+bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int nab, int P, int req_stages,
+                 TeamCfg *out);
+// A ONE_CTA or CLUSTER plan that asks for whole rows, and a row that allows it.
 bool team_plan_config(const DeviceInfo &di, const credit_args *a, const credit_plan_t *p, TeamCfg *out);
 int ring_max_clusters(int device, int op, int tin, int tout, int P, int threads, long long smem, bool tm = false);
 int affine_arrays(const credit_args *a);

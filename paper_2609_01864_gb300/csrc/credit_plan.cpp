@@ -97,37 +97,61 @@ int two_pass_split(int sm_count, long long rows, long long cols, int isz) {
     return static_cast<int>(G < 1 ? 1 : G);
 }
 
-// Narrow rows: the one-CTA path with whole rows in shared memory (k_row_team),
-// up to the row width at which it stops being the fastest plan.  Measured on
-// GB300 against the learned model's picks (rows 96-16384, widths 256 B to 96
-// KiB, on and off the 16-byte grid; us, the model's pick -> this one):
-//   16384 x 4096 BF16 RMSNorm 80 -> 48, 65536 x 1024 FP32 softmax 252 -> 92,
-//   20325 x 3616 BF16 softmax 130 -> 52, 16384 x 8192 BF16 -> FP8 RMSNorm
-//   167 -> 81, FP8 LayerNorm 332 -> 112, 10800 x 4096 BF16 int8 93 -> 29,
+// Rows (or slices of rows) of one CTA's teams that fit shared memory beside the op's gamma / beta.
+static long long team_room(const DeviceInfo &di, long long cols, int isz, int nab, int P) {
+    const long long V = 16 / isz, groups = (cols / V + P - 1) / P;
+    const long long aff = nab * (groups + 3) * V * 4, room = di.smem_optin - (20 << 10) - aff;
+    return groups < 1 ? 16 : room < 0 ? 0 : room / (groups * 16);
+}
+
+// Rows for k_row_team: whole rows in one CTA (P = 1), or split over a cluster.
+// Measured on GB300 against the learned model's picks (us, the model's pick ->
+// this one).
+// P = 1, rows of 256 B to 96 KiB, 96 to 16384 of them, on and off the 16-byte
+// grid:
+//   16384 x 4096 BF16 RMSNorm 80 -> 47, 65536 x 1024 FP32 softmax 252 -> 92,
+//   20325 x 3616 BF16 softmax 130 -> 50, 16384 x 8192 BF16 -> FP8 RMSNorm
+//   167 -> 81, FP8 LayerNorm 332 -> 115, 10800 x 4096 BF16 int8 93 -> 26,
 //   1000 rows of 24 KiB: 5-60% faster for every op and type but FP8 softmax.
-// The limits: norms of rows on the 16-byte grid go to the tensor-memory path
+// Its limits: norms of rows on the 16-byte grid go to the tensor-memory path
 // from 48 KiB (1000 x 64 KiB BF16 RMSNorm 29 against 38), off the grid, where
 // that path loses its staged gamma / beta, only above 96 KiB; E4M3 softmax and
 // log-sum-exp have their code tables (24 KiB rows of FP8 log-sum-exp 11
 // against 15, 32 KiB of FP8 softmax 13 against 15); log-sum-exp has no output
 // for the second look at the row to save, in BF16 it draws level at 32 KiB.
+// P > 1, where the other paths are weak: rows off the grid, and norms with FP8
+// rows or outputs.  The smallest P that leaves an SM room for three teams with
+// gamma / beta (1500 rows; with two teams the copies show: 300 KiB BF16
+// LayerNorm P = 8 580, P = 16 296, 504 before): LayerNorm 140 KiB FP32 128 ->
+// 110, BF16 252 -> 140, FP8 1359 -> 436, RMSNorm 200 KiB BF16 217 -> 146, 140
+// KiB BF16 -> FP8 252 -> 126 (on the grid 208 -> 120), FP8 726 -> 267, softmax
+// 300 KiB BF16 222 -> 194, int8 200 KiB BF16 234 -> 102; without gamma P = 2
+// stays behind P = 4 (140 KiB int8 84 against 71).  Few rows keep P = 1 up to
+// 96 KiB (100 x 48 KiB FP32 LayerNorm 9 against 12) unless they are FP8, whose
+// arithmetic is worth more CTAs (100 x 64 KiB LayerNorm 40 -> 24).
 static bool row_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, int tout,
                      credit_plan_t *p) {
-    const int isz = dtype_size(tin);
-    const bool norm = op == CREDIT_OP_LAYERNORM || op == CREDIT_OP_RMSNORM;
+    const int isz = dtype_size(tin), nab = op == CREDIT_OP_LAYERNORM ? 2 : op == CREDIT_OP_RMSNORM ? 1 : 0;
+    const bool grid = cols * isz % 16 == 0, fp8 = tin == 2 || tout == 2, sm8 = op == CREDIT_OP_SOFTMAX && tin == 2;
+    const long long bytes = cols * isz;
     long long limit = 96 << 10;
     if (op == CREDIT_OP_LOGSUMEXP) limit = tin == 0 ? limit : tin == 1 ? 32 << 10 : 8 << 10;
-    else if (op == CREDIT_OP_SOFTMAX && tin == 2) limit = 24 << 10;
-    else if (norm && tin != 2 && tout != 2 && cols * isz % 16 == 0) limit = 48 << 10;
+    else if (sm8) limit = 24 << 10;
+    else if (nab && !fp8 && grid) limit = 48 << 10;
+    int P = bytes <= limit ? 1 : 0;
+    const bool split = op != CREDIT_OP_LOGSUMEXP && !sm8 && (!grid || (nab && fp8)) && bytes <= (grid ? 450 << 10 : 1 << 20);
+    if (split && (P == 0 || (nab && (tin == 2 || rows >= 4LL * di.sm_count)))) {
+        int q = nab || P ? 1 : 4;
+        while (q <= 16 && team_room(di, cols, isz, nab, q) < 3) q *= 2;
+        if (q <= 16 && (q > 1 || P)) P = q;
+    }
     TeamCfg tc;
-    if (cols * isz > limit ||
-        !team_config(di, rows, cols, isz, op == CREDIT_OP_LAYERNORM ? 2 : op == CREDIT_OP_RMSNORM, 0, &tc))
-        return false;
+    if (P == 0 || !team_config(di, rows, cols, isz, nab, P, 0, &tc)) return false;
     std::memset(p, 0, sizeof(*p));
     p->source = 3;
-    p->path = CREDIT_PATH_ONE_CTA;
-    p->cluster_size = 1;
-    p->ctas_per_row = 1;
+    p->path = P == 1 ? CREDIT_PATH_ONE_CTA : CREDIT_PATH_CLUSTER;
+    p->cluster_size = P;
+    p->ctas_per_row = P;
     p->retain = CREDIT_RETAIN_ROW;
     p->smem_bytes = tc.smem;
     return true;

@@ -39,7 +39,10 @@ constexpr int kTeamMaxStages = 4;
 // Shared memory: [0, 1024) mbarriers [team][stage], [1024, 1024 + teams * 512)
 // reduction scratch [team][4][32 floats], gamma, beta (16-byte
 // multiples plus one pad group each), then the stages.
-__host__ __device__ constexpr int team_ctrl_bytes(int teams) { return kTeamMaxTeams * kTeamMaxStages * 8 + teams * 512; }
+constexpr int kTeamXchBytes = 544;  // cluster exchange of one team: 512 bytes of slots, four mbarriers
+__host__ __device__ constexpr int team_ctrl_bytes(int teams, bool cluster) {
+    return kTeamMaxTeams * kTeamMaxStages * 8 + teams * (512 + (cluster ? kTeamXchBytes : 0));
+}
 
 // gamma / beta in shared memory, in planes: float4 number j = i / 4 of the
 // array lies in plane j % NP at position j / NP, NP = V / 4 float4s per
@@ -55,15 +58,34 @@ struct AffinePlanes {
 template <int NP>
 __host__ __device__ constexpr int affine_np(int N) { return ((N + 3) / 4 + NP - 1) / NP + 1; }
 
-// Group i's SV values at hv of a row on the 16-byte grid (no shift).
-template <int NP, int SV>
-__device__ __forceinline__ void planes_group(const AffinePlanes &a, int i, int hv, float (&v)[SV]) {
-    const uint32_t base = smem_addr(a.p) + 16u * static_cast<uint32_t>(i);
+// Where one row's groups find their values: group gi, starting at column
+// i0 + gi * V of the array, reads float4s k = 0, 1, ... at a[k] + 16 gi (a
+// group is NP float4s, so float4 k of every group lies in one plane).  i0 may
+// lie anywhere: q = i0 % 4 values of float4 0 belong to the group before.
+template <int NP>
+struct AffineRow {
+    uint32_t a[NP + 1];
+    int q;
+    __device__ __forceinline__ AffineRow(const AffinePlanes &p, int i0) : q(i0 & 3) {
+        const int j0 = i0 >> 2;
 #pragma unroll
-    for (int k = 0; k < SV / 4; ++k)
+        for (int k = 0; k <= NP; ++k)
+            a[k] = smem_addr(p.p) + 16u * static_cast<uint32_t>((j0 + k) % NP * p.np + (j0 + k) / NP);
+    }
+};
+// SV values from element hv of group gi on, Q = r.q known at compile time: the float4s that cover them, whole
+// (one more than SV / 4 where Q > 0), `array` bytes after the first array (beta after gamma).
+template <int Q, int NP, int SV>
+__device__ __forceinline__ void affine_load(const AffineRow<NP> &r, uint32_t array, int gi, int hv, float (&v)[SV]) {
+    constexpr int n = SV / 4 + (Q > 0 ? 1 : 0);
+    float f[4 * n];
+#pragma unroll
+    for (int k = 0; k < n; ++k)
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(v[4 * k]), "=f"(v[4 * k + 1]), "=f"(v[4 * k + 2]), "=f"(v[4 * k + 3])
-                     : "r"(base + 16u * static_cast<uint32_t>((hv / 4 + k) * a.np)));
+                     : "=f"(f[4 * k]), "=f"(f[4 * k + 1]), "=f"(f[4 * k + 2]), "=f"(f[4 * k + 3])
+                     : "r"(r.a[hv / 4 + k] + array + 16u * static_cast<uint32_t>(gi)));
+#pragma unroll
+    for (int j = 0; j < SV; ++j) v[j] = f[j + Q];
 }
 
 template <int NP>
@@ -78,7 +100,7 @@ __device__ __forceinline__ void planes_fill(float *dst, int np, const float *src
 // at any column): the vectors that cover the values are read whole and shifted
 // (SV / 4 + 1 reads instead of SV).
 template <int NP, int SV>
-__device__ __forceinline__ void planes_load(const AffinePlanes &a, int i0, float (&v)[SV]) {
+__device__ __forceinline__ void affine_shift(const AffinePlanes &a, int i0, float (&v)[SV]) {
     const int q = i0 & 3, j0 = i0 >> 2;
     auto ld = [&](int k, float *f) {
         const int j = j0 + k;
@@ -99,6 +121,32 @@ __device__ __forceinline__ void planes_load(const AffinePlanes &a, int i0, float
     for (int k = 0; k < SV + 2; ++k) f[k] = q1 ? f[k + 1] : f[k];
 #pragma unroll
     for (int k = 0; k < SV; ++k) v[k] = q2 ? f[k + 2] : f[k];
+}
+
+// gamma and, with TWO, beta of part of a group (b: beta's planes), the row's phase q tested here.  BF16 rows
+// (NP = 2) have one copy of the reads per phase: the selects of affine_shift cost them 5 of some 30 instructions
+// per element (16384 x 4095 LayerNorm 79 -> 73 us); FP32 and FP8 rows measure better with the selects (4096 x
+// 6001 FP32 LayerNorm 50 against 55, where the copies spill).
+template <bool GRID, bool TWO, int NP, int SV>
+__device__ __forceinline__ void affine_pair(const AffineRow<NP> &r, const AffinePlanes &pg, const AffinePlanes &pb,
+                                            int i0, int gi, int hv, float (&g)[SV], float (&b)[SV]) {
+    const uint32_t at = TWO ? smem_addr(pb.p) - smem_addr(pg.p) : 0u;
+    if (GRID || (NP == 2 && r.q == 0)) {
+        affine_load<0>(r, 0u, gi, hv, g);
+        if constexpr (TWO) affine_load<0>(r, at, gi, hv, b);
+    } else if constexpr (NP != 2) {
+        affine_shift<NP>(pg, i0, g);
+        if constexpr (TWO) affine_shift<NP>(pb, i0, b);
+    } else if (r.q == 1) {
+        affine_load<1>(r, 0u, gi, hv, g);
+        if constexpr (TWO) affine_load<1>(r, at, gi, hv, b);
+    } else if (r.q == 2) {
+        affine_load<2>(r, 0u, gi, hv, g);
+        if constexpr (TWO) affine_load<2>(r, at, gi, hv, b);
+    } else {
+        affine_load<3>(r, 0u, gi, hv, g);
+        if constexpr (TWO) affine_load<3>(r, at, gi, hv, b);
+    }
 }
 
 // V floats from i0 on of an array of N in global memory (L1 / L2; a null array
@@ -260,7 +308,7 @@ __device__ __forceinline__ void exp_args(const uint4 &w, int hv, float a, float 
 // (no head or tail elements, one geometry for all rows); otherwise each row is
 // cut on the grid of its own address.  AFF: gamma / beta (ones / zeros where
 // null) in shared memory; otherwise read through L1.
-template <int OP, int TIN, int TOUT, bool GRID, bool AFF>
+template <int OP, int TIN, int TOUT, bool GRID, bool AFF, bool CL>
 __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int isz = Fmt<TIN>::size, V = Fmt<TIN>::V, osz = Fmt<TOUT>::size, NP = V / 4;
@@ -273,29 +321,39 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
 
     const int T = blockDim.x, t = threadIdx.x, team = threadIdx.y, teams = blockDim.y, S = a.ring;
     const int N = static_cast<int>(a.cols);
-    const int gmax = N / V;  // groups of a row are at most this many
+    const int P = CL ? static_cast<int>(cluster_nctarank()) : 1, c = CL ? static_cast<int>(cluster_ctarank()) : 0;
+    const int lp = CL ? 31 - __clz(P) : 0;           // P is a power of two
+    const int gmax = (N / V + P - 1) >> lp;          // groups of a row's slice are at most this many
+    const int cb = CL ? ((N / V - 1) * c >> lp) * V : 0;  // no slice of this CTA starts before this column
+    const int cn = CL ? min(N - cb, gmax * V + 3 * V) : N;  // columns of gamma / beta any slice needs
     uint64_t *full = reinterpret_cast<uint64_t *>(smem) + team * kTeamMaxStages;
     float *red = reinterpret_cast<float *>(smem + kTeamMaxTeams * kTeamMaxStages * 8) + team * 128;
     const bool has_g = kNormOp && a.gamma != nullptr, has_b = OP == OP_LN && a.beta != nullptr;
-    const int np = affine_np<NP>(N);
-    float *gsm = reinterpret_cast<float *>(smem + team_ctrl_bytes(teams));
+    const int np = affine_np<NP>(cn);
+    float *gsm = reinterpret_cast<float *>(smem + team_ctrl_bytes(teams, CL));
     float *bsm = gsm + (AFF ? NP * np * 4 : 0);
     const AffinePlanes gp{gsm, np}, bp{bsm, np};
     unsigned char *stages = reinterpret_cast<unsigned char *>(bsm + (AFF && OP == OP_LN ? NP * np * 4 : 0)) +
                             static_cast<size_t>(team) * S * gmax * 16;
-    const long long stride = static_cast<long long>(gridDim.x) * teams;
-    const long long row_first = static_cast<long long>(blockIdx.x) * teams + team;
+    // cluster exchange (CL): slots [stage][row parity][16 sources][2 floats] and mbarriers [stage][parity] of the team
+    unsigned char *xch = smem + team_ctrl_bytes(teams, false) + team * kTeamXchBytes;
+    uint64_t *xbar = reinterpret_cast<uint64_t *>(xch + 512);
+    const long long stride = static_cast<long long>(gridDim.x >> lp) * teams;
+    const long long row_first = static_cast<long long>(blockIdx.x >> lp) * teams + team;
     const float inv_n = 1.0f / static_cast<float>(N);
 
+    // a row's head, groups and tail, and the groups lo .. lo + n - 1 of this CTA's slice
     struct Geo {
-        int h0, G, t0;
+        int h0, G, t0, lo, n;
     };
     auto geo = [&](const unsigned char *row) {
-        if constexpr (GRID) return Geo{0, gmax, 0};
+        if constexpr (GRID) return Geo{0, gmax, 0, 0, gmax};
         Geo g;
         g.h0 = min(static_cast<int>((0u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row))) & 15u) / isz, N);
         g.G = (N - g.h0) / V;
         g.t0 = (N - g.h0) % V;
+        g.lo = CL ? g.G * c >> lp : 0;
+        g.n = CL ? (g.G * (c + 1) >> lp) - g.lo : g.G;
         return g;
     };
     auto in_row = [&](long long row) { return a.in + row * a.ld_in * isz; };
@@ -303,10 +361,10 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
     auto issue = [&](long long row, int slot) {
         const unsigned char *p = in_row(row);
         const Geo g = geo(p);
-        if (!GRID && g.G == 0) return;
-        const uint32_t bytes = static_cast<uint32_t>(g.G) * 16u;
+        if (!GRID && g.n == 0) return;
+        const uint32_t bytes = static_cast<uint32_t>(g.n) * 16u;
         unsigned char *dst = stages + static_cast<uint32_t>(slot) * (gmax * 16u);
-        const unsigned char *src = p + g.h0 * isz;
+        const unsigned char *src = p + g.h0 * isz + g.lo * 16;
         mbar_arrive_expect_tx(&full[slot], bytes);
         for (uint32_t o = 0; o < bytes; o += kMaxChunkBytes)
             bulk_g2s(dst + o, src + o, min(bytes - o, static_cast<uint32_t>(kMaxChunkBytes)), &full[slot]);
@@ -314,22 +372,48 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
     // edge elements, one per thread (fewer than 16 of each; a team has at least 32 threads)
     auto edge_index = [&](const Geo &g) -> int {
         if constexpr (GRID) return -1;
-        return t < g.h0 ? t : (T - 1 - t < g.t0 ? g.h0 + g.G * V + (T - 1 - t) : -1);
+        if ((!CL || c == 0) && t < g.h0) return t;
+        return (!CL || c == P - 1) && T - 1 - t < g.t0 ? g.h0 + g.G * V + (T - 1 - t) : -1;
     };
 
     // the first rows are requested before anything else; only this thread uses the barriers before the block's
     // barrier below
     if (t == 0) {
         for (int k = 0; k < S; ++k) mbar_init(&full[k], 1);
+        if constexpr (CL) {
+            for (int k = 0; k < 4; ++k) mbar_init(&xbar[k], 1);
+        }
         fence_mbar_init();
         for (int k = 0; k < S; ++k)
             if (row_first + k * stride < a.rows) issue(row_first + k * stride, k);
     }
     if constexpr (AFF) {  // gamma / beta, once for every row of this SM
-        planes_fill<NP>(gsm, np, a.gamma, 1.0f, N, team * T + t, T * teams);
-        if constexpr (OP == OP_LN) planes_fill<NP>(bsm, np, a.beta, 0.0f, N, team * T + t, T * teams);
+        planes_fill<NP>(gsm, np, has_g ? a.gamma + cb : nullptr, 1.0f, cn, team * T + t, T * teams);
+        if constexpr (OP == OP_LN)
+            planes_fill<NP>(bsm, np, has_b ? a.beta + cb : nullptr, 0.0f, cn, team * T + t, T * teams);
     }
     __syncthreads();
+    if constexpr (CL) {  // every peer's exchange barriers exist before the first push
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
+    // Push all-gather of two floats per CTA among the cluster's teams of one number (Eq. 5): each CTA's partial
+    // goes to slot c of every CTA, its own included.  Slots and barriers alternate with the row: a CTA pushes into
+    // a parity again only after its exchange of the row between, which needed a push that each peer made after it
+    // had read this parity's slots.  Lane q < P returns CTA q's partial.
+    auto exchange = [&](int stage, float p0, float p1, uint32_t k) -> float2 {
+        const uint32_t par = k & 1u;
+        float *slots = reinterpret_cast<float *>(xch) + (stage * 2 + par) * 32;
+        uint64_t *bar = &xbar[stage * 2 + par];
+        if (t < P) {
+            fence_release_smem_cluster();
+            st_async_v2f32(mapa_shared(smem_addr(slots + 2 * c), t), p0, p1, mapa_shared(smem_addr(bar), t));
+        }
+        if (t == 0) mbar_arrive_expect_tx(bar, static_cast<uint32_t>(P) * 8u);
+        mbar_wait_bounded_cluster(bar, (k >> 1) & 1u, a.err);
+        const int q = t & 31;
+        return q < P ? make_float2(slots[2 * q], slots[2 * q + 1]) : make_float2(0.0f, 0.0f);
+    };
 
     float rawn = 0.0f, scn = 1.0f;  // the next row's edge element (unscaled) and input scale
     auto fetch_next = [&](long long row) {
@@ -347,6 +431,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
     int slot = 0;
     uint32_t lap = 0;
     bool odd = false;  // row parity: reductions that are a row's only one alternate between two arrays
+    uint32_t it = 0;   // rows done (CL)
     for (long long row = row_first; row < a.rows; row += stride, out_p += out_step, odd = !odd) {
         const Geo g = geo(GRID ? nullptr : in_row(row));
         const int ie = edge_index(g);
@@ -356,7 +441,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
         const unsigned char *stage = stages + static_cast<uint32_t>(slot) * (gmax * 16u);
 
         // ---- the row in shared memory
-        if (GRID || g.G > 0) mbar_wait_bounded(&full[slot], lap & 1u, a.err);
+        if (GRID || g.n > 0) mbar_wait_bounded(&full[slot], lap & 1u, a.err);
         const uint32_t neg = TIN == DT_E4M3 && kSm ? e4m3_sign_mask(in_sc) : 0u;
         auto lds = [&](int gi) {
             const uint4 x = *reinterpret_cast<const uint4 *>(stage + 16 * gi);
@@ -365,10 +450,10 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
         };
         auto each = [&](auto &&fn) {  // this thread's groups
 #pragma unroll 1
-            for (int gi = t; gi < g.G; gi += T) fn(gi, lds(gi));
+            for (int gi = t; gi < g.n; gi += T) fn(gi, lds(gi));
         };
         float K = 0.0f;
-        if constexpr (OP == OP_LN) K = decode_one<TIN>(GRID || g.G > 0 ? stage : in_row(row), in_sc);
+        if constexpr (OP == OP_LN) K = decode_one<TIN>(GRID || g.n > 0 ? stage : in_row(row), in_sc);
         const float a1 = fabsf(in_sc);
         // after the row's first reduction: every thread is done with the previous row, whose stage takes its next
         // row (one stage: at the end of the row instead)
@@ -407,6 +492,13 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
             });
             if (edge) sum += ex2_ftz(fmaf(xe - mz, kLog2e, lift));
             st.b = team_reduce<false>(sum, red + 32, team, T);
+            if constexpr (CL) {  // (max, sum) of every slice about the row's maximum
+                const float2 p = exchange(0, st.a, st.b, it);
+                const bool mine = (t & 31) < P;
+                st.a = warp_max_redux(mine ? p.x : -INFINITY);
+                // an all -inf slice has the sum 0 about 0; a NaN sum stays NaN
+                st.b = warp_sum(mine ? (p.x == -INFINITY ? p.y : p.y * ex2_ftz((p.x - st.a) * kLog2e)) : 0.0f);
+            }
         } else if constexpr (OP == OP_LN) {
             float2 s2 = make_float2(0.0f, 0.0f);
             each([&](int gi, const uint4 &x) {
@@ -423,7 +515,9 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
             if (edge) s1 += xe - K;
             s1 = team_reduce<false>(s1, red, team, T);
             refill();
-            st.a = fmaf(s1, inv_n, K);
+            // the slice's count, mean and squared deviations (the row's where it is not split)
+            const float n_c = CL ? static_cast<float>(g.n * V + (c == 0 ? g.h0 : 0) + (c == P - 1 ? g.t0 : 0)) : 1.0f;
+            st.a = CL ? K + s1 / n_c : fmaf(s1, inv_n, K);
             float2 q2 = make_float2(0.0f, 0.0f);
             each([&](int gi, const uint4 &x) {
 #pragma unroll
@@ -440,6 +534,18 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
             float m2 = q2.x + q2.y;
             if (edge) m2 = fmaf(xe - st.a, xe - st.a, m2);
             m2 = team_reduce<false>(m2, red + 32, team, T);
+            if constexpr (CL) {
+                // mean = m_0 + sum n_q (m_q - m_0) / N, M2 = sum (M2_q + n_q (m_q - mean)^2)
+                const float2 p = exchange(0, st.a, m2, it);
+                const int q = t & 31;
+                const float n_q = q < P ? static_cast<float>(((g.G * (q + 1) >> lp) - (g.G * q >> lp)) * V +
+                                                             (q == 0 ? g.h0 : 0) + (q == P - 1 ? g.t0 : 0))
+                                        : 0.0f;
+                const float m_0 = __shfl_sync(0xffffffffu, p.x, 0);
+                st.a = fmaf(warp_sum(n_q * (p.x - m_0)), inv_n, m_0);
+                const float d = p.x - st.a;
+                m2 = warp_sum(fmaf(n_q * d, d, p.y));
+            }
             st.b = rsqrtf(fmaf(m2, inv_n, a.eps));
         } else if constexpr (OP == OP_RMS) {
             float2 q2 = make_float2(0.0f, 0.0f);
@@ -459,33 +565,34 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
             if (edge) ss = fmaf(xe, xe, ss);
             ss = team_reduce<false>(ss, red + (odd ? 32 : 0), team, T);
             refill();
+            if constexpr (CL) ss = warp_sum(exchange(0, ss, 0.0f, it).x);
             st.a = rsqrtf(fmaf(ss, inv_n, a.eps));
         } else {
             GroupMax<TIN, true> gm;
             each([&](int, const uint4 &x) { gm.add(x); });
             float am = fmaxf(gm.value(), 0.0f);
             if (edge) am = fmaxf(am, fabsf(xe));
-            const float p[2] = {team_reduce<true>(am, red + (odd ? 32 : 0), team, T), 0.0f};
+            am = team_reduce<true>(am, red + (odd ? 32 : 0), team, T);
             refill();
+            if constexpr (CL) am = warp_max_redux(exchange(0, am, 0.0f, it).x);
+            const float p[2] = {am, 0.0f};
             st = combine_partials<OP>(p, 2, 1, RowSlice{}, V, N, a.eps);
         }
 
         // ---- outputs
         if constexpr (OP == OP_LSE) {
-            if (t == 0) reinterpret_cast<float *>(a.out)[row] = st.a + logf(st.b);
+            if (c == 0 && t == 0) reinterpret_cast<float *>(a.out)[row] = st.a + logf(st.b);
         } else {
             // the norms' outputs hv .. hv + SV - 1 of group u, before the FP8 scaling
+            const AffineRow<NP> ar(gp, GRID || !AFF ? 0 : g.h0 + g.lo * V - cb);
             auto norm_part = [&](int gi, const uint4 &x, int hv, float (&y)[SV]) {
-                const int i0 = g.h0 + gi * V + hv;
                 float gg[SV], bb[SV];
                 decode_part<TIN>(x, hv, in_sc, y);
-                if constexpr (AFF && GRID) planes_group<NP>(gp, gi, hv, gg);
-                else if constexpr (AFF) planes_load<NP>(gp, i0, gg);
-                else ldg_shift<SV>(a.gamma, i0, N, 1.0f, gg);
-                if constexpr (OP == OP_LN) {
-                    if constexpr (AFF && GRID) planes_group<NP>(bp, gi, hv, bb);
-                    else if constexpr (AFF) planes_load<NP>(bp, i0, bb);
-                    else ldg_shift<SV>(a.beta, i0, N, 0.0f, bb);
+                if constexpr (AFF) {
+                    affine_pair<GRID, OP == OP_LN>(ar, gp, bp, g.h0 + (g.lo + gi) * V + hv - cb, gi, hv, gg, bb);
+                } else {
+                    ldg_shift<SV>(a.gamma, g.h0 + (g.lo + gi) * V + hv, N, 1.0f, gg);
+                    if constexpr (OP == OP_LN) ldg_shift<SV>(a.beta, g.h0 + (g.lo + gi) * V + hv, N, 0.0f, bb);
                 }
 #pragma unroll
                 for (int j = 0; j < SV; j += 2) {  // norm_h, two elements per packed op
@@ -518,18 +625,19 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
                 });
                 if (edge) am = fmaxf(am, fabsf(norm_edge()));
                 am = team_reduce<true>(am, red + 64 + (odd ? 32 : 0), team, T);
+                if constexpr (CL) am = warp_max_redux(exchange(1, am, 0.0f, it).x);
                 mul = am > 0.0f ? 448.0f / am : 1.0f;
-                if (t == 0) a.out_scale[row] = am > 0.0f ? am / 448.0f : 1.0f;
+                if (c == 0 && t == 0) a.out_scale[row] = am > 0.0f ? am / 448.0f : 1.0f;
             } else if constexpr (OP == OP_SOFTMAX) {
                 mul = TOUT == DT_E4M3 ? 448.0f : 1.0f / st.b;
                 cL = TOUT == DT_E4M3 ? 8.807354922057604f /* log2 448 */ : kExpLift - log2f(st.b);
                 if constexpr (TOUT == DT_E4M3) {
-                    if (t == 0) a.out_scale[row] = (1.0f / st.b) * (1.0f / 448.0f);
+                    if (c == 0 && t == 0) a.out_scale[row] = (1.0f / st.b) * (1.0f / 448.0f);
                 }
             } else if constexpr (OP == OP_Q8) {
-                if (t == 0) a.out_scale[row] = st.a;
+                if (c == 0 && t == 0) a.out_scale[row] = st.a;
             }
-            unsigned char *out_body = out_p + g.h0 * osz;
+            unsigned char *out_body = out_p + (g.h0 + g.lo * V) * osz;
             const bool out_vec = GRID || (reinterpret_cast<uintptr_t>(out_body) % vec_bytes) == 0;
             each([&](int gi, const uint4 &x) {
                 uint32_t ow[V * osz / 4];
@@ -583,6 +691,11 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_row_team(const RowArgs a
             slot = 0;
             ++lap;
         }
+        if constexpr (CL) ++it;
+    }
+    if constexpr (CL) {  // no CTA leaves while a peer may still push into it
+        cluster_arrive_release();
+        cluster_wait_acquire();
     }
 }
 

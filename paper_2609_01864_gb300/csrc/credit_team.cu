@@ -11,35 +11,36 @@
 
 namespace credit {
 
+// Clusters: rows at any phase, gamma / beta always in shared memory.
 template <int OP, int TOUT>
-static const void *team_fn(bool grid, bool aff) {
-    if constexpr (OP == OP_LN || OP == OP_RMS) {
-        if (aff)
-            return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, true>)
-                        : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, true>);
-    }
-    return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, false>)
-                : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, false>);
+static const void *team_fn(bool grid, bool aff, bool cluster) {
+    constexpr bool N = OP == OP_LN || OP == OP_RMS;
+    if (cluster) return reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, true>);
+    if (N && aff)
+        return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, N, false>)
+                    : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, false>);
+    return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, false, false>)
+                : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, false, false>);
 }
 
 template <int OP>
-static const void *team_out(int tout, bool grid, bool aff) {
+static const void *team_out(int tout, bool grid, bool aff, bool cluster) {
     switch (tout) {
-    case DT_F32: return team_fn<OP, DT_F32>(grid, aff);
-    case DT_BF16: return team_fn<OP, DT_BF16>(grid, aff);
-    case DT_E4M3: return team_fn<OP, DT_E4M3>(grid, aff);
+    case DT_F32: return team_fn<OP, DT_F32>(grid, aff, cluster);
+    case DT_BF16: return team_fn<OP, DT_BF16>(grid, aff, cluster);
+    case DT_E4M3: return team_fn<OP, DT_E4M3>(grid, aff, cluster);
     default: return nullptr;
     }
 }
 
-const void *CREDIT_CAT(team_kernel_tin, CREDIT_TIN)(int op, int tout, bool grid, bool aff) {
+const void *CREDIT_CAT(team_kernel_tin, CREDIT_TIN)(int op, int tout, bool grid, bool aff, bool cluster) {
     switch (op) {
-    case OP_SOFTMAX: return team_out<OP_SOFTMAX>(tout, grid, aff);
-    case OP_LSE: return team_fn<OP_LSE, DT_F32>(grid, aff);
-    case OP_LN: return team_out<OP_LN>(tout, grid, aff);
-    case OP_RMS: return team_out<OP_RMS>(tout, grid, aff);
+    case OP_SOFTMAX: return team_out<OP_SOFTMAX>(tout, grid, aff, cluster);
+    case OP_LSE: return team_fn<OP_LSE, DT_F32>(grid, aff, cluster);
+    case OP_LN: return team_out<OP_LN>(tout, grid, aff, cluster);
+    case OP_RMS: return team_out<OP_RMS>(tout, grid, aff, cluster);
 #if CREDIT_TIN != 2
-    case OP_Q8: return tout == DT_I8 ? team_fn<OP_Q8, DT_I8>(grid, aff) : nullptr;
+    case OP_Q8: return tout == DT_I8 ? team_fn<OP_Q8, DT_I8>(grid, aff, cluster) : nullptr;
 #endif
     default: return nullptr;
     }

@@ -83,8 +83,38 @@ def test_any_phase(op, tin, tout, off_in, off_out, ld_in, ld_out):
     assert (guard[:off_out].float() == 3.0).all() and (y[:, cols:].float() == 3.0).all()
 
 
+@pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("tin,tout", [(C.F32, C.F32), (C.BF16, C.BF16), (C.FP8_E4M3, C.FP8_E4M3), (C.BF16, C.FP8_E4M3)])
+@pytest.mark.parametrize("P", [2, 4, 8, 16])
+@pytest.mark.parametrize("groups,extra,rows", [(32, 0, 700), (131, 3, 700), (1023, 1, 90), (2049, -1, 7)])
+def test_clusters(op, tin, tout, P, groups, extra, rows):
+    """Rows split over a cluster: `groups` 16-byte groups per CTA (32: the fewest the plan takes as such), slices of
+    unlike sizes, several rows per team so that every exchange slot and stage is reused, rows off the grid."""
+    cols = P * groups * 16 // SIZE[tin] + extra
+    if op == C.LOGSUMEXP:
+        tout = C.F32
+    x, s, g, b = _case(op, tin, tout, rows, cols, cols + P)
+    plan = C.make_plan(C.PATH_CLUSTER, P, retain=C.RETAIN_ROW)
+    y = torch.empty(1, device="cuda")
+    if C.plan_check(op, x.cuda(), y, plan, out_dtype=tout, in_scale=None if s is None else s.cuda(),
+                    out_scale=y) != C.OK:
+        pytest.skip("gamma / beta and a slice exceed shared memory, and so does AUTO")
+    U.check_against_oracle(op, x, s, out_dtype=tout, plan=plan, gamma=g, beta=b)
+
+
+@pytest.mark.parametrize("op", [C.SOFTMAX, C.LAYERNORM, C.RMSNORM])
 @pytest.mark.parametrize("dt", [C.F32, C.BF16])
-@pytest.mark.parametrize("cols", [8, 100, 4096, 20001])
+def test_planned_rows_off_the_grid(op, dt):
+    """The planner's choice on wide rows off the 16-byte grid is a cluster of this kernel and matches the oracle."""
+    cols = 140 * 1024 // SIZE[dt] - 3
+    p = C.plan(op, 700, cols, dt)
+    assert (p.path, p.retain) == (C.PATH_CLUSTER, C.RETAIN_ROW)
+    x, s, g, b = _case(op, dt, dt, 48, cols, 5)
+    U.check_against_oracle(op, x, s, gamma=g, beta=b)
+
+
+@pytest.mark.parametrize("dt", [C.F32, C.BF16])
+@pytest.mark.parametrize("cols", [8, 100, 4096, 20001, 60001])
 def test_int8_and_in_place(dt, cols):
     import numpy as np
     import oracle as O
@@ -92,12 +122,13 @@ def test_int8_and_in_place(dt, cols):
     x[5] = 0
     d = x.cuda()
     y, sc = torch.empty(200, cols, dtype=torch.int8, device="cuda"), torch.empty(200, device="cuda")
-    C.run_ex(C.QUANT_INT8, d, y, plan=ROW, in_dtype=dt, out_dtype=C.INT8, out_scale=sc)
+    plan = ROW if cols < 60000 else C.make_plan(C.PATH_CLUSTER, 4, retain=C.RETAIN_ROW)
+    C.run_ex(C.QUANT_INT8, d, y, plan=plan, in_dtype=dt, out_dtype=C.INT8, out_scale=sc)
     codes, scales = O.quant_int8(x.float().numpy())
     assert np.array_equal(y.cpu().numpy(), codes) and np.array_equal(sc.cpu().numpy(), scales)
     z = torch.empty_like(d)
-    C.run_ex(C.SOFTMAX, d, z, plan=ROW)
-    C.run_ex(C.SOFTMAX, d, d, plan=ROW)  # in == out
+    C.run_ex(C.SOFTMAX, d, z, plan=plan)
+    C.run_ex(C.SOFTMAX, d, d, plan=plan)  # in == out
     assert torch.equal(d, z)
 
 
