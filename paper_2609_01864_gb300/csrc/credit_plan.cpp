@@ -128,7 +128,13 @@ static long long team_room(const DeviceInfo &di, long long cols, int isz, int na
 // 300 KiB BF16 222 -> 194, int8 200 KiB BF16 234 -> 102; without gamma P = 2
 // stays behind P = 4 (140 KiB int8 84 against 71).  Few rows keep P = 1 up to
 // 96 KiB (100 x 48 KiB FP32 LayerNorm 9 against 12) unless they are FP8, whose
-// arithmetic is worth more CTAs (100 x 64 KiB LayerNorm 40 -> 24).
+// arithmetic is worth more CTAs (100 x 64 KiB LayerNorm 40 -> 24).  With fewer
+// than four rows per SM the two-pass paths find the rows in L2: softmax (150 x
+// 200 KiB FP32 16 against 19) and FP32 norms of up to 256 KiB (150 x 140 KiB
+// RMSNorm 13 against 17; 300 KiB 32 -> 29) stay there.  Softmax is split from
+// 128 KiB (1300 x 96 KiB BF16 60 against 64) to 256 KiB in FP32 (1300 x 300
+// KiB 156 against 173), 512 KiB in BF16 (600 x 420 KiB 136 -> 112, 960 KiB 279
+// against 319).
 static bool row_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, int tout,
                      credit_plan_t *p) {
     const int isz = dtype_size(tin), nab = op == CREDIT_OP_LAYERNORM ? 2 : op == CREDIT_OP_RMSNORM ? 1 : 0;
@@ -139,8 +145,13 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
     else if (sm8) limit = 24 << 10;
     else if (nab && !fp8 && grid) limit = 48 << 10;
     int P = bytes <= limit ? 1 : 0;
-    const bool split = op != CREDIT_OP_LOGSUMEXP && !sm8 && (!grid || (nab && fp8)) && bytes <= (grid ? 450 << 10 : 1 << 20);
-    if (split && (P == 0 || (nab && (tin == 2 || rows >= 4LL * di.sm_count)))) {
+    const bool many = rows >= 4LL * di.sm_count;
+    const bool pays = op == CREDIT_OP_SOFTMAX ? many && bytes > 128 << 10 && bytes <= (tin == 0 ? 256 << 10 : 512 << 10)
+                      : nab && tin == 0 && tout == 0 ? many || (bytes > 256 << 10 && bytes <= 512 << 10)
+                                                     : true;
+    const bool split = op != CREDIT_OP_LOGSUMEXP && !sm8 && pays && (!grid || (nab && fp8)) &&
+                       bytes <= (grid ? 450 << 10 : 1 << 20);
+    if (split && (P == 0 || (nab && (tin == 2 || many)))) {
         int q = nab || P ? 1 : 4;
         while (q <= 16 && team_room(di, cols, isz, nab, q) < 3) q *= 2;
         if (q <= 16 && (q > 1 || P)) P = q;
