@@ -381,7 +381,12 @@ typedef struct {
  *       G = 1 keeps rows of up to 96 KiB per array that fit in shared memory
  *       between the two looks.  Any alignment (fastest where a, dy and dx
  *       start at the same offset from a 16-byte boundary).
- * fill_share and retain must be 0.  Asynchronous on `stream`; the statuses
+ *   CLUSTER with retain = CREDIT_RETAIN_ROW (threads and ring_chunks 0; the
+ *       logits ops and softmax from its output)  rows split over the CTAs of a
+ *       cluster, which hold several rows at a time, one per team of threads.
+ *       Any alignment at which a and dy start at the same offset from a
+ *       16-byte boundary; otherwise CREDIT_ERR_UNSUPPORTED.
+ * fill_share and (but for that plan) retain must be 0.  Asynchronous on `stream`; the statuses
  * of credit_run_ex.
  */
 credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *plan, cudaStream_t stream);
@@ -395,7 +400,9 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
  * a and dy, and gamma for the norms) fit, else the split two-pass path.  The
  * logits and pair ops, whose per-row merges grow with the cluster size, are
  * staged only for P <= 4 with slices of at most 64 KiB per array (pair ops at
- * P = 4: the largest that fit).  source = 3 (built-in rule).
+ * P = 4: the largest that fit); wide logits rows, and narrower BF16 ones from
+ * four rows per SM on, take the smallest cluster that holds two rows at a
+ * time (CREDIT_RETAIN_ROW).  source = 3 (built-in rule).
  */
 credit_status credit_plan_bwd(int32_t op, int64_t rows, int64_t cols, credit_dtype dtype, credit_plan_t *out);
 

@@ -68,6 +68,7 @@ struct BwdKernels {
     const void *staged;
     const void *fused[2], *stats[2], *apply[2];  // [rows off the 16-byte grid]
     const void *team[2][2];  // [rows on the 16-byte grid][gamma in shared memory]
+    const void *team_cl;     // rows split over a cluster (null: op without)
 };
 
 namespace {
@@ -1017,11 +1018,16 @@ __global__ void __launch_bounds__(kBwdThreads, kPair<OP> && !OFF ? 4 : 1) k_bwd_
 // start and end on it), edge elements one per thread, loaded one row ahead
 // with the row's saved statistics.  Shared memory makes a further look at the
 // row cheap, so the logits ops take the maximum first and the pair ops the
-// means first (plain sums; no online states and no Chan merges).
+// means first (plain sums; no online states and no Chan merges).  CL: a row is
+// split over the P CTAs of a cluster (the CLUSTER path), whose teams of one
+// number exchange their partials as in k_row_team.
 constexpr int kBwdTeamRed = 4 * 96;  // floats of reduction scratch per team: 4 arrays of 3 sums x 32 warps
 
-__host__ __device__ constexpr int bwd_team_ctrl(int T, int teams) {
-    return kTeamMaxTeams * kTeamMaxStages * 8 + (T > 32 ? teams * kBwdTeamRed * 4 : 0);
+constexpr int kBwdXchBytes = 544;      // cluster exchange of one team: 512 bytes of slots, two mbarriers
+
+__host__ __device__ constexpr int bwd_team_ctrl(int T, int teams, bool cluster) {
+    return kTeamMaxTeams * kTeamMaxStages * 8 + (T > 32 ? teams * kBwdTeamRed * 4 : 0) +
+           (cluster ? teams * kBwdXchBytes : 0);
 }
 
 // K sums over a team's T threads (the tree of team_reduce).
@@ -1042,42 +1048,51 @@ __device__ __forceinline__ void team_sums(float (&v)[K], float *red, int bar, in
 
 __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 
-template <int OP, int DT, bool GRID, bool AFF>
+template <int OP, int DT, bool GRID, bool AFF, bool CL>
 __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V, NP = V / 4;
     const int T = blockDim.x, t = threadIdx.x, team = threadIdx.y, teams = blockDim.y, S = p.nbuf;
-    const int N = static_cast<int>(p.cols), gmax = N / V;
+    const int N = static_cast<int>(p.cols);
+    const int P = CL ? static_cast<int>(cluster_nctarank()) : 1, c = CL ? static_cast<int>(cluster_ctarank()) : 0;
+    const int lp = CL ? 31 - __clz(P) : 0;   // P is a power of two
+    const int gmax = (N / V + P - 1) >> lp;  // groups of a row's slice are at most this many
     uint64_t *full = reinterpret_cast<uint64_t *>(smem) + team * kTeamMaxStages;
     float *red = reinterpret_cast<float *>(smem + kTeamMaxTeams * kTeamMaxStages * 8) + (T > 32 ? team * kBwdTeamRed : 0);
+    // cluster exchange of the team: slots [row parity][16 sources][4 floats] and mbarriers [parity]
+    unsigned char *xch = smem + bwd_team_ctrl(T, teams, false) + team * kBwdXchBytes;
+    uint64_t *xbar = reinterpret_cast<uint64_t *>(xch + 512);
     const int np = affine_np<NP>(N);
-    float *gsm = reinterpret_cast<float *>(smem + bwd_team_ctrl(T, teams));
+    float *gsm = reinterpret_cast<float *>(smem + bwd_team_ctrl(T, teams, CL));
     const AffinePlanes gp{gsm, np};
     const uint32_t arr = gmax * 16u;  // bytes of one array's stage
     unsigned char *stages = reinterpret_cast<unsigned char *>(gsm + (AFF ? NP * np * 4 : 0)) +
                             static_cast<size_t>(team) * S * 2 * arr;
-    const long long stride = static_cast<long long>(gridDim.x) * teams;
-    const long long row_first = static_cast<long long>(blockIdx.x) * teams + team;
+    const long long stride = static_cast<long long>(gridDim.x >> lp) * teams;
+    const long long row_first = static_cast<long long>(blockIdx.x >> lp) * teams + team;
 
+    // a row's head, groups and tail, and the groups lo .. lo + n - 1 of this CTA's slice
     struct Geo {
-        int h0, G, t0;
+        int h0, G, t0, lo, n;
     };
     auto offset = [&](long long row) { return static_cast<size_t>(row * p.ld) * isz; };
     auto geo = [&](size_t off) {
-        if constexpr (GRID) return Geo{0, gmax, 0};
+        if constexpr (GRID) return Geo{0, gmax, 0, 0, gmax};
         Geo g;
         g.h0 = min(static_cast<int>((0u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.a) + off)) & 15u) / isz, N);
         g.G = (N - g.h0) / V;
         g.t0 = (N - g.h0) % V;
+        g.lo = CL ? g.G * c >> lp : 0;
+        g.n = CL ? (g.G * (c + 1) >> lp) - g.lo : g.G;
         return g;
     };
     auto issue = [&](long long row, int slot) {  // thread 0: both arrays' groups into a stage
         const size_t off = offset(row);
         const Geo g = geo(off);
-        if (!GRID && g.G == 0) return;
-        const uint32_t bytes = static_cast<uint32_t>(g.G) * 16u;
+        if (!GRID && g.n == 0) return;
+        const uint32_t bytes = static_cast<uint32_t>(g.n) * 16u;
         unsigned char *da = stages + static_cast<uint32_t>(slot) * 2u * arr;
-        const size_t src = off + g.h0 * isz;
+        const size_t src = off + g.h0 * isz + g.lo * 16;
         mbar_arrive_expect_tx(&full[slot], 2 * bytes);
         for (uint32_t o = 0; o < bytes; o += kMaxChunkBytes) {
             const uint32_t n = min(bytes - o, static_cast<uint32_t>(kMaxChunkBytes));
@@ -1087,17 +1102,42 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
     };
     auto edge_index = [&](const Geo &g) -> int {
         if constexpr (GRID) return -1;
-        return t < g.h0 ? t : (T - 1 - t < g.t0 ? g.h0 + g.G * V + (T - 1 - t) : -1);
+        if ((!CL || c == 0) && t < g.h0) return t;
+        return (!CL || c == P - 1) && T - 1 - t < g.t0 ? g.h0 + g.G * V + (T - 1 - t) : -1;
     };
 
     if (t == 0) {
         for (int k = 0; k < S; ++k) mbar_init(&full[k], 1);
+        if constexpr (CL) {
+            for (int k = 0; k < 2; ++k) mbar_init(&xbar[k], 1);
+        }
         fence_mbar_init();
         for (int k = 0; k < S; ++k)
             if (row_first + k * stride < p.rows) issue(row_first + k * stride, k);
     }
     if constexpr (AFF) planes_fill<NP>(gsm, np, p.gamma, 1.0f, N, team * T + t, T * teams);
     __syncthreads();
+    if constexpr (CL) {  // every peer's exchange barriers exist before the first push
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
+    // Push all-gather of four floats per CTA (the protocol of k_row_team's): lane q < P gets CTA q's.
+    uint32_t it = 0;  // exchanges (rows) done
+    auto exchange = [&](float4 v) -> float4 {
+        const uint32_t par = it & 1u;
+        float4 *slots = reinterpret_cast<float4 *>(xch) + par * 16;
+        uint64_t *bar = &xbar[par];
+        if (t < P) {
+            fence_release_smem_cluster();
+            st_async_v4f32(mapa_shared(smem_addr(slots + c), t), v, mapa_shared(smem_addr(bar), t));
+        }
+        if (t == 0) mbar_arrive_expect_tx(bar, static_cast<uint32_t>(P) * 16u);
+        mbar_wait_bounded_cluster(bar, (it >> 1) & 1u, p.err);
+        ++it;
+        const int q = t & 31;
+        return q < P ? slots[q] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    };
+    const bool mine = (t & 31) < P;  // lanes that hold a CTA's partial
 
     BwdRow<OP> Rn;  // the next row's saved statistics and edge elements
     float ean = 0.0f, edn = 0.0f;
@@ -1126,11 +1166,11 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         const float ea = ean, ed = edn;
         if (row + stride < p.rows) fetch_next(row + stride);
         const unsigned char *da = stages + static_cast<uint32_t>(slot) * 2u * arr, *dd = da + arr;
-        if (GRID || g.G > 0) mbar_wait_bounded(&full[slot], lap & 1u, p.err);
+        if (GRID || g.n > 0) mbar_wait_bounded(&full[slot], lap & 1u, p.err);
 
         auto each = [&](auto &&fn) {  // this thread's groups
 #pragma unroll 1
-            for (int gi = t; gi < g.G; gi += T) {
+            for (int gi = t; gi < g.n; gi += T) {
                 float fa[V], fd[V];
                 decode_group<DT>(*reinterpret_cast<const uint4 *>(da + 16 * gi), fa, 1.0f);
                 decode_group<DT>(*reinterpret_cast<const uint4 *>(dd + 16 * gi), fd, 1.0f);
@@ -1192,11 +1232,12 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                 team_sums(v1, red + (odd ? 96 : 0), team, T);
                 v[0] = v1[0];
             }
+            if constexpr (CL) v[0] = warp_sum(exchange(make_float4(v[0], 0.0f, 0.0f, 0.0f)).x);
             kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0] * R.rstd, N);
         } else if constexpr (kLogits<OP>) {
             GroupMax<DT, false> gm;
 #pragma unroll 1
-            for (int gi = t; gi < g.G; gi += T) gm.add(*reinterpret_cast<const uint4 *>(da + 16 * gi));
+            for (int gi = t; gi < g.n; gi += T) gm.add(*reinterpret_cast<const uint4 *>(da + 16 * gi));
             float m = gm.value();
             if (edge) m = fmaxf(m, ea);
             m = team_reduce<true>(m, red, team, T);
@@ -1219,11 +1260,18 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                 v[1] = OP == BOP_SMLOGITS ? fmaf(e, ed, v[1]) : v[1] + ed;
             }
             team_sums(v, red + 96, team, T);
+            if constexpr (CL) {  // every slice's sums about the row's maximum
+                const float4 x = exchange(make_float4(m, v[0], v[1], 0.0f));
+                m = warp_max_redux(mine ? x.x : -INFINITY);
+                const float r = !mine ? 0.0f : x.x == -INFINITY ? 1.0f : ex2_ftz((x.x - m) * kLog2e);
+                v[0] = warp_sum(mine ? x.y * r : 0.0f);
+                v[1] = warp_sum(mine ? (OP == BOP_SMLOGITS ? x.z * r : x.z) : 0.0f);
+            }
             kc = logit_coeffs<OP>(m, v[0], v[1]);
         } else {
             // means about the row's first group's first elements, then the centred sums
-            const float ka = GRID || g.G > 0 ? decode_one<DT>(da, 1.0f) : decode_one<DT>(p.a + off, 1.0f);
-            const float kd = GRID || g.G > 0 ? decode_one<DT>(dd, 1.0f) : decode_one<DT>(p.dy + off, 1.0f);
+            const float ka = GRID || g.n > 0 ? decode_one<DT>(da, 1.0f) : decode_one<DT>(p.a + off, 1.0f);
+            const float kd = GRID || g.n > 0 ? decode_one<DT>(dd, 1.0f) : decode_one<DT>(p.dy + off, 1.0f);
             float2 u0 = f2(0.0f), u1 = f2(0.0f);
             each([&](int, float (&fa)[V], float (&fd)[V]) {
 #pragma unroll
@@ -1287,8 +1335,9 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
 
         // ---- gradients
         const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
-        unsigned char *xr = p.dx + off + g.h0 * isz;
-        unsigned char *xr2 = kPair<OP> ? p.dx2 + off + g.h0 * isz : nullptr;
+        const size_t at = off + g.h0 * isz + g.lo * 16;
+        unsigned char *xr = p.dx + at;
+        unsigned char *xr2 = kPair<OP> ? p.dx2 + at : nullptr;
         const bool vec = GRID || ((reinterpret_cast<uintptr_t>(xr) | reinterpret_cast<uintptr_t>(xr2)) & 15u) == 0;
         each([&](int gi, float (&fa)[V], float (&fd)[V]) {
             float y[V];
@@ -1346,10 +1395,21 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
             ++lap;
         }
     }
+    if constexpr (CL) {  // no CTA leaves while a peer may still push into it
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
 }
 
 
 #ifdef CREDIT_BWD_DT
+template <int OP>
+const void *cluster_team_of() {
+    if constexpr (kLogits<OP> || OP == BOP_SOFTMAX)
+        return reinterpret_cast<const void *>(&k_bwd_team<OP, CREDIT_BWD_DT, false, false, true>);
+    else
+        return nullptr;
+}
 template <int OP>
 BwdKernels bwd_kernels_of() {
     constexpr int DT = CREDIT_BWD_DT;
@@ -1361,10 +1421,11 @@ BwdKernels bwd_kernels_of() {
              reinterpret_cast<const void *>(&k_bwd_tp_stats<OP, DT, true>)},
             {reinterpret_cast<const void *>(&k_bwd_tp_apply<OP, DT, false>),
              reinterpret_cast<const void *>(&k_bwd_tp_apply<OP, DT, true>)},
-            {{reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, false>),
-              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, A>)},
-             {reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, false>),
-              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, A>)}}};
+            {{reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, false, false>),
+              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, false, A, false>)},
+             {reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, false, false>),
+              reinterpret_cast<const void *>(&k_bwd_team<OP, DT, true, A, false>)}},
+            cluster_team_of<OP>()};
 }
 #endif
 }  // namespace
@@ -1457,27 +1518,77 @@ bool bwd_config(const DeviceInfo &di, long long N, int isz, int P, int req_nbuf,
     return false;
 }
 
+// CTAs per row of a cluster team plan (CLUSTER, retain ROW), 0 where the other
+// paths are the better ones.  Logits ops: the smallest cluster of which a CTA
+// holds two rows' slices at a time.  Measured (GB300, 1200 rows, staged or
+// two-pass -> this): BF16 on the 16-byte grid 96 KiB per array 87 -> 71 us,
+// 140 KiB 150 -> 120, 200 KiB 182 -> 152, 300 KiB 276 -> 271, 420 KiB 382 ->
+// 339; FP32 300 KiB 273 -> 236, 420 KiB 377 -> 295, off the grid 96 KiB 71 ->
+// 65, 200 KiB 187 -> 135, 420 KiB 383 -> 298; 100 FP32 rows of 300 KiB 60 ->
+// 30.  Behind stay FP32 rows on the grid within the staged kernel's four
+// slices of 64 KiB (1300 x 200 KiB 147 against 153), BF16 rows a little wider
+// than those (1300 x 264 KiB 276 against 290), few rows on the grid (150 x 100
+// KiB BF16 15 against 18) or narrow off it (100 x 96 KiB FP32 9 against 14),
+// and single slices (1000 KiB 883 against 1201).  Softmax from its output, off
+// the grid only (on it the staged kernel is at the copy rate), not few rows
+// (300 x 100 KiB FP32 19 against 24): clusters of 16 while four slices fit,
+// 140 KiB BF16 122 -> 101, 256 KiB 226 -> 187, 420 KiB 370 -> 347; three
+// slices lose (600 KiB 530 against 677), smaller clusters gain less.  The
+// norms, with gamma beside the slices, and the pair ops lose or stay level at
+// most widths.
+int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, bool grid) {
+    const long long bytes = cols * dtype_size(dtype);
+    const bool logits = op == BOP_SMLOGITS || op == BOP_XENT, many = rows >= 4LL * di.sm_count;
+    bool pays = false;
+    if (logits && grid)
+        pays = bytes > (dtype == CREDIT_F32 ? 256 << 10 : 300 << 10) ||
+               (dtype == CREDIT_BF16 && many && bytes > 64 << 10 && bytes <= 256 << 10);
+    else if (logits)
+        pays = bytes > (many ? 64 << 10 : 128 << 10);
+    else if (op == BOP_SOFTMAX && !grid)
+        pays = many && bytes > kBwdTeamMaxBytes;
+    if (!pays) return 0;
+    const long long room = di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16, true);
+    for (int P = logits ? 2 : 16; P <= kMaxCluster; P *= 2)
+        if (room / ((bytes / 16 + P - 1) / P * 32) >= (logits ? 2 : 4)) return P;
+    return 0;
+}
+
+credit_plan_t bwd_row_plan(int P) {
+    credit_plan_t p;
+    std::memset(&p, 0, sizeof(p));
+    p.path = CREDIT_PATH_CLUSTER;
+    p.cluster_size = p.ctas_per_row = P;
+    p.retain = CREDIT_RETAIN_ROW;
+    p.source = 3;
+    return p;
+}
+
 // Geometry of k_bwd_team; false where it does not apply: the arrays' rows at
 // different phases of the 16-byte grid, or no room for a row of both arrays.
 struct BwdTeamCfg {
-    int threads, teams, stages, grid;
+    int P, threads, teams, stages, grid;
     bool grid_rows, gamma_smem;
     long long smem;
 };
-bool bwd_team_config(const DeviceInfo &di, const credit_bwd_args *a, BwdTeamCfg *out) {
-    const int isz = dtype_size(a->dtype), V = 16 / isz;
-    const uintptr_t ua = reinterpret_cast<uintptr_t>(a->a), ud = reinterpret_cast<uintptr_t>(a->dy);
-    if (((ua ^ ud) & 15u) != 0 || ua % isz != 0) return false;
-    const long long groups = a->cols / V, per_sm = (a->rows + di.sm_count - 1) / di.sm_count;
-    if (a->cols * isz > kBwdTeamMaxBytes) return false;
-    const bool norm = a->op == BOP_LN || a->op == BOP_RMS;
+bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, int P, BwdTeamCfg *out) {
+    const int isz = dtype_size(dtype), V = 16 / isz;
+    const bool norm = op == BOP_LN || op == BOP_RMS;
+    if (P < 1 || P > kMaxCluster || (P & (P - 1)) != 0 || (P > 1 && cols / V < 32 * P)) return false;
+    if (P == 1 && cols * isz > kBwdTeamMaxBytes) return false;
+    const long long groups = (cols / V + P - 1) / P, walkers = di.sm_count / P;
+    const long long per_sm = (rows + walkers - 1) / walkers;
     auto warps = [](long long n) { return n < 1 ? 32 : (n + 31) / 32 * 32; };
     BwdTeamCfg r;
+    r.P = P;
+    const long long NP = V / 4, aff = norm ? NP * (((cols + 3) / 4 + NP - 1) / NP + 1) * 16 : 0;
     // teams of four 16-byte groups of each array per thread, as many as have a row and fit shared memory with
     // one stage; where that leaves threads over, each team takes more of them
     const long long T4 = warps((groups + kTeamGroups - 1) / kTeamGroups);
     long long teams = kTeamMaxThreads / (T4 < kTeamMaxThreads ? T4 : kTeamMaxThreads);
-    const long long fit = groups > 0 ? (di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16)) / (groups * 32) : teams;
+    const long long most_ctrl = bwd_team_ctrl(kTeamMaxThreads / 16, 16, P > 1);
+    const long long fit =
+        groups > 0 ? (di.smem_optin - most_ctrl) / (groups * 32) : teams;
     if (teams > fit) teams = fit;
     if (teams > per_sm) teams = per_sm;
     if (teams < 1) return false;
@@ -1488,18 +1599,24 @@ bool bwd_team_config(const DeviceInfo &di, const credit_bwd_args *a, BwdTeamCfg 
     }
     r.teams = static_cast<int>(teams);
     r.threads = static_cast<int>(T);
-    const long long np4 = (a->cols + 3) / 4, NP = V / 4, aff = norm ? NP * ((np4 + NP - 1) / NP + 1) * 16 : 0;
-    const long long stage = groups * 32 * r.teams, room = di.smem_optin - bwd_team_ctrl(r.threads, r.teams);
+    const long long stage = groups * 32 * r.teams, ctrl = bwd_team_ctrl(r.threads, r.teams, P > 1);
+    const long long room = di.smem_optin - ctrl;
     r.gamma_smem = norm && aff + stage <= room && per_sm > r.teams;
     const long long left = room - (r.gamma_smem ? aff : 0);
     r.stages = stage == 0 || 2 * stage <= left ? 2 : stage <= left ? 1 : 0;
     if (r.stages == 0) return false;
-    r.smem = bwd_team_ctrl(r.threads, r.teams) + (r.gamma_smem ? aff : 0) + r.stages * stage;
-    const long long ctas = (a->rows + r.teams - 1) / r.teams;
-    r.grid = static_cast<int>(ctas < di.sm_count ? ctas : di.sm_count);
-    r.grid_rows = a->cols % V == 0 && rows_aligned(a);
+    r.smem = ctrl + (r.gamma_smem ? aff : 0) + r.stages * stage;
+    const long long ctas = (rows + r.teams - 1) / r.teams;
+    r.grid = static_cast<int>(ctas < walkers ? ctas : walkers);
+    r.grid_rows = false;
     *out = r;
     return true;
+}
+
+// a and dy at one phase of the 16-byte grid (k_bwd_team cuts both arrays alike)
+bool phases_agree(const credit_bwd_args *a) {
+    const uintptr_t ua = reinterpret_cast<uintptr_t>(a->a), ud = reinterpret_cast<uintptr_t>(a->dy);
+    return ((ua ^ ud) & 15u) == 0 && ua % dtype_size(a->dtype) == 0;
 }
 
 // gamma is staged in shared memory by the norms when present and 16-byte aligned.
@@ -1508,7 +1625,8 @@ bool stage_gamma(int op, const float *gamma) {
 }
 
 credit_status check_bwd_plan(int dev, const credit_bwd_args *a, const credit_plan_t *p, BwdCfg *cfg, int *maxc) {
-    if (p->fill_share != 0.0f || p->retain != 0) return CREDIT_ERR_UNSUPPORTED;
+    const bool team_rows = p->retain == CREDIT_RETAIN_ROW && p->path == CREDIT_PATH_CLUSTER;
+    if (p->fill_share != 0.0f || (p->retain != 0 && !team_rows)) return CREDIT_ERR_UNSUPPORTED;
     if (p->threads != 0 && p->threads != kBwdThreads) return CREDIT_ERR_UNSUPPORTED;
     BwdKernels k;
     if (!bwd_kernels(a->op, a->dtype, &k)) return CREDIT_ERR_UNSUPPORTED;
@@ -1519,6 +1637,17 @@ credit_status check_bwd_plan(int dev, const credit_bwd_args *a, const credit_pla
     if (p->path != CREDIT_PATH_ONE_CTA && p->path != CREDIT_PATH_CLUSTER) return CREDIT_ERR_UNSUPPORTED;
     const int P = p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size;
     if (p->path == CREDIT_PATH_CLUSTER && P < 2) return CREDIT_ERR_UNSUPPORTED;
+    if (team_rows) {
+        BwdTeamCfg tc;
+        const DeviceInfo *di = device_info(dev);
+        if (p->threads != 0 || p->ring_chunks != 0 || k.team_cl == nullptr || di == nullptr || !phases_agree(a) ||
+            !bwd_team_config(*di, a->op, a->dtype, a->rows, a->cols, P, &tc))
+            return CREDIT_ERR_UNSUPPORTED;
+        const credit_status st = prepare_staged_kernel(dev, k.team_cl);
+        if (st != CREDIT_OK) return st;
+        *maxc = staged_max_clusters(dev, k.team_cl, P, tc.threads * tc.teams, tc.smem, false);
+        return *maxc > 0 ? CREDIT_OK : CREDIT_ERR_UNSUPPORTED;
+    }
     if (p->ring_chunks < 0 || p->ring_chunks > 2) return CREDIT_ERR_UNSUPPORTED;
     if (!rows_aligned(a)) return CREDIT_ERR_UNSUPPORTED;
     const DeviceInfo *di = device_info(dev);
@@ -1533,7 +1662,7 @@ credit_status check_bwd_plan(int dev, const credit_bwd_args *a, const credit_pla
 
 inline bool kPairOp(int op) { return op == BOP_WVAR || op == BOP_PEARSON; }
 
-credit_status plan_bwd_for(int dev, int op, long long cols, int dtype, credit_plan_t *out) {
+credit_status plan_bwd_for(int dev, int op, long long rows, long long cols, int dtype, credit_plan_t *out) {
     std::memset(out, 0, sizeof(*out));
     out->source = 3;
     out->threads = kBwdThreads;
@@ -1542,6 +1671,10 @@ credit_status plan_bwd_for(int dev, int op, long long cols, int dtype, credit_pl
     if (di != nullptr && cols * isz > bwd_team_bytes(op)) {
         BwdKernels k;
         if (!bwd_kernels(op, dtype, &k)) return CREDIT_ERR_UNSUPPORTED;
+        if (const int P = bwd_row_cluster(*di, op, dtype, rows, cols, true)) {
+            *out = bwd_row_plan(P);
+            return CREDIT_OK;
+        }
         const bool merge_heavy = op == BOP_SMLOGITS || op == BOP_XENT || kPairOp(op);
         if (merge_heavy) {
             // the logits ops carry a per-row merge of (max, sum, dot) states, the pair ops Chan merges of
@@ -1623,7 +1756,7 @@ credit_status credit_plan_bwd(int32_t op, int64_t rows, int64_t cols, credit_dty
     int dev = 0;
     const credit_status st = ensure_init(&dev, nullptr);
     if (st != CREDIT_OK) return st;
-    return plan_bwd_for(dev, op, cols, dtype, out);
+    return plan_bwd_for(dev, op, rows, cols, dtype, out);
 }
 
 credit_status credit_bwd_plan_check(const credit_bwd_args *args, const credit_plan_t *plan) {
@@ -1647,8 +1780,15 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
     if (plan) {
         chosen = *plan;
     } else {
-        if ((st = plan_bwd_for(dev, args->op, args->cols, args->dtype, &chosen)) != CREDIT_OK) return st;
-        if (chosen.path != CREDIT_PATH_TWO_PASS && !rows_aligned(args)) {  // staged paths need aligned rows
+        if ((st = plan_bwd_for(dev, args->op, args->rows, args->cols, args->dtype, &chosen)) != CREDIT_OK) return st;
+        if (!rows_aligned(args) && phases_agree(args)) {
+            if (const int P = bwd_row_cluster(*device_info(dev), args->op, args->dtype, args->rows, args->cols, false))
+                chosen = bwd_row_plan(P);
+        }
+        if (chosen.path != CREDIT_PATH_TWO_PASS && !rows_aligned(args) &&
+            (chosen.retain != CREDIT_RETAIN_ROW || !phases_agree(args))) {  // staged paths need aligned rows
+            chosen.retain = 0;
+            chosen.threads = kBwdThreads;
             chosen.path = CREDIT_PATH_TWO_PASS;
             chosen.cluster_size = 1;
             long long g = args->cols * dtype_size(args->dtype) / (256LL << 10);
@@ -1667,6 +1807,25 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
     const long long rows = args->rows;
     cudaError_t e;
 
+    // k_bwd_team: one CTA per row, or (tP > 1) rows split over clusters
+    const int tP = chosen.retain == CREDIT_RETAIN_ROW ? chosen.cluster_size
+                   : chosen.path == CREDIT_PATH_TWO_PASS && chosen.ctas_per_row == 1 ? 1 : 0;
+    BwdTeamCfg tc;
+    if (tP > 0 && phases_agree(args) &&
+        bwd_team_config(*device_info(dev), args->op, args->dtype, rows, args->cols, tP, &tc)) {
+        const bool grid_rows = rows_aligned(args) && args->cols % (16 / dtype_size(args->dtype)) == 0;
+        const void *fn = tP > 1 ? k.team_cl : k.team[grid_rows][tc.gamma_smem];
+        if ((st = prepare_staged_kernel(dev, fn)) != CREDIT_OK) return st;
+        const int grid = tP > 1 && tc.grid > maxc ? maxc : tc.grid;  // every cluster resident
+        BwdArgs r = base;
+        r.nbuf = tc.stages;
+        void *kargs[] = {&r};
+        e = launch_kernel(fn, dim3(static_cast<unsigned>(grid * tP)), dim3(tc.threads, tc.teams),
+                          static_cast<size_t>(tc.smem), tP, stream, kargs);
+        if (e != cudaSuccess) return cuda_st(e);
+        g_launch_count.fetch_add(1);
+        return CREDIT_OK;
+    }
     if (chosen.path != CREDIT_PATH_TWO_PASS) {
         const long long ncl = rows < maxc ? rows : maxc;
         BwdArgs r = base;
@@ -1683,18 +1842,6 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
         return CREDIT_OK;
     }
     const int G = chosen.ctas_per_row;
-    BwdTeamCfg tc;
-    if (G == 1 && bwd_team_config(*device_info(dev), args, &tc)) {
-        const void *fn = k.team[tc.grid_rows][tc.gamma_smem];
-        if ((st = prepare_staged_kernel(dev, fn)) != CREDIT_OK) return st;
-        BwdArgs r = base;
-        r.nbuf = tc.stages;
-        void *kargs[] = {&r};
-        e = launch_kernel(fn, dim3(tc.grid), dim3(tc.threads, tc.teams), static_cast<size_t>(tc.smem), 1, stream, kargs);
-        if (e != cudaSuccess) return cuda_st(e);
-        g_launch_count.fetch_add(1);
-        return CREDIT_OK;
-    }
     const int off = !rows_aligned(args);
     const size_t rec = (args->op == BOP_SMLOGITS || args->op == BOP_XENT) ? 4
                        : (args->op == BOP_WVAR || args->op == BOP_PEARSON) ? 8 : 2;  // floats per partial

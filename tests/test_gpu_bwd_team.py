@@ -95,3 +95,33 @@ def test_in_place(op):
     C.run_bwd(op, ga, gd, out, **kw)
     C.run_bwd(op, ga, gd, gd, **kw)
     assert torch.equal(out, gd)
+
+
+# rows split over clusters: several rows at a time per CTA, one CTA per row's slice up to 16
+@pytest.mark.parametrize("op", [C.SOFTMAX_BWD, C.SOFTMAX_LOGITS_BWD, C.XENT_BWD])
+@pytest.mark.parametrize("dtype", [C.F32, C.BF16])
+@pytest.mark.parametrize("P,rows,kb,extra", [(2, 5, 70, 1), (2, 700, 64, 0), (4, 320, 96, 3), (16, 130, 64, -1),
+                                             (16, 7, 900, 5), (8, 1, 200, 0)])
+def test_cluster_rows(op, dtype, P, rows, kb, extra):
+    plan = C.make_plan(C.PATH_CLUSTER, P, retain=C.RETAIN_ROW, threads=0)
+    cols = kb * 1024 // (4 if dtype == C.F32 else 2) + extra
+    check(op, dtype, rows, cols, plan, off=(1, 1, 2) if extra else (0, 0, 0), seed=rows)
+
+
+@pytest.mark.parametrize("op", [C.SOFTMAX_BWD, C.SOFTMAX_LOGITS_BWD, C.XENT_BWD])
+def test_cluster_rows_chosen(op):
+    for dtype in (C.F32, C.BF16):
+        cols = 150 * 1024 // (4 if dtype == C.F32 else 2) + 1
+        check(op, dtype, 640, cols, None, seed=1)
+        check(op, dtype, 6, cols, None, off=(1, 2, 1), seed=2)  # unlike phases: another path
+
+
+def test_cluster_rows_refused():
+    x = torch.zeros(4, 40000, device="cuda")
+    m = torch.zeros(4, device="cuda")
+    plan = C.make_plan(C.PATH_CLUSTER, 4, retain=C.RETAIN_ROW, threads=0)
+    n0 = C.launch_count()
+    assert C.run_bwd_status(C.RMSNORM_BWD, x, x, x, plan=plan, rstd=m) == C.ERR_UNSUPPORTED
+    odd = torch.zeros(4 * 40000 + 1, device="cuda")[1:].view(4, 40000)
+    assert C.run_bwd_status(C.XENT_BWD, x, odd, x, plan=plan) == C.ERR_UNSUPPORTED
+    assert C.launch_count() == n0
