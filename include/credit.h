@@ -419,8 +419,11 @@ credit_status credit_bwd_plan_check(const credit_bwd_args *args, const credit_pl
  * rows of one width share the cluster in one work item, the w CTAs of a row
  * exchanging partials over DSMEM (w = 1: the one-CTA path, w = P: the cluster
  * path).  Rows beyond the capacity at w = P stream twice within the cluster.
- * Info: narrow_items counts the items of width 1, wide_items those of width
- * > 1, huge_items the streamed rows.  The project's addition; the paper runs
+ * Batches whose rows all fit a cluster's shared memory may instead run with
+ * every row over 1, 2, 4, ... 256 warps (threads = 512; an item is then a row,
+ * clusters those of all its launches, one per cluster size).
+ * Info: narrow_items counts the items of one CTA, wide_items those of several,
+ * huge_items the streamed rows.  The project's addition; the paper runs
  * one shape per launch.
  */
 typedef struct {
@@ -437,7 +440,8 @@ typedef struct {
 } credit_ragged_info_t;
 /* Build the work list, autotune (tune != 0: cluster size 4/8/16 x staging
  * capacity (48 KiB to 208 KiB) x threads (128, 256) x vector width (1 or 2
- * groups), each timed on this batch -- this launches the kernel
+ * groups), and rows over warps with 2 to 16 of a CTA's warps per row,
+ * each timed on this batch -- this launches the kernel
  * and writes out_base), and capture the chosen launch in a CUDA graph.
  * Allocates the device work list; in_base / out_base must stay valid while
  * the handle is used.  BF16 and FP32 only (FP8 rows would need scales). */
