@@ -191,6 +191,25 @@ static bool quant_plan(const DeviceInfo &di, int device, long long rows, long lo
     return true;
 }
 
+// Staged cluster plans whose rows lie off the 16-byte grid, where int8 codes
+// are stored byte by byte from the writer warps and LayerNorm's gamma / beta
+// are read element by element: the two-pass path is ahead (300 rows, this <-
+// the plan): 280001 FP32 int8 128 us <- 196, 600001 BF16 int8 166 <- 346,
+// 400001 FP32 LayerNorm 286 <- 872, 400001 FP8 LayerNorm (70 rows) 127 <- 249.
+// RMSNorm and softmax, with one or no such array, stay (1500 x 280001 FP32 787
+// against 892, 611 against 805).
+static void off_grid_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, credit_plan_t *p) {
+    const int isz = dtype_size(tin);
+    if (p->path != CREDIT_PATH_CLUSTER || p->retain == CREDIT_RETAIN_ROW || cols * isz % 16 == 0 ||
+        (op != CREDIT_OP_LAYERNORM && op != CREDIT_OP_QUANT_INT8))
+        return;
+    std::memset(p, 0, sizeof(*p));
+    p->source = 3;
+    p->path = CREDIT_PATH_TWO_PASS;
+    p->cluster_size = 1;
+    p->ctas_per_row = two_pass_split(di.sm_count, rows, cols, isz);
+}
+
 void heuristic_plan(const DeviceInfo &di, int device, int op, long long rows, long long cols, int tin, int tout,
                     credit_plan_t *p) {
     if (row_plan(di, op, rows, cols, tin, tout, p)) return;
@@ -268,6 +287,7 @@ credit_status credit_plan_ex(credit_op op, int64_t rows, int64_t cols, credit_dt
     if (!(cache && row_plan(*di, op, rows, cols, in_dtype, tout, out)) &&
         (q8 || !model_plan(*di, dev, op, rows, cols, in_dtype, tout, out)))
         heuristic_plan(*di, dev, op, rows, cols, in_dtype, tout, out);
+    if (cache) off_grid_plan(*di, op, rows, cols, in_dtype, out);
     if (cache) {
         std::lock_guard<std::mutex> lk(g_plan_mu);
         if (g_cache_gen == gen) {

@@ -525,6 +525,16 @@ __device__ __forceinline__ uint4 ld_global_v4_hint(const void *p, uint64_t polic
                  : "l"(p), "l"(policy));
     return v;
 }
+// 4-byte load into the first word, with an L2 cache policy (HINT) or without.
+template <bool HINT>
+__device__ __forceinline__ uint4 ld_global_u32_hint(const void *p, uint64_t policy) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if constexpr (HINT)
+        asm volatile("ld.global.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v.x) : "l"(p), "l"(policy));
+    else
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(v.x) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void st_global_v4_hint(void *p, const uint4 &v, uint64_t policy) {
     asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(v.x), "r"(v.y),
                  "r"(v.z), "r"(v.w), "l"(policy)

@@ -149,48 +149,6 @@ __device__ __forceinline__ void affine_pair(const AffineRow<NP> &r, const Affine
     }
 }
 
-// V floats from i0 on of an array of N in global memory (L1 / L2; a null array
-// is all dflt), the same way: no vector that reaches outside it is read (such a group loads its
-// elements one by one).
-template <int V>
-__device__ __forceinline__ void ldg_shift(const float *p, long long i0, long long N, float dflt, float (&v)[V]) {
-    if (p == nullptr) {
-#pragma unroll
-        for (int k = 0; k < V; ++k) v[k] = dflt;
-        return;
-    }
-    const int q = static_cast<int>(((reinterpret_cast<uintptr_t>(p) >> 2) + static_cast<uintptr_t>(i0)) & 3);
-    const float4 *b = reinterpret_cast<const float4 *>(p + i0 - q);
-    if (q == 0) {
-#pragma unroll
-        for (int k = 0; k < V / 4; ++k) {
-            const float4 x = __ldg(b + k);
-            v[4 * k] = x.x;
-            v[4 * k + 1] = x.y;
-            v[4 * k + 2] = x.z;
-            v[4 * k + 3] = x.w;
-        }
-    } else if (i0 >= q && i0 - q + V + 4 <= N) {
-        float f[V + 4];
-#pragma unroll
-        for (int k = 0; k < V / 4 + 1; ++k) {
-            const float4 x = __ldg(b + k);
-            f[4 * k] = x.x;
-            f[4 * k + 1] = x.y;
-            f[4 * k + 2] = x.z;
-            f[4 * k + 3] = x.w;
-        }
-        const bool q1 = (q & 1) != 0, q2 = (q & 2) != 0;
-#pragma unroll
-        for (int k = 0; k < V + 2; ++k) f[k] = q1 ? f[k + 1] : f[k];
-#pragma unroll
-        for (int k = 0; k < V; ++k) v[k] = q2 ? f[k + 2] : f[k];
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; ++k) v[k] = __ldg(p + i0 + k);
-    }
-}
-
 // All-reduce over the T threads of a team (T > 32: through red, one float per
 // warp, and named barrier `bar`).  Every warp merges the warps' values with
 // the same shuffle tree, so every thread returns the same value.
@@ -203,32 +161,6 @@ __device__ __forceinline__ float team_reduce(float v, float *red, int bar, int T
     named_bar_sync(bar, T);
     const float t = lane < nw ? red[lane] : (MAX ? -INFINITY : 0.0f);
     return MAX ? warp_max_redux(t) : warp_sum(t);
-}
-
-// Store V outputs packed in words: 16- / 8- / 4-byte stores (vec), else one
-// store per element.
-template <int DT, int V>
-__device__ __forceinline__ void store_words(unsigned char *p, const uint32_t (&w)[V * Fmt<DT>::size / 4], bool vec) {
-    constexpr int bytes = V * Fmt<DT>::size;
-    if (vec) {
-        if constexpr (bytes >= 16) {
-#pragma unroll
-            for (int k = 0; k < bytes / 16; ++k)
-                *reinterpret_cast<uint4 *>(p + 16 * k) = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
-        } else if constexpr (bytes == 8) {
-            *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
-        } else {
-            *reinterpret_cast<uint32_t *>(p) = w[0];
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; ++k) {
-            if constexpr (Fmt<DT>::size == 4) reinterpret_cast<uint32_t *>(p)[k] = w[k];
-            else if constexpr (Fmt<DT>::size == 2)
-                reinterpret_cast<uint16_t *>(p)[k] = static_cast<uint16_t>(w[k / 2] >> (16 * (k & 1)));
-            else p[k] = static_cast<unsigned char>(w[k / 4] >> (8 * (k & 3)));
-        }
-    }
 }
 
 // Elements hv .. hv + SV - 1 of one 16-byte group (E4M3 groups are worked on in two halves of 8).

@@ -223,6 +223,75 @@ __device__ __forceinline__ void load_affine(const float *p, long long i0, bool v
     }
 }
 
+// V floats from i0 on of an array of N in global memory (L1 / L2; a null array
+// is all dflt), as
+// aligned vectors shifted by their phase: no vector that reaches outside it is read (such a group loads its
+// elements one by one).
+template <int V>
+__device__ __forceinline__ void ldg_shift(const float *p, long long i0, long long N, float dflt, float (&v)[V]) {
+    if (p == nullptr) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) v[k] = dflt;
+        return;
+    }
+    const int q = static_cast<int>(((reinterpret_cast<uintptr_t>(p) >> 2) + static_cast<uintptr_t>(i0)) & 3);
+    const float4 *b = reinterpret_cast<const float4 *>(p + i0 - q);
+    if (q == 0) {
+#pragma unroll
+        for (int k = 0; k < V / 4; ++k) {
+            const float4 x = __ldg(b + k);
+            v[4 * k] = x.x;
+            v[4 * k + 1] = x.y;
+            v[4 * k + 2] = x.z;
+            v[4 * k + 3] = x.w;
+        }
+    } else if (i0 >= q && i0 - q + V + 4 <= N) {
+        float f[V + 4];
+#pragma unroll
+        for (int k = 0; k < V / 4 + 1; ++k) {
+            const float4 x = __ldg(b + k);
+            f[4 * k] = x.x;
+            f[4 * k + 1] = x.y;
+            f[4 * k + 2] = x.z;
+            f[4 * k + 3] = x.w;
+        }
+        const bool q1 = (q & 1) != 0, q2 = (q & 2) != 0;
+#pragma unroll
+        for (int k = 0; k < V + 2; ++k) f[k] = q1 ? f[k + 1] : f[k];
+#pragma unroll
+        for (int k = 0; k < V; ++k) v[k] = q2 ? f[k + 2] : f[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; ++k) v[k] = __ldg(p + i0 + k);
+    }
+}
+
+// Store V outputs packed in words: 16- / 8- / 4-byte stores (vec), else one
+// store per element.
+template <int DT, int V>
+__device__ __forceinline__ void store_words(unsigned char *p, const uint32_t (&w)[V * Fmt<DT>::size / 4], bool vec) {
+    constexpr int bytes = V * Fmt<DT>::size;
+    if (vec) {
+        if constexpr (bytes >= 16) {
+#pragma unroll
+            for (int k = 0; k < bytes / 16; ++k)
+                *reinterpret_cast<uint4 *>(p + 16 * k) = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+        } else if constexpr (bytes == 8) {
+            *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
+        } else {
+            *reinterpret_cast<uint32_t *>(p) = w[0];
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            if constexpr (Fmt<DT>::size == 4) reinterpret_cast<uint32_t *>(p)[k] = w[k];
+            else if constexpr (Fmt<DT>::size == 2)
+                reinterpret_cast<uint16_t *>(p)[k] = static_cast<uint16_t>(w[k / 2] >> (16 * (k & 1)));
+            else p[k] = static_cast<unsigned char>(w[k / 4] >> (8 * (k & 3)));
+        }
+    }
+}
+
 // SV affine values from the shared-memory affine ring (p == nullptr: dflt).
 template <int SV>
 __device__ __forceinline__ void load_affine_smem(const float *p, int off, float dflt, float (&v)[SV]) {
@@ -1186,6 +1255,38 @@ __device__ __forceinline__ void sweep_global(const unsigned char *in_row, const 
     (void)c;
 }
 
+// The same, four elements per thread at a time: a warp's float4 loads of gamma
+// / beta then cover 512 contiguous bytes, where a 16-element group of FP8 per
+// thread spreads each over four times the cache lines.
+template <int TIN, int L2H, class F>
+__device__ __forceinline__ void sweep_quads(const unsigned char *in_row, const RowSlice &s, float in_sc,
+                                            F &&fn /* fn(long long elem_index, float(&)[4]) */) {
+    constexpr int V = Fmt<TIN>::V, isz = Fmt<TIN>::size, U = 8;
+    static_assert(isz == 1, "E4M3 rows");
+    const unsigned char *body = in_row + s.h0 * isz;
+    const uint64_t pol = sweep_policy<L2H>();
+    const long long q1 = s.g_hi * (V / 4);
+    for (long long q0 = s.g_lo * (V / 4) + threadIdx.x; q0 < q1; q0 += static_cast<long long>(U) * blockDim.x) {
+        uint4 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long q = q0 + static_cast<long long>(u) * blockDim.x;
+            if (q >= q1) continue;
+            w[u] = ld_global_u32_hint<L2H != 0>(body + q * 4, pol);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long q = q0 + static_cast<long long>(u) * blockDim.x;
+            if (q >= q1) continue;
+            float f[V], x[4];
+            decode_group<TIN>(w[u], f, in_sc);  // elements 4 and on are not used
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = f[k];
+            fn(s.h0 + q * 4, x);
+        }
+    }
+}
+
 // sweep_global on the raw 16-byte groups: fn(first element index, group).
 template <int TIN, int L2H = 0, class F>
 __device__ __forceinline__ void sweep_global_raw(const unsigned char *in_row, const RowSlice &s,
@@ -1234,6 +1335,35 @@ __device__ __forceinline__ float2 stats_sweep(const RowArgs &a, const unsigned c
     return block_reduce_stream<OP>(st, red, slice_count(s, Fmt<TIN>::V, P, c));
 }
 
+// A norm's sweep over rows whose gamma / beta lie off the 16-byte grid, which
+// they then do by another phase in every row: fn(first element, elements,
+// gamma, beta) with both read as shifted vectors, in groups of 16 bytes of the
+// row, for E4M3 of four elements.  Element by element they bound the passes:
+// (1500 rows of 700001 columns, before -> now) BF16 LayerNorm 2167 us -> 1339,
+// BF16 -> FP8 RMSNorm 2169 -> 1529, FP8 LayerNorm 6369 -> 2761 (4320 in groups
+// of 16).  On the grid the plain loop is ahead (1500 x 512K BF16 LayerNorm 888
+// against 1208 in fours).
+template <int OP, int TIN, int L2H, class F>
+__device__ __forceinline__ void sweep_norm_off(const RowArgs &a, const unsigned char *in_row, const RowSlice &s, int P,
+                                               int c, float in_sc, F &&fn) {
+    constexpr int V = Fmt<TIN>::V;
+    if constexpr (TIN == DT_E4M3) {
+        sweep_quads<TIN, L2H>(in_row, s, in_sc, [&](long long i0, const float(&f)[4]) {
+            float gg[4], bb[4] = {};
+            ldg_shift<4>(a.gamma, i0, a.cols, 1.0f, gg);
+            if constexpr (OP == OP_LN) ldg_shift<4>(a.beta, i0, a.cols, 0.0f, bb);
+            fn(i0, f, gg, bb);
+        });
+    } else {
+        sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
+            float gg[V], bb[V] = {};
+            ldg_shift<V>(a.gamma, i0, a.cols, 1.0f, gg);
+            if constexpr (OP == OP_LN) ldg_shift<V>(a.beta, i0, a.cols, 0.0f, bb);
+            fn(i0, f, gg, bb);
+        });
+    }
+}
+
 template <int OP, int TIN, int L2H = 0>
 __device__ __forceinline__ float amax_sweep(const RowArgs &a, const unsigned char *in_row, const RowSlice &s, int P,
                                             int c, float in_sc, const Stats &st, float *red) {
@@ -1241,13 +1371,20 @@ __device__ __forceinline__ float amax_sweep(const RowArgs &a, const unsigned cha
     const bool g_vec = a.gamma == nullptr || ((reinterpret_cast<uintptr_t>(a.gamma + s.h0) & 15u) == 0);
     const bool b_vec = a.beta == nullptr || ((reinterpret_cast<uintptr_t>(a.beta + s.h0) & 15u) == 0);
     float am = 0.0f;
-    sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
-        float gg[V], bb[V];
-        load_affine<V>(a.gamma, i0, g_vec, 1.0f, gg);
-        load_affine<V>(a.beta, i0, b_vec, 0.0f, bb);
+    if (g_vec && b_vec)
+        sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
+            float gg[V], bb[V];
+            load_affine<V>(a.gamma, i0, true, 1.0f, gg);
+            load_affine<V>(a.beta, i0, true, 0.0f, bb);
 #pragma unroll
-        for (int j = 0; j < V; ++j) am = fmaxf(am, fabsf(norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f)));
-    });
+            for (int j = 0; j < V; ++j) am = fmaxf(am, fabsf(norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f)));
+        });
+    else
+        sweep_norm_off<OP, TIN, L2H>(a, in_row, s, P, c, in_sc, [&](long long, const auto &f, const auto &gg, const auto &bb) {
+#pragma unroll
+            for (int j = 0; j < static_cast<int>(sizeof(gg) / 4); ++j)
+                am = fmaxf(am, fabsf(norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f)));
+        });
     sweep_edges<TIN>(in_row, s, P, c, in_sc, [&](long long i, float x) {
         const float gg = a.gamma ? a.gamma[i] : 1.0f, bb = (OP == OP_LN && a.beta) ? a.beta[i] : 0.0f;
         am = fmaxf(am, fabsf(norm_h<OP>(x, st, gg, bb)));
@@ -1263,8 +1400,6 @@ __device__ __forceinline__ void apply_sweep(const RowArgs &a, long long row, con
     unsigned char *out_row = a.out + row * a.ld_out * osz;
     constexpr int vec_bytes = (V * osz) < 16 ? (V * osz) : 16;
     const bool out_vec = ((reinterpret_cast<uintptr_t>(out_row) + s.h0 * osz) % vec_bytes) == 0;
-    const bool g_vec = a.gamma == nullptr || ((reinterpret_cast<uintptr_t>(a.gamma + s.h0) & 15u) == 0);
-    const bool b_vec = a.beta == nullptr || ((reinterpret_cast<uintptr_t>(a.beta + s.h0) & 15u) == 0);
     if constexpr (OP == OP_SOFTMAX && TIN == DT_E4M3 && TOUT == DT_E4M3) {
         // E4M3 codes in and out, from the raw input codes (softmax_e4m3_codes)
         const float M = st.a, a1 = fabsf(in_sc), c8 = log2f(448.0f);
@@ -1303,14 +1438,28 @@ __device__ __forceinline__ void apply_sweep(const RowArgs &a, long long row, con
         sweep_edges<TIN>(in_row, s, P, c, in_sc,
                          [&](long long i, float x) { store_one<TOUT>(out_row + i * osz, q8_code(x, st.a, st.b)); });
     } else {
-        sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
-            float gg[V], bb[V], y[V];
-            load_affine<V>(a.gamma, i0, g_vec, 1.0f, gg);
-            if constexpr (OP == OP_LN) load_affine<V>(a.beta, i0, b_vec, 0.0f, bb);
+        const bool g_vec = a.gamma == nullptr || ((reinterpret_cast<uintptr_t>(a.gamma + s.h0) & 15u) == 0);
+        const bool b_vec = a.beta == nullptr || ((reinterpret_cast<uintptr_t>(a.beta + s.h0) & 15u) == 0);
+        if (g_vec && b_vec) {
+            sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
+                float gg[V], bb[V], y[V];
+                load_affine<V>(a.gamma, i0, true, 1.0f, gg);
+                if constexpr (OP == OP_LN) load_affine<V>(a.beta, i0, true, 0.0f, bb);
 #pragma unroll
-            for (int j = 0; j < V; ++j) y[j] = norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f) * qmul;
-            store_group<TOUT, V>(out_row + i0 * osz, y, out_vec);
-        });
+                for (int j = 0; j < V; ++j) y[j] = norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f) * qmul;
+                store_group<TOUT, V>(out_row + i0 * osz, y, out_vec);
+            });
+        } else {
+            const bool quad_vec = ((reinterpret_cast<uintptr_t>(out_row) + s.h0 * osz) % (4 * osz)) == 0;
+            sweep_norm_off<OP, TIN, L2H>(
+                a, in_row, s, P, c, in_sc, [&](long long i0, const auto &f, const auto &gg, const auto &bb) {
+                    constexpr int W = TIN == DT_E4M3 ? 4 : V;
+                    float y[W];
+#pragma unroll
+                    for (int j = 0; j < W; ++j) y[j] = norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f) * qmul;
+                    store_group<TOUT, W>(out_row + i0 * osz, y, W == V ? out_vec : quad_vec);
+                });
+        }
         sweep_edges<TIN>(in_row, s, P, c, in_sc, [&](long long i, float x) {
             const float gg = a.gamma ? a.gamma[i] : 1.0f, bb = (OP == OP_LN && a.beta) ? a.beta[i] : 0.0f;
             store_one<TOUT>(out_row + i * osz, norm_h<OP>(x, st, gg, bb) * qmul);
