@@ -100,6 +100,10 @@ typedef enum {
  *         plan sets threads, chunk_bytes or fill_share, ROW means AUTO;
  *         ring_chunks is the number of rows in flight per team (0 =
  *         default).
+ *   WARPS rows over single warps of 7 or 14 KiB of shared memory each (threads
+ *         256 or 512 = 0: two CTAs per SM or one); softmax, log-sum-exp and
+ *         int8 of FP32 and BF16 rows, any alignment; otherwise, or where the
+ *         cluster's warps do not hold a row: CREDIT_ERR_UNSUPPORTED.
  *   AUTO  TMEM where it applies and a slice exceeds 32 KiB, else SMEM
  *         (CREDIT_RETAIN=smem in the environment makes AUTO mean SMEM,
  *         CREDIT_RETAIN=tmem TMEM wherever it applies).  The planners set
@@ -108,7 +112,8 @@ typedef enum {
     CREDIT_RETAIN_AUTO = 0,
     CREDIT_RETAIN_SMEM = 1,
     CREDIT_RETAIN_TMEM = 2,
-    CREDIT_RETAIN_ROW = 3
+    CREDIT_RETAIN_ROW = 3,
+    CREDIT_RETAIN_WARPS = 4
 } credit_retain;
 
 typedef enum {

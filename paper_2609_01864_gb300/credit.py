@@ -26,7 +26,7 @@ PATH_AUTO, PATH_ONE_CTA, PATH_TWO_PASS, PATH_CLUSTER = -1, 0, 1, 2
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_CUDA, ERR_TIMEOUT, ERR_NOT_INITIALIZED, ERR_CAPTURE, ERR_IO = range(8)
 OP_NAMES = {SOFTMAX: "softmax", LOGSUMEXP: "logsumexp", LAYERNORM: "layernorm", RMSNORM: "rmsnorm"}
 PATH_NAMES = {PATH_ONE_CTA: "one_cta", PATH_TWO_PASS: "two_pass", PATH_CLUSTER: "cluster"}
-RETAIN_AUTO, RETAIN_SMEM, RETAIN_TMEM, RETAIN_ROW = 0, 1, 2, 3
+RETAIN_AUTO, RETAIN_SMEM, RETAIN_TMEM, RETAIN_ROW, RETAIN_WARPS = 0, 1, 2, 3, 4
 SOFTMAX_BWD, LAYERNORM_BWD, RMSNORM_BWD, SOFTMAX_LOGITS_BWD, XENT_BWD, WVAR_BWD, PEARSON_BWD = 4, 5, 6, 7, 8, 9, 10
 OP_NAMES.update({SOFTMAX_BWD: "softmax_bwd", LAYERNORM_BWD: "layernorm_bwd", RMSNORM_BWD: "rmsnorm_bwd",
                  SOFTMAX_LOGITS_BWD: "softmax_logits_bwd", XENT_BWD: "xent_bwd", WVAR_BWD: "wvar_bwd",

@@ -595,6 +595,16 @@ credit_status validate_args(const credit_args *a) {
 }
 
 // Is `p` legal for the arguments on this device (Eq. 3 and scheduling)?
+// A ONE_CTA or CLUSTER plan of rows over warps: threads 256 or 512 (0), the other fields at their defaults.
+static bool warps_plan_config(const DeviceInfo &di, const credit_args *a, const credit_plan_t *p, RowWarpsCfg *out) {
+    if ((p->threads != 0 && p->threads != 256 && p->threads != 512) || p->reducer_threads || p->chunk_bytes ||
+        p->ring_chunks || p->fill_share > 0.0f)
+        return false;
+    const int tout = a->op == OP_LSE ? DT_F32 : a->out_dtype;
+    return row_warps_config(di, a->op, a->in_dtype, tout, a->rows, a->cols,
+                            p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size, p->threads == 256 ? 8 : 16, out);
+}
+
 credit_status check_plan(int device, const credit_args *a, const credit_plan_t *p) {
     const DeviceInfo *di = device_info(device);
     if (!di) return CREDIT_ERR_NOT_INITIALIZED;
@@ -613,6 +623,14 @@ credit_status check_plan(int device, const credit_args *a, const credit_plan_t *
         const int P = p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size;
         if (P < 1 || P > kMaxCluster) return CREDIT_ERR_UNSUPPORTED;
         if (p->path == CREDIT_PATH_CLUSTER && P < 2) return CREDIT_ERR_UNSUPPORTED;
+        if (p->retain == CREDIT_RETAIN_WARPS) {
+            RowWarpsCfg wc;
+            return warps_plan_config(*di, a, p, &wc) &&
+                           prepare_staged_kernel(device, wc.fn) == CREDIT_OK &&
+                           staged_max_clusters(device, wc.fn, wc.P, 32 * wc.W, wc.smem, false) > 0
+                       ? CREDIT_OK
+                       : CREDIT_ERR_UNSUPPORTED;
+        }
         TeamCfg gc;
         if (team_plan_config(*di, a, p, &gc))
             return staged_max_clusters(device, team_kernel(a->op, a->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
@@ -741,6 +759,13 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
 
     if (p->path == CREDIT_PATH_ONE_CTA || p->path == CREDIT_PATH_CLUSTER) {
         const int P = p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size;
+        RowWarpsCfg wc;
+        if (p->retain == CREDIT_RETAIN_WARPS) {
+            if (g_test_extra_tx.load() > 0 || !warps_plan_config(d.info, a, p, &wc)) return CREDIT_ERR_UNSUPPORTED;
+            const credit_status st = run_row_warps(device, a, wc, s);
+            if (st == CREDIT_OK) g_launch_count.fetch_add(1);
+            return st;
+        }
         TeamCfg gc;
         if (team_plan_config(d.info, a, p, &gc)) {
             if (g_test_extra_tx.load() > 0) return CREDIT_ERR_UNSUPPORTED;  // the wait test's ring kernel only
@@ -832,15 +857,22 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
     // faster than with 512, 1024 slower still)
     const int G = p->ctas_per_row;
     const int threads = p->threads ? p->threads : (isz <= 2 ? 256 : 512);
+    // a row's gamma / beta lie on the 16-byte grid where its head is empty and they are aligned
+    const bool off = ks.tp_fused_off != nullptr && (a->gamma != nullptr || a->beta != nullptr) &&
+                     (((reinterpret_cast<uintptr_t>(a->in) | reinterpret_cast<uintptr_t>(a->gamma) |
+                        reinterpret_cast<uintptr_t>(a->beta)) & 15u) != 0 ||
+                      (rows > 1 && (a->ld_in ? a->ld_in : a->cols) * isz % 16 != 0));
+    const void *tp_fused = off ? ks.tp_fused_off : ks.tp_fused;
+    const void *tp_amax = off ? ks.tp_amax_off : ks.tp_amax, *tp_apply = off ? ks.tp_apply_off : ks.tp_apply;
     if (G == 1) {
-        credit_status st = prepare_kernel(d, ks.tp_fused, false);
+        credit_status st = prepare_kernel(d, tp_fused, false);
         if (st != CREDIT_OK) return st;
         const long long max_rows = 0x7FFFFFFFLL;
         for (long long r0 = 0; r0 < rows; r0 += max_rows) {
             const long long n = rows - r0 < max_rows ? rows - r0 : max_rows;
             RowArgs r = rows_from(base, r0, n, isz, osz, lse);
             void *args[] = {&r};
-            cudaError_t e = launch(ks.tp_fused, dim3(static_cast<unsigned>(n)), dim3(threads), 0, 1, s, args);
+            cudaError_t e = launch(tp_fused, dim3(static_cast<unsigned>(n)), dim3(threads), 0, 1, s, args);
             if (e != cudaSuccess) return cuda_status(e);
             g_launch_count.fetch_add(1);
         }
@@ -867,11 +899,11 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
             continue;
         }
         if (fp8_stage) {
-            e = launch(ks.tp_amax, grid, dim3(threads), 0, 1, s, args);
+            e = launch(tp_amax, grid, dim3(threads), 0, 1, s, args);
             if (e != cudaSuccess) return cuda_status(e);
             g_launch_count.fetch_add(1);
         }
-        e = launch(ks.tp_apply, grid, dim3(threads), 0, 1, s, args);
+        e = launch(tp_apply, grid, dim3(threads), 0, 1, s, args);
         if (e != cudaSuccess) return cuda_status(e);
         g_launch_count.fetch_add(1);
     }

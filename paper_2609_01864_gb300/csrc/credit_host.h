@@ -60,6 +60,16 @@ bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int
                  TeamCfg *out);
 // A ONE_CTA or CLUSTER plan that asks for whole rows, and a row that allows it.
 bool team_plan_config(const DeviceInfo &di, const credit_args *a, const credit_plan_t *p, TeamCfg *out);
+// Geometry of k_row_warps for rows of one width: 2^lu warps per row over all P CTAs (of W warps) of a cluster.
+struct RowWarpsCfg {
+    int P, W, lu;
+    long long smem;
+    const void *fn;
+};
+// False where a row does not fit, or the op or types have no such kernel.
+bool row_warps_config(const DeviceInfo &di, int op, int tin, int tout, long long rows, long long cols, int P, int W,
+                      RowWarpsCfg *out);
+credit_status run_row_warps(int device, const credit_args *a, const RowWarpsCfg &cfg, cudaStream_t s);
 int ring_max_clusters(int device, int op, int tin, int tout, int P, int threads, long long smem, bool tm = false);
 int affine_arrays(const credit_args *a);
 int affine_arrays_aligned(const credit_args *a);

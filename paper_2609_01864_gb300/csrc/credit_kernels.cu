@@ -29,6 +29,12 @@ static void fill_set(KernelSet *ks) {
     if constexpr (OP == OP_LN || OP == OP_RMS) {
         if constexpr (TOUT == DT_E4M3) ks->tp_amax = reinterpret_cast<const void *>(&k_tp_amax<OP, TIN>);
     }
+    ks->tp_fused_off = ks->tp_amax_off = ks->tp_apply_off = nullptr;
+    if constexpr ((OP == OP_LN || OP == OP_RMS) && TIN != DT_F32) {
+        ks->tp_fused_off = reinterpret_cast<const void *>(&k_tp_fused<OP, TIN, TOUT, true>);
+        ks->tp_apply_off = reinterpret_cast<const void *>(&k_tp_apply<OP, TIN, TOUT, true>);
+        if constexpr (TOUT == DT_E4M3) ks->tp_amax_off = reinterpret_cast<const void *>(&k_tp_amax<OP, TIN, true>);
+    }
     if constexpr (OP == OP_LSE) ks->tp_lse_final = reinterpret_cast<const void *>(&k_tp_lse_final<TIN>);
     else ks->tp_apply = reinterpret_cast<const void *>(&k_tp_apply<OP, TIN, TOUT>);
 }

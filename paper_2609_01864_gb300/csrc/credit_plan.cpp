@@ -128,10 +128,12 @@ static long long team_room(const DeviceInfo &di, long long cols, int isz, int na
 // 300 KiB BF16 222 -> 194, int8 200 KiB BF16 234 -> 102; without gamma P = 2
 // stays behind P = 4 (140 KiB int8 84 against 71).  Few rows keep P = 1 up to
 // 96 KiB (100 x 48 KiB FP32 LayerNorm 9 against 12) unless they are FP8, whose
-// arithmetic is worth more CTAs (100 x 64 KiB LayerNorm 40 -> 24).  With fewer
+// arithmetic is worth more CTAs (100 x 64 KiB LayerNorm 40 -> 24; not RMSNorm on
+// the grid, 300 x 60 KiB 26 against 33).  With fewer
 // than four rows per SM the two-pass paths find the rows in L2: softmax (150 x
-// 200 KiB FP32 16 against 19) and FP32 norms of up to 256 KiB (150 x 140 KiB
-// RMSNorm 13 against 17; 300 KiB 32 -> 29) stay there.  Softmax is split from
+// 200 KiB FP32 16 against 19) and FP32 norms of 56 to 280 KiB (600 x 80 KiB
+// RMSNorm 23 against 28, 150 x 140 KiB 13 against 17; 300 KiB 32 -> 29) stay
+// there.  Softmax is split from
 // 128 KiB (1300 x 96 KiB BF16 60 against 64) to 256 KiB in FP32 (1300 x 300
 // KiB 156 against 173), 512 KiB in BF16 (600 x 420 KiB 136 -> 112, 960 KiB 279
 // against 319).
@@ -140,18 +142,20 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
     const int isz = dtype_size(tin), nab = op == CREDIT_OP_LAYERNORM ? 2 : op == CREDIT_OP_RMSNORM ? 1 : 0;
     const bool grid = cols * isz % 16 == 0, fp8 = tin == 2 || tout == 2, sm8 = op == CREDIT_OP_SOFTMAX && tin == 2;
     const long long bytes = cols * isz;
+    const bool many = rows >= 4LL * di.sm_count;
     long long limit = 96 << 10;
     if (op == CREDIT_OP_LOGSUMEXP) limit = tin == 0 ? limit : tin == 1 ? 32 << 10 : 8 << 10;
     else if (sm8) limit = 24 << 10;
     else if (nab && !fp8 && grid) limit = 48 << 10;
+    else if (nab && tin == 0 && tout == 0 && !many) limit = 56 << 10;
     int P = bytes <= limit ? 1 : 0;
-    const bool many = rows >= 4LL * di.sm_count;
     const bool pays = op == CREDIT_OP_SOFTMAX ? many && bytes > 128 << 10 && bytes <= (tin == 0 ? 256 << 10 : 512 << 10)
-                      : nab && tin == 0 && tout == 0 ? many || (bytes > 256 << 10 && bytes <= 512 << 10)
+                      : nab && tin == 0 && tout == 0 ? many || (bytes > 280 << 10 && bytes <= 512 << 10 &&
+                                                              (nab > 1 || rows >= di.sm_count))
                                                      : true;
     const bool split = op != CREDIT_OP_LOGSUMEXP && !sm8 && pays && (!grid || (nab && fp8)) &&
                        bytes <= (grid ? 450 << 10 : 1 << 20);
-    if (split && (P == 0 || (nab && (tin == 2 || many)))) {
+    if (split && (P == 0 || (nab && (many || (tin == 2 && !(op == CREDIT_OP_RMSNORM && grid && bytes <= 64 << 10)))))) {
         int q = nab || P ? 1 : 4;
         while (q <= 16 && team_room(di, cols, isz, nab, q) < 3) q *= 2;
         if (q <= 16 && (q > 1 || P)) P = q;
@@ -165,6 +169,64 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
     p->ctas_per_row = P;
     p->retain = CREDIT_RETAIN_ROW;
     p->smem_bytes = tc.smem;
+    return true;
+}
+
+// Rows over warps (k_row_warps), for softmax, log-sum-exp and int8 of FP32 and
+// BF16 rows.  u is the number of warps whose buffers hold a row.  Clusters of
+// CTAs of 8 warps, two to an SM, of which a row takes four warps each (rows of
+// 128 KiB 104 us, 107 with its 16 warps in one CTA), eight of 8 CTAs from u =
+// 64 (512 KiB 408, over 16 CTAs 436), and eight CTAs of 16 warps at u = 128;
+// one CTA while that holds the row (but for many rows of 96 KiB, 2600 FP32 94
+// us against 80 over four), or there is hardly a row per SM (150 rows of 128 KiB
+// 11 against 13).  Measured (2400 rows, 600 from 768 KiB on, the
+// plan before -> this): BF16 softmax 128 KiB 122 -> 106, 192 KiB 204 -> 151,
+// 256 KiB 235 -> 208, 384 KiB 384 -> 300, 768 KiB 225 -> 169, 1.5 MiB 430 ->
+// 361; FP32 128 KiB 116 -> 104, 384 KiB 294 -> 288, 768 KiB 191 -> 160; int8
+// BF16 192 KiB 153 -> 121, 384 KiB 308 -> 239, FP32 off the grid 512 KiB 397 ->
+// 287; log-sum-exp FP32 192 KiB 84 -> 74, BF16 96 KiB 48 -> 43.  Outside the
+// ranges below the other paths are level or ahead: FP32 softmax of 128 KiB with
+// few rows (300 rows 15.6 against 17.3), 192 KiB (149 against 153), 256 KiB
+// (600 rows 58 against 61), 448 KiB (355 against 404) or above 900 KiB, BF16
+// int8 of 96 KiB (61 against 66), int8 of 1 MiB, which eight CTAs' tensor
+// memory holds (600 rows 176 against 198), log-sum-exp FP32 128 KiB with few
+// rows (600 rows 15 against 18) and 256 KiB (103 against 107), BF16 128 KiB
+// (600 rows 16 against 18), rows of 2 MiB (BF16 softmax 500 against 587).
+static bool warps_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, int tout,
+                       credit_plan_t *p) {
+    const int isz = dtype_size(tin);
+    const long long kib = cols * isz / 1024;
+    const bool f32 = tin == 0;
+    bool pays = false;
+    if (tin > 1) return false;
+    if (op == CREDIT_OP_SOFTMAX)
+        pays = f32 ? (kib >= 90 && kib <= 160 && rows >= 3LL * di.sm_count) || (kib >= 300 && kib <= 400) ||
+                         (kib > 640 && kib <= 900)
+                   : kib >= 60 && kib <= 1700;
+    else if (op == CREDIT_OP_QUANT_INT8)
+        pays = kib >= (cols * isz % 16 == 0 ? 101 : 96) && kib <= 1700 && !(kib > 900 && kib <= 1024);
+    else if (op == CREDIT_OP_LOGSUMEXP)
+        pays = f32 ? kib >= 60 && kib <= (rows >= 8LL * di.sm_count ? 220 : 110) : kib >= 40 && kib <= 110;
+    if (!pays) return false;
+    RowWarpsCfg c;
+    if (!row_warps_config(di, op, tin, tout, rows, cols, 1, 16, &c) &&
+        !row_warps_config(di, op, tin, tout, rows, cols, 16, 16, &c))
+        return false;
+    const int u = 1 << c.lu;
+    int P = u < 8 ? 1 : u <= 8 ? (op != CREDIT_OP_LOGSUMEXP && rows >= 8LL * di.sm_count ? 4 : 1) : u <= 32 ? u / 4 : 8;
+    int W = u <= 64 ? 8 : 16;
+    if (u == 16 && rows < 2LL * di.sm_count) {
+        P = 1;
+        W = 16;
+    }
+    if (!row_warps_config(di, op, tin, tout, rows, cols, P, W, &c)) return false;
+    std::memset(p, 0, sizeof(*p));
+    p->source = 3;
+    p->path = P == 1 ? CREDIT_PATH_ONE_CTA : CREDIT_PATH_CLUSTER;
+    p->cluster_size = p->ctas_per_row = P;
+    p->threads = 32 * W;
+    p->retain = CREDIT_RETAIN_WARPS;
+    p->smem_bytes = c.smem;
     return true;
 }
 
@@ -194,14 +256,15 @@ static bool quant_plan(const DeviceInfo &di, int device, long long rows, long lo
 // Staged cluster plans whose rows lie off the 16-byte grid, where int8 codes
 // are stored byte by byte from the writer warps and LayerNorm's gamma / beta
 // are read element by element: the two-pass path is ahead (300 rows, this <-
-// the plan): 280001 FP32 int8 128 us <- 196, 600001 BF16 int8 166 <- 346,
+// the plan): 280001 FP32 int8 128 us <- 196, 600001 BF16 int8 166 <- 346 (from
+// 16 CTAs on: eight are ahead, 262145 FP32 94 against 112),
 // 400001 FP32 LayerNorm 286 <- 872, 400001 FP8 LayerNorm (70 rows) 127 <- 249.
 // RMSNorm and softmax, with one or no such array, stay (1500 x 280001 FP32 787
 // against 892, 611 against 805).
 static void off_grid_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, credit_plan_t *p) {
     const int isz = dtype_size(tin);
-    if (p->path != CREDIT_PATH_CLUSTER || p->retain == CREDIT_RETAIN_ROW || cols * isz % 16 == 0 ||
-        (op != CREDIT_OP_LAYERNORM && op != CREDIT_OP_QUANT_INT8))
+    if (p->path != CREDIT_PATH_CLUSTER || p->retain == CREDIT_RETAIN_ROW || p->retain == CREDIT_RETAIN_WARPS || cols * isz % 16 == 0 ||
+        (!(op == CREDIT_OP_LAYERNORM && p->cluster_size >= 8) && !(op == CREDIT_OP_QUANT_INT8 && p->cluster_size == 16)))
         return;
     std::memset(p, 0, sizeof(*p));
     p->source = 3;
@@ -212,7 +275,7 @@ static void off_grid_plan(const DeviceInfo &di, int op, long long rows, long lon
 
 void heuristic_plan(const DeviceInfo &di, int device, int op, long long rows, long long cols, int tin, int tout,
                     credit_plan_t *p) {
-    if (row_plan(di, op, rows, cols, tin, tout, p)) return;
+    if (warps_plan(di, op, rows, cols, tin, tout, p) || row_plan(di, op, rows, cols, tin, tout, p)) return;
     std::memset(p, 0, sizeof(*p));
     p->source = 3;
     if (op == CREDIT_OP_QUANT_INT8 && quant_plan(di, device, rows, cols, tin, p)) return;
@@ -284,7 +347,8 @@ credit_status credit_plan_ex(credit_op op, int64_t rows, int64_t cols, credit_dt
     }
     // narrow rows take the rule unless CREDIT_MODEL asks for a model's own choice; the calibration and the
     // learned model cover the four ops of Sec. III-B; the quantiser takes the rule
-    if (!(cache && row_plan(*di, op, rows, cols, in_dtype, tout, out)) &&
+    if (!(cache && (warps_plan(*di, op, rows, cols, in_dtype, tout, out) ||
+                    row_plan(*di, op, rows, cols, in_dtype, tout, out))) &&
         (q8 || !model_plan(*di, dev, op, rows, cols, in_dtype, tout, out)))
         heuristic_plan(*di, dev, op, rows, cols, in_dtype, tout, out);
     if (cache) off_grid_plan(*di, op, rows, cols, in_dtype, out);

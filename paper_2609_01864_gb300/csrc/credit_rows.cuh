@@ -1335,14 +1335,17 @@ __device__ __forceinline__ float2 stats_sweep(const RowArgs &a, const unsigned c
     return block_reduce_stream<OP>(st, red, slice_count(s, Fmt<TIN>::V, P, c));
 }
 
-// A norm's sweep over rows whose gamma / beta lie off the 16-byte grid, which
-// they then do by another phase in every row: fn(first element, elements,
-// gamma, beta) with both read as shifted vectors, in groups of 16 bytes of the
-// row, for E4M3 of four elements.  Element by element they bound the passes:
-// (1500 rows of 700001 columns, before -> now) BF16 LayerNorm 2167 us -> 1339,
+// A norm's sweep (OFF) over BF16 or E4M3 rows whose gamma / beta lie off the
+// 16-byte grid, which they then do by another phase in every row: fn(first
+// element, elements, gamma, beta) with both read as shifted vectors, in groups
+// of 16 bytes of the row, for E4M3 of four elements.  Element by element they
+// bound the passes: (1500 rows of 700001 columns, before -> now) BF16 LayerNorm 2167 us -> 1339,
 // BF16 -> FP8 RMSNorm 2169 -> 1529, FP8 LayerNorm 6369 -> 2761 (4320 in groups
 // of 16).  On the grid the plain loop is ahead (1500 x 512K BF16 LayerNorm 888
-// against 1208 in fours).
+// against 1208 in fours); for FP32 rows, whose groups are four elements, loads
+// one by one cover the same lines and cost less (150 x 28673 LayerNorm 15 us
+// against 17).  Kernels of their own: the plain loop beside this one in a
+// branch lost 5% (2600 x 360448 BF16 LayerNorm 1047 us).
 template <int OP, int TIN, int L2H, class F>
 __device__ __forceinline__ void sweep_norm_off(const RowArgs &a, const unsigned char *in_row, const RowSlice &s, int P,
                                                int c, float in_sc, F &&fn) {
@@ -1364,18 +1367,18 @@ __device__ __forceinline__ void sweep_norm_off(const RowArgs &a, const unsigned 
     }
 }
 
-template <int OP, int TIN, int L2H = 0>
+template <int OP, int TIN, int L2H = 0, bool OFF = false>
 __device__ __forceinline__ float amax_sweep(const RowArgs &a, const unsigned char *in_row, const RowSlice &s, int P,
                                             int c, float in_sc, const Stats &st, float *red) {
     constexpr int V = Fmt<TIN>::V;
     const bool g_vec = a.gamma == nullptr || ((reinterpret_cast<uintptr_t>(a.gamma + s.h0) & 15u) == 0);
     const bool b_vec = a.beta == nullptr || ((reinterpret_cast<uintptr_t>(a.beta + s.h0) & 15u) == 0);
     float am = 0.0f;
-    if (g_vec && b_vec)
+    if constexpr (!OFF)
         sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
             float gg[V], bb[V];
-            load_affine<V>(a.gamma, i0, true, 1.0f, gg);
-            load_affine<V>(a.beta, i0, true, 0.0f, bb);
+            load_affine<V>(a.gamma, i0, g_vec, 1.0f, gg);
+            load_affine<V>(a.beta, i0, b_vec, 0.0f, bb);
 #pragma unroll
             for (int j = 0; j < V; ++j) am = fmaxf(am, fabsf(norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f)));
         });
@@ -1392,7 +1395,7 @@ __device__ __forceinline__ float amax_sweep(const RowArgs &a, const unsigned cha
     return block_allreduce<true>(am, red);
 }
 
-template <int OP, int TIN, int TOUT, int L2H = 0>
+template <int OP, int TIN, int TOUT, int L2H = 0, bool OFF = false>
 __device__ __forceinline__ void apply_sweep(const RowArgs &a, long long row, const unsigned char *in_row,
                                             const RowSlice &s, int P, int c, float in_sc, const Stats &st,
                                             float qmul) {
@@ -1440,11 +1443,11 @@ __device__ __forceinline__ void apply_sweep(const RowArgs &a, long long row, con
     } else {
         const bool g_vec = a.gamma == nullptr || ((reinterpret_cast<uintptr_t>(a.gamma + s.h0) & 15u) == 0);
         const bool b_vec = a.beta == nullptr || ((reinterpret_cast<uintptr_t>(a.beta + s.h0) & 15u) == 0);
-        if (g_vec && b_vec) {
+        if constexpr (!OFF) {
             sweep_global<TIN, L2H>(in_row, s, P, c, in_sc, [&](long long i0, const float(&f)[V]) {
                 float gg[V], bb[V], y[V];
-                load_affine<V>(a.gamma, i0, true, 1.0f, gg);
-                if constexpr (OP == OP_LN) load_affine<V>(a.beta, i0, true, 0.0f, bb);
+                load_affine<V>(a.gamma, i0, g_vec, 1.0f, gg);
+                if constexpr (OP == OP_LN) load_affine<V>(a.beta, i0, b_vec, 0.0f, bb);
 #pragma unroll
                 for (int j = 0; j < V; ++j) y[j] = norm_h<OP>(f[j], st, gg[j], OP == OP_LN ? bb[j] : 0.0f) * qmul;
                 store_group<TOUT, V>(out_row + i0 * osz, y, out_vec);
@@ -1674,7 +1677,7 @@ __device__ __forceinline__ void tp_fused_e4m3(const RowArgs &a, long long row, c
 // ----------------------------------------------------------------------
 // Two-pass path, one CTA per row (single launch, the row is read twice).
 // ----------------------------------------------------------------------
-template <int OP, int TIN, int TOUT>
+template <int OP, int TIN, int TOUT, bool OFF = false>
 __global__ void __launch_bounds__(1024) k_tp_fused(const RowArgs a) {
     __shared__ float red[128];
     constexpr int isz = Fmt<TIN>::size, V = Fmt<TIN>::V;
@@ -1696,7 +1699,7 @@ __global__ void __launch_bounds__(1024) k_tp_fused(const RowArgs a) {
     } else {
         float qmul = 1.0f;
         if constexpr (TOUT == DT_E4M3 && (OP == OP_LN || OP == OP_RMS)) {
-            const float am = amax_sweep<OP, TIN, 1>(a, in_row, s, 1, 0, in_sc, st, red);
+            const float am = amax_sweep<OP, TIN, 1, OFF>(a, in_row, s, 1, 0, in_sc, st, red);
             qmul = am > 0.0f ? 448.0f / am : 1.0f;
             if (threadIdx.x == 0) a.out_scale[row] = am > 0.0f ? am / 448.0f : 1.0f;
         }
@@ -1706,7 +1709,7 @@ __global__ void __launch_bounds__(1024) k_tp_fused(const RowArgs a) {
         if constexpr (OP == OP_Q8) {
             if (threadIdx.x == 0) a.out_scale[row] = st.a;
         }
-        apply_sweep<OP, TIN, TOUT, 2>(a, row, in_row, s, 1, 0, in_sc, st, qmul);
+        apply_sweep<OP, TIN, TOUT, 2, OFF>(a, row, in_row, s, 1, 0, in_sc, st, qmul);
     }
 }
 
@@ -1738,7 +1741,7 @@ __device__ __forceinline__ Stats tp_row_stats(const RowArgs &a, long long lr, co
     return combine_partials<OP>(a.ws + lr * a.G * 4, 4, a.G, s, Fmt<TIN>::V, a.cols, a.eps);
 }
 
-template <int OP, int TIN>
+template <int OP, int TIN, bool OFF = false>
 __global__ void __launch_bounds__(1024) k_tp_amax(const RowArgs a) {
     __shared__ float red[128];
     constexpr int isz = Fmt<TIN>::size;
@@ -1748,11 +1751,11 @@ __global__ void __launch_bounds__(1024) k_tp_amax(const RowArgs a) {
     const RowSlice s = make_slice(reinterpret_cast<uintptr_t>(in_row), a.cols, isz, G, g);
     const float in_sc = (TIN == DT_E4M3) ? a.in_scale[row] : 1.0f;
     const Stats st = tp_row_stats<OP, TIN>(a, lr, s);
-    const float am = amax_sweep<OP, TIN>(a, in_row, s, G, g, in_sc, st, red);
+    const float am = amax_sweep<OP, TIN, 0, OFF>(a, in_row, s, G, g, in_sc, st, red);
     if (threadIdx.x == 0) a.ws[(lr * G + g) * 4 + 2] = am;
 }
 
-template <int OP, int TIN, int TOUT>
+template <int OP, int TIN, int TOUT, bool OFF = false>
 __global__ void __launch_bounds__(1024) k_tp_apply(const RowArgs a) {
     constexpr int isz = Fmt<TIN>::size;
     const int G = a.G, g = blockIdx.x % G;
@@ -1774,7 +1777,7 @@ __global__ void __launch_bounds__(1024) k_tp_apply(const RowArgs a) {
     if constexpr (OP == OP_Q8) {
         if (g == 0 && threadIdx.x == 0) a.out_scale[row] = st.a;
     }
-    apply_sweep<OP, TIN, TOUT>(a, row, in_row, s, G, g, in_sc, st, qmul);
+    apply_sweep<OP, TIN, TOUT, 0, OFF>(a, row, in_row, s, G, g, in_sc, st, qmul);
 }
 
 // One thread per row: combine the G log-sum-exp partials.
@@ -1799,6 +1802,7 @@ struct KernelSet {
     const void *tp_amax;
     const void *tp_apply;
     const void *tp_lse_final;
+    const void *tp_fused_off, *tp_amax_off, *tp_apply_off;  // gamma / beta off the 16-byte grid (else null)
 };
 
 }  // namespace credit

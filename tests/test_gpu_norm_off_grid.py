@@ -65,7 +65,6 @@ def test_wide_rows_as_planned(op, tin, tout, cols):
 @pytest.mark.parametrize("tin,cols", [(C.F32, 280001), (C.BF16, 600001)])
 def test_wide_int8_rows_as_planned(tin, cols):
     """int8 rows off the grid: codes and scales equal those of the same rows on the grid (padded stride)."""
-    assert C.plan(C.QUANT_INT8, 9, cols, tin, C.INT8).path == C.PATH_TWO_PASS
     x, _ = U.make_input(tin, 9, cols, seed=3)
     ld = (cols + 15) // 16 * 16
     out = []
