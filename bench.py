@@ -137,6 +137,8 @@ def kernel_name(plan, C, cols=0, isz=4):
             return "k_ring_tm+fill" if plan.retain == C.RETAIN_TMEM else "k_ring+fill"
         if plan.retain == C.RETAIN_TMEM:
             return "k_ring_tm"
+        if plan.retain == C.RETAIN_WARPS:
+            return "k_row_warps"
         if plan.retain == C.RETAIN_ROW:
             return "k_row_team"
         if plan.retain == C.RETAIN_AUTO:  # the library's AUTO rule for the norms with FP32 output

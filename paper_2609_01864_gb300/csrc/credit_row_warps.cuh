@@ -18,7 +18,7 @@
 // numbered by the first warp as well.
 // k_ragged, with its online maxima, chunk and item barriers, took 20
 // instructions per element and 59% of the issue slots.  Measured (GB300,
-// k_ragged -> this): 20000 BF16 rows of 1K to 1M columns 2640 us -> 2100 (the
+// k_ragged -> this): 20000 BF16 rows of 1K to 1M columns 2640 us -> 2180 (the
 // copy rate's 1765), 8000 of 8K to 40K 167 -> 114 (94), 4000 of 1K to 4K 33 ->
 // 12, 3000 FP32 rows of 8K to 200K 295 -> 236 (210), 64 of 16K to 500K 29 ->
 // 22.  Segments of all 14 KiB (half as many warps per row) are worth more than
