@@ -832,38 +832,47 @@ __device__ __forceinline__ void bwd_singles(const BwdSpan &s, F &&fn) {
     for (long long i = e_lo + threadIdx.x; i < e_hi; i += blockDim.x) fn(i);
 }
 
-// fn(first element, a, dy, gamma) on every group of a span.  OFF: rows off the
+// fn(byte offset in the arrays, a, dy, gamma) on every group of a span.  OFF: rows off the
 // 16-byte grid, whose gamma lies at any phase (ldg_shift) and whose two groups
 // of each array in flight repay the registers (1440 x 46161 FP32 LayerNorm dx
 // 220 us with two, 227 with one; on the grid the plain loop with one is 3%
 // ahead, its 32-36 registers leave room for four CTAs of 512 threads).
 template <int OP, int DT, bool OFF, class F>
 __device__ __forceinline__ void bwd_groups(const BwdArgs &p, long long row, const BwdSpan &s, F &&fn) {
-    constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V, U = OFF ? 2 : 1;
+    constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V, U = 2;
     if (!s.vec) return;
     const bool g_vec = p.gamma == nullptr || (reinterpret_cast<uintptr_t>(p.gamma) & 15u) == 0;
     const size_t off = static_cast<size_t>(row * p.ld + s.h0) * isz;
     const float *gam = kNorm<OP> ? p.gamma : nullptr;
-    for (long long k0 = s.lo + threadIdx.x; k0 < s.hi; k0 += U * blockDim.x) {
-        uint4 wa[U], wd[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const long long k = k0 + u * blockDim.x;
-            if (u == 0 || k < s.hi) {
-                wa[u] = ld_global_v4(p.a + off + 16 * k);
-                wd[u] = ld_global_v4(p.dy + off + 16 * k);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const long long k = k0 + u * blockDim.x;
-            if (u > 0 && k >= s.hi) continue;
+    if constexpr (!OFF) {
+        for (long long k = s.lo + threadIdx.x; k < s.hi; k += blockDim.x) {
             float fa[V], fd[V], fg[V];
-            decode_group<DT>(wa[u], fa, 1.0f);
-            decode_group<DT>(wd[u], fd, 1.0f);
-            if constexpr (OFF) ldg_shift<V>(gam, s.h0 + k * V, p.cols, 1.0f, fg);
-            else load_affine<V>(gam, k * V, g_vec, 1.0f, fg);
-            fn(s.h0 + k * V, fa, fd, fg);
+            decode_group<DT>(ld_global_v4(p.a + off + 16 * k), fa, 1.0f);
+            decode_group<DT>(ld_global_v4(p.dy + off + 16 * k), fd, 1.0f);
+            load_affine<V>(gam, k * V, g_vec, 1.0f, fg);
+            fn(off + 16 * k, fa, fd, fg);
+        }
+    } else {
+        for (long long k0 = s.lo + threadIdx.x; k0 < s.hi; k0 += U * blockDim.x) {
+            uint4 wa[U], wd[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const long long k = k0 + u * blockDim.x;
+                if (u == 0 || k < s.hi) {
+                    wa[u] = ld_global_v4(p.a + off + 16 * k);
+                    wd[u] = ld_global_v4(p.dy + off + 16 * k);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const long long k = k0 + u * blockDim.x;
+                if (u > 0 && k >= s.hi) continue;
+                float fa[V], fd[V], fg[V];
+                decode_group<DT>(wa[u], fa, 1.0f);
+                decode_group<DT>(wd[u], fd, 1.0f);
+                ldg_shift<V>(gam, s.h0 + k * V, p.cols, 1.0f, fg);
+                fn(off + 16 * k, fa, fd, fg);
+            }
         }
     }
 }
@@ -875,7 +884,7 @@ __device__ __forceinline__ BwdState<OP> bwd_sums(const BwdArgs &p, long long row
     const size_t off = static_cast<size_t>(row * p.ld) * isz;
     const float *gam = kNorm<OP> ? p.gamma : nullptr;
     BwdState<OP> st;
-    bwd_groups<OP, DT, OFF>(p, row, s, [&](long long, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
+    bwd_groups<OP, DT, OFF>(p, row, s, [&](size_t, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
         st.template add<V>(R, fa, fd, fg);
     });
     bwd_singles<OFF>(s, [&](long long i) {
@@ -891,18 +900,18 @@ __device__ __forceinline__ void bwd_apply(const BwdArgs &p, long long row, const
     constexpr int isz = Fmt<DT>::size, V = Fmt<DT>::V;
     const size_t off = static_cast<size_t>(row * p.ld) * isz;
     const float *gam = kNorm<OP> ? p.gamma : nullptr;
-    bwd_groups<OP, DT, OFF>(p, row, s, [&](long long i, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
+    bwd_groups<OP, DT, OFF>(p, row, s, [&](size_t at, const float (&fa)[V], const float (&fd)[V], const float (&fg)[V]) {
         float y[V];
         if constexpr (kPair<OP>) {
             float y2[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) R.dx_pair(fa[v], fd[v], kc, y[v], y2[v]);
-            store_group<DT, V>(p.dx + off + i * isz, y, true);
-            store_group<DT, V>(p.dx2 + off + i * isz, y2, true);
+            store_group<DT, V>(p.dx + at, y, true);
+            store_group<DT, V>(p.dx2 + at, y2, true);
         } else {
 #pragma unroll
             for (int v = 0; v < V; ++v) y[v] = R.dx(fa[v], fd[v], fg[v], kc);
-            store_group<DT, V>(p.dx + off + i * isz, y, true);
+            store_group<DT, V>(p.dx + at, y, true);
         }
     });
     bwd_singles<OFF>(s, [&](long long i) {
