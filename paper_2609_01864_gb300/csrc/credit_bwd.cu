@@ -1055,6 +1055,31 @@ __device__ __forceinline__ void team_sums(float (&v)[K], float *red, int bar, in
     for (int k = 0; k < K; ++k) v[k] = warp_sum(lane < nw ? red[32 * k + lane] : 0.0f);
 }
 
+// Does an element of the warp lie so far below the row's maximum that its exponential is no normal number?  d: the
+// smallest element of each lane less the maximum.  ex2.ftz gives 0 for those; such warps take exp_fast, which the
+// other backward paths use throughout (its range handling costs three instructions per element).  Looking for them
+// costs 2% (4096 x 131072 BF16 cross entropy 784 -> 798 us); exponentials raised by 2^24 for all elements, as in the
+// forward softmax, would cost less but round the exponents near 0 three times as coarsely.
+__device__ __forceinline__ bool reaches_subnormal(float d) {
+    return __any_sync(0xffffffffu, d * kLog2e < -126.0f) != 0;
+}
+
+// The lowest of the elements added, 0 if none is negative: as unsigned numbers negative floats are above the others
+// and ordered by magnitude, so one three-input integer maximum takes two words (half a floating-point minimum's
+// instructions for BF16 pairs).
+template <int DT>
+struct LowestBits {
+    uint32_t m = 0u;
+    __device__ __forceinline__ void add(const uint4 &w) {
+        if constexpr (DT == DT_F32) m = __vimax3_u32(__vimax3_u32(m, w.x, w.y), w.z, w.w);
+        else m = __vimax3_u16x2(__vimax3_u16x2(m, w.x, w.y), w.z, w.w);
+    }
+    __device__ __forceinline__ float value() const {
+        if constexpr (DT == DT_F32) return fminf(__uint_as_float(m), 0.0f);
+        else return fminf(fminf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u)), 0.0f);
+    }
+};
+
 __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 
 template <int OP, int DT, bool GRID, bool AFF, bool CL>
@@ -1213,6 +1238,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         };
 
         Coef kc;
+        float lo = 0.0f;  // logits: the smallest of this thread's elements and 0 (edges apart)
         if constexpr (!kLogits<OP> && !kPair<OP>) {
             float2 s0 = f2(0.0f), s1 = f2(0.0f);
             each([&](int gi, float (&fa)[V], float (&fd)[V]) {
@@ -1245,15 +1271,32 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
             kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0] * R.rstd, N);
         } else if constexpr (kLogits<OP>) {
             GroupMax<DT, false> gm;
+            LowestBits<DT> gl;
 #pragma unroll 1
-            for (int gi = t; gi < g.n; gi += T) gm.add(*reinterpret_cast<const uint4 *>(da + 16 * gi));
+            for (int gi = t; gi < g.n; gi += T) {
+                const uint4 x = *reinterpret_cast<const uint4 *>(da + 16 * gi);
+                gm.add(x);
+                gl.add(x);
+            }
+            lo = gl.value();
             float m = gm.value();
             if (edge) m = fmaxf(m, ea);
             m = team_reduce<true>(m, red, team, T);
             refill();
             const float mz = m == -INFINITY ? 0.0f : m;
             float2 sS = f2(0.0f), sT = f2(0.0f);
+            // a term below the normal numbers counts in T beside a large dy (in S it does not)
+            const bool low = OP == BOP_SMLOGITS && reaches_subnormal(lo - mz);
             each([&](int, float (&fa)[V], float (&fd)[V]) {
+                if (low) {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        const float e = exp_fast(fa[v] - mz);
+                        sS.x += e;
+                        sT.x = fmaf(e, fd[v], sT.x);
+                    }
+                    return;
+                }
 #pragma unroll
                 for (int v = 0; v < V; v += 2) {
                     const float2 x = __fmul2_rn(__fadd2_rn(make_float2(fa[v], fa[v + 1]), f2(-mz)), f2(kLog2e));
@@ -1264,7 +1307,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
             });
             float v[2] = {sS.x + sS.y, sT.x + sT.y};
             if (edge) {
-                const float e = ex2_ftz((ea - mz) * kLog2e);
+                const float e = exp_fast(ea - mz);
                 v[0] += e;
                 v[1] = OP == BOP_SMLOGITS ? fmaf(e, ed, v[1]) : v[1] + ed;
             }
@@ -1272,7 +1315,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
             if constexpr (CL) {  // every slice's sums about the row's maximum
                 const float4 x = exchange(make_float4(m, v[0], v[1], 0.0f));
                 m = warp_max_redux(mine ? x.x : -INFINITY);
-                const float r = !mine ? 0.0f : x.x == -INFINITY ? 1.0f : ex2_ftz((x.x - m) * kLog2e);
+                const float r = !mine ? 0.0f : x.x == -INFINITY ? 1.0f : exp_fast(x.x - m);
                 v[0] = warp_sum(mine ? x.y * r : 0.0f);
                 v[1] = warp_sum(mine ? (OP == BOP_SMLOGITS ? x.z * r : x.z) : 0.0f);
             }
@@ -1348,7 +1391,14 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         unsigned char *xr = p.dx + at;
         unsigned char *xr2 = kPair<OP> ? p.dx2 + at : nullptr;
         const bool vec = GRID || ((reinterpret_cast<uintptr_t>(xr) | reinterpret_cast<uintptr_t>(xr2)) & 15u) == 0;
-        each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+        const bool low = kLogits<OP> && reaches_subnormal(lo - kc.c0);
+        if (low) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+            float y[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) y[v] = kLogits<OP> ? R.dx(fa[v], fd[v], 1.0f, kc) : 0.0f;
+            store_group<DT, V>(xr + 16 * gi, y, vec);
+        });
+        if (!low) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
             float y[V];
             if constexpr (kPair<OP>) {
                 float y2[V];
