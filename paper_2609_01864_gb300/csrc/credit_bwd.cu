@@ -1251,13 +1251,14 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                         x = __fadd2_rn(x, f2(-R.mean));
                         s0 = __fadd2_rn(s0, d);
                     }
+                    if constexpr (kNorm<OP>) x = __fmul2_rn(x, f2(R.rstd));  // xh: in range whatever the row's scale
                     s1 = __ffma2_rn(x, d, s1);
                 }
             });
             float v[2] = {s1.x + s1.y, s0.x + s0.y};
             if (edge) {
                 const float d = ed * eg;
-                v[0] = fmaf(OP == BOP_LN ? ea - R.mean : ea, d, v[0]);
+                v[0] = fmaf((OP == BOP_LN ? ea - R.mean : ea) * R.rstd, d, v[0]);  // softmax: rstd 1
                 v[1] += d;
             }
             if constexpr (OP == BOP_LN) {
@@ -1268,7 +1269,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                 v[0] = v1[0];
             }
             if constexpr (CL) v[0] = warp_sum(exchange(make_float4(v[0], 0.0f, 0.0f, 0.0f)).x);
-            kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0] * R.rstd, N);
+            kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0], N);
         } else if constexpr (kLogits<OP>) {
             GroupMax<DT, false> gm;
             LowestBits<DT> gl;
@@ -1386,7 +1387,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         if constexpr (!kLogits<OP> && !kPair<OP>) refill();
 
         // ---- gradients
-        const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
+        const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
         const size_t at = off + g.h0 * isz + g.lo * 16;
         unsigned char *xr = p.dx + at;
         unsigned char *xr2 = kPair<OP> ? p.dx2 + at : nullptr;
@@ -1422,8 +1423,8 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                             r = __fmul2_rn(f2(R.w), __ffma2_rn(e, f2(kc.c1), make_float2(-d.x, -d.y)));
                         }
                     } else {
-                        const float2 xm = OP == BOP_LN ? __fadd2_rn(x, f2(-R.mean)) : x;
-                        r = __ffma2_rn(d, f2(R.rstd), __ffma2_rn(xm, f2(k1), f2(k0)));
+                        const float2 xh = __fmul2_rn(OP == BOP_LN ? __fadd2_rn(x, f2(-R.mean)) : x, f2(R.rstd));
+                        r = __ffma2_rn(d, f2(R.rstd), __ffma2_rn(xh, f2(k1), f2(k0)));
                     }
                     y[v] = r.x;
                     y[v + 1] = r.y;

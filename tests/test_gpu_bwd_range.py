@@ -6,6 +6,8 @@ import torch
 
 from paper_2609_01864_gb300 import credit as C
 
+import parity_util as U
+
 pytestmark = pytest.mark.gpu
 PLANS = {"planned": None, "one_cta": C.make_plan(C.PATH_TWO_PASS, ctas_per_row=1),
          "split": C.make_plan(C.PATH_TWO_PASS, ctas_per_row=3),
@@ -58,3 +60,25 @@ def test_logits_far_below_the_maximum(op, plan, cols):
     bound[3, big] += 2.0 ** -22
     err = np.abs(dx.cpu().double().numpy() - ref)
     assert np.isfinite(err).all() and (err <= bound).all(), (err / bound).max()
+
+
+@pytest.mark.parametrize("plan", ["planned", "one_cta", "split"])
+@pytest.mark.parametrize("op", [C.LAYERNORM_BWD, C.RMSNORM_BWD])
+@pytest.mark.parametrize("scale", [1e-25, 1e19, 1e23, 1e36])
+@pytest.mark.parametrize("cols", [4096, 4099])
+def test_norm_rows_of_any_scale(op, plan, scale, cols):
+    """Saved statistics of rows so small or large that rstd^2, or a sum of x g, leaves FP32 (the result does not)."""
+    rows = 9
+    _, dy, gamma, _, _ = U.bwd_inputs(op, C.F32, rows, cols, seed=3)
+    a = torch.randn(rows, cols, generator=torch.Generator().manual_seed(11), dtype=torch.float64).mul(scale).float()
+    a64 = a.double()
+    mean = a64.mean(1).float() if op == C.LAYERNORM_BWD else None
+    rstd = (1.0 / (a64.std(1, correction=0) if op == C.LAYERNORM_BWD else a64.square().mean(1).sqrt())).float()
+    kw = {k: v.cuda() for k, v in dict(gamma=gamma, mean=mean, rstd=rstd).items() if v is not None}
+    dx = torch.full((rows, cols), float("nan"), device="cuda")
+    C.run_bwd(op, a.cuda(), dy.cuda(), dx, plan=PLANS[plan], **kw)
+    torch.cuda.synchronize()
+    assert C.device_error() == C.OK
+    ref = U.bwd_reference(op, C.F32, a, dy, gamma, mean, rstd, rows, cols)
+    assert torch.isfinite(dx).all()
+    assert U.bwd_error(op, C.F32, U.to64(dx), ref, a, dy, gamma, mean, rstd, cols) <= 1.0
