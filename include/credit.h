@@ -25,6 +25,10 @@
  * Conventions shared by every entry point:
  *  - Device pointers are plain device addresses owned by the caller.  The
  *    library owns only a per-device workspace that credit_init() allocates.
+ *    Forward calls split over at most 2048 partial records (rows x
+ *    ctas_per_row) take a part of it per stream and per capture, and may
+ *    overlap calls on other streams; larger TWO_PASS plans and the backward
+ *    ops' share the rest, and must not overlap one another.
  *  - All work is enqueued asynchronously on `stream` (0 = legacy default
  *    stream).  The return value reports argument and launch errors; faults
  *    found on the device (a bounded wait that gave up) are reported later by

@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <utility>
 
 #include "../../include/credit.h"
 #include "credit_host.h"
@@ -33,6 +34,11 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kWorkspaceFloats = size_t(16) << 20;  // 64 MiB of two-pass partials
+// Beside it, a workspace of its own for each stream and each capture that runs split two-pass calls of up to 2048
+// partial records (all that two_pass_split asks for: fewer than 8 per SM), so that calls on several streams, and
+// replays of captured ones, do not meet in one.  2 x 512 of 32 KiB.
+constexpr size_t kSlotFloats = 2048 * 4;
+constexpr int kSlots = 512;
 
 struct DeviceState {
     std::mutex mu;
@@ -44,6 +50,9 @@ struct DeviceState {
     cudaEvent_t fork = nullptr, join = nullptr;
     std::map<const void *, bool> attr_done;
     std::map<std::tuple<const void *, int, int, long long>, int> clusters;  // max active clusters
+    std::map<std::pair<unsigned long long, unsigned long long>, int> slots;  // (stream, capture + 1 or 0) -> its number
+    int eager_slots = 0, captured_slots = 0;
+    unsigned long long slot_use[kSlots] = {}, slot_clock = 0;  // eager slots: last use
 };
 DeviceState g_dev[kMaxDevices];
 
@@ -440,6 +449,45 @@ float *device_workspace(int device, size_t *floats) {
     return g_dev[device].ws;
 }
 
+// The two-pass workspace of a stream, or of a stream's part of the capture it is in; null where `floats` is more than
+// it holds or there is none left.  Stream and capture numbers are never reused.  A captured call keeps its slot for
+// good, since its graph may run at any time; when all 512 of the others are taken, a new stream gets the one used
+// longest ago.
+static float *stream_workspace(DeviceState &d, cudaStream_t s, size_t floats) {
+    if (floats > kSlotFloats) return nullptr;
+    unsigned long long id = 0, capture = 0;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamGetCaptureInfo(s, &st, &capture) == cudaSuccess;
+    const bool captured = st != cudaStreamCaptureStatusNone;
+    // cudaStreamGetId ends a capture with an error; within one, a stream's handle names it
+    if (!known || (!captured && cudaStreamGetId(s, &id) != cudaSuccess)) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (captured) id = reinterpret_cast<uintptr_t>(s);
+    const std::pair<unsigned long long, unsigned long long> key(id, captured ? capture + 1 : 0);
+    std::lock_guard<std::mutex> lk(d.mu);
+    auto it = d.slots.find(key);
+    if (it == d.slots.end()) {
+        int slot;
+        if (captured) {
+            if (d.captured_slots == kSlots) return nullptr;
+            slot = kSlots + d.captured_slots++;
+        } else if (d.eager_slots < kSlots) {
+            slot = d.eager_slots++;
+        } else {
+            auto old = d.slots.end();
+            for (auto j = d.slots.begin(); j != d.slots.end(); ++j)
+                if (j->second < kSlots && (old == d.slots.end() || d.slot_use[j->second] < d.slot_use[old->second])) old = j;
+            slot = old->second;
+            d.slots.erase(old);
+        }
+        it = d.slots.emplace(key, slot).first;
+    }
+    if (!captured) d.slot_use[it->second] = ++d.slot_clock;
+    return d.ws + kWorkspaceFloats + it->second * kSlotFloats;
+}
+
 }  // namespace credit
 
 // ------------------------------------------------------------------ C ABI
@@ -487,7 +535,8 @@ credit_status credit_init(int device) {
     info.cc_minor = v;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrClockRate, device) == cudaSuccess) info.clock_khz = v;
     if (info.cc_major < 10) return CREDIT_ERR_UNSUPPORTED;  // needs Blackwell (sm_103a build)
-    if ((e = cudaMalloc(&d.ws, kWorkspaceFloats * sizeof(float))) != cudaSuccess) return cuda_status(e);
+    if ((e = cudaMalloc(&d.ws, (kWorkspaceFloats + 2 * kSlots * kSlotFloats) * sizeof(float))) != cudaSuccess)
+        return cuda_status(e);
     if ((e = cudaMalloc(&d.err, 64)) != cudaSuccess) return cuda_status(e);
     if ((e = cudaMemset(d.err, 0, 64)) != cudaSuccess) return cuda_status(e);
     if ((e = cudaStreamCreateWithFlags(&d.side, cudaStreamNonBlocking)) != cudaSuccess) return cuda_status(e);
@@ -879,12 +928,14 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
         return CREDIT_OK;
     }
     const long long cap_rows = static_cast<long long>(d.info.ws_floats / (static_cast<size_t>(G) * 4));
+    float *own = rows <= cap_rows ? stream_workspace(d, s, static_cast<size_t>(rows) * G * 4) : nullptr;
     const long long max_rows = cap_rows < 0x7FFFFFFFLL / G ? cap_rows : 0x7FFFFFFFLL / G;
     const bool fp8_stage = (a->op == OP_LN || a->op == OP_RMS) && tout == DT_E4M3;
     for (long long r0 = 0; r0 < rows; r0 += max_rows) {
         const long long n = rows - r0 < max_rows ? rows - r0 : max_rows;
         RowArgs r = rows_from(base, r0, n, isz, osz, lse);
         r.G = G;
+        if (own != nullptr) r.ws = own;
         void *args[] = {&r};
         const dim3 grid(static_cast<unsigned>(G * n));
         cudaError_t e = launch(ks.tp_stats, grid, dim3(threads), 0, 1, s, args);
@@ -939,6 +990,11 @@ credit_status credit_run_ex(const credit_args *args, const credit_plan_t *plan, 
         if (st != CREDIT_OK) return st;
     }
     if ((st = check_plan(dev, args, &chosen)) != CREDIT_OK) return st;
+    // a small call without a workspace of its own (more than 512 captured streams): whole rows, which need none
+    const size_t floats = static_cast<size_t>(args->rows) * static_cast<size_t>(chosen.ctas_per_row) * 4;
+    if (!plan && chosen.path == CREDIT_PATH_TWO_PASS && chosen.ctas_per_row > 1 && floats <= kSlotFloats &&
+        stream_workspace(g_dev[dev], stream, floats) == nullptr)
+        chosen.ctas_per_row = 1;
     return run_with_plan(dev, args, &chosen, stream);
 }
 
