@@ -534,6 +534,15 @@ void build_items(const std::vector<RRow> &rows, int isz, int P, int cap, std::ve
     }
 }
 
+// Copy a work list to the device, on the handle's stream, which does not wait for the legacy stream (nor does
+// cudaMemcpy from pageable memory for the last of its copies), and to the end, since the list is the caller's own.
+template <class T>
+bool upload(credit_ragged *h, T *dst, const std::vector<T> &src) {
+    return cudaMemcpyAsync(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, h->cap_stream) ==
+               cudaSuccess &&
+           cudaStreamSynchronize(h->cap_stream) == cudaSuccess;
+}
+
 // Median of three runs of a launch on the handle's stream (15 of a short one), after a warm-up.
 template <class F>
 cudaError_t time_launch(credit_ragged *h, F &&launch, float *us) {
@@ -589,9 +598,7 @@ credit_status upload_and_launch_config(credit_ragged *h, int P, int threads, int
         return CREDIT_ERR_UNSUPPORTED;
     }
     const long long ncl = std::min<long long>(maxc, static_cast<long long>(items.size()));
-    if (cudaMemcpy(h->d_rows, sorted.data(), sorted.size() * sizeof(RRow), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->d_items, items.data(), items.size() * sizeof(RItem), cudaMemcpyHostToDevice) != cudaSuccess)
-        return CREDIT_ERR_CUDA;
+    if (!upload(h, h->d_rows, sorted) || !upload(h, h->d_items, items)) return CREDIT_ERR_CUDA;
     RaggedArgs ra;
     ra.in = h->in;
     ra.out = h->out;
@@ -742,8 +749,7 @@ credit_status warps_config(credit_ragged *h, const WarpShape &w, float *us) {
     std::vector<WarpLaunch> ls;
     credit_status st = warps_plan(h, w, sorted, ls);
     if (st != CREDIT_OK) return st;
-    if (cudaMemcpy(h->d_rows, sorted.data(), sorted.size() * sizeof(RRow), cudaMemcpyHostToDevice) != cudaSuccess)
-        return CREDIT_ERR_CUDA;
+    if (!upload(h, h->d_rows, sorted)) return CREDIT_ERR_CUDA;
     int low = 0, high = 0;
     cudaDeviceGetStreamPriorityRange(&low, &high);
     std::vector<cudaStream_t> side(ls.size() - 1, nullptr);
@@ -857,7 +863,7 @@ credit_status credit_ragged_create(const credit_ragged_row *host_rows, int64_t n
         credit_ragged_destroy(h);
         return CREDIT_ERR_CUDA;
     }
-    cudaMemset(h->d_err, 0, 16);
+    cudaMemsetAsync(h->d_err, 0, 16, h->cap_stream);
     // autotune: cluster size x staging capacity x threads x vector width, timed on this batch
     const int Ps[3] = {4, 8, 16};
     const int vws[2] = {1, 2};  // 16-byte groups each thread reads before using them
