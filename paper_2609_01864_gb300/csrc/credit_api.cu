@@ -279,7 +279,7 @@ bool ring_config_tm(const DeviceInfo &di, long long N, int isz, int P, int req_r
 // without room for a stage per team, gives each team more threads.
 bool team_config(const DeviceInfo &di, long long rows, long long N, int isz, int nab, int P, int req_stages,
                  TeamCfg *out) {
-    if (N <= 0 || P < 1 || P > kMaxCluster || (P & (P - 1)) != 0) return false;
+    if (N <= 0 || !team_cluster(di, P)) return false;
     const long long V = 16 / isz, groups = (N / V + P - 1) / P;  // of a slice, at any phase of the row
     if (groups * 16 > di.smem_optin || (P > 1 && N / V < 32 * P)) return false;
     TeamCfg r;

@@ -1609,7 +1609,7 @@ int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, lon
         pays = many && bytes > kBwdTeamMaxBytes;
     if (!pays) return 0;
     const long long room = di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16, true);
-    for (int P = logits ? 2 : 16; P <= kMaxCluster; P *= 2)
+    for (int P = logits ? 2 : 16; team_cluster(di, P); P *= 2)
         if (room / ((bytes / 16 + P - 1) / P * 32) >= (logits ? 2 : 4)) return P;
     return 0;
 }
@@ -1634,7 +1634,7 @@ struct BwdTeamCfg {
 bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, int P, BwdTeamCfg *out) {
     const int isz = dtype_size(dtype), V = 16 / isz;
     const bool norm = op == BOP_LN || op == BOP_RMS;
-    if (P < 1 || P > kMaxCluster || (P & (P - 1)) != 0 || (P > 1 && cols / V < 32 * P)) return false;
+    if (!team_cluster(di, P) || (P > 1 && cols / V < 32 * P)) return false;
     if (P == 1 && cols * isz > kBwdTeamMaxBytes) return false;
     const long long groups = (cols / V + P - 1) / P, walkers = di.sm_count / P;
     const long long per_sm = (rows + walkers - 1) / walkers;

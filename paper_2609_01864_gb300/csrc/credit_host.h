@@ -46,6 +46,10 @@ constexpr long long kTmAutoMinSlice = 32768;
 // Tensor-memory retention geometry (k_ring_tm); false where it does not apply.
 bool ring_config_tm(const DeviceInfo &di, long long N, int isz, int P, int req_ring, int req_chunk, int nab,
                     RingCfg *out);
+// A cluster size that the whole-row kernels take: a power of two up to 16 on a device (or partition) of as many SMs.
+inline bool team_cluster(const DeviceInfo &di, int P) {
+    return P >= 1 && P <= 16 && (P & (P - 1)) == 0 && P <= di.sm_count;
+}
 // Geometry of k_row_team: teams of `threads` threads, `teams` of them in the
 // SM's one CTA, `stages` rows in flight per team; rows split over clusters of
 // P CTAs, `grid` of them.

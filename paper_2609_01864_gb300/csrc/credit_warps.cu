@@ -29,7 +29,7 @@ bool row_warps_config(const DeviceInfo &di, int op, int tin, int tout, long long
                       RowWarpsCfg *out) {
     if (tin != DT_F32 && tin != DT_BF16) return false;
     if (op == OP_SOFTMAX ? tout != tin : op == OP_Q8 ? tout != DT_I8 : op != OP_LSE) return false;
-    if (P < 1 || P > 16 || (P & (P - 1)) != 0 || (W != kWWarps && W != kWWarps / 2)) return false;
+    if (!team_cluster(di, P) || (W != kWWarps && W != kWWarps / 2)) return false;
     if (rows > (1LL << 30) || cols > (1LL << 24) || warps_smem(W) > di.smem_optin) return false;
     const long long groups = cols * dtype_size(tin) / 16 + 1;
     int lu = 0;
