@@ -643,7 +643,6 @@ credit_status validate_args(const credit_args *a) {
     return CREDIT_OK;
 }
 
-// Is `p` legal for the arguments on this device (Eq. 3 and scheduling)?
 // A ONE_CTA or CLUSTER plan of rows over warps: threads 256 or 512 (0), the other fields at their defaults.
 static bool warps_plan_config(const DeviceInfo &di, const credit_args *a, const credit_plan_t *p, RowWarpsCfg *out) {
     if ((p->threads != 0 && p->threads != 256 && p->threads != 512) || p->reducer_threads || p->chunk_bytes ||
@@ -654,6 +653,7 @@ static bool warps_plan_config(const DeviceInfo &di, const credit_args *a, const 
                             p->path == CREDIT_PATH_ONE_CTA ? 1 : p->cluster_size, p->threads == 256 ? 8 : 16, out);
 }
 
+// Is `p` legal for the arguments on this device (Eq. 3 and scheduling)?
 credit_status check_plan(int device, const credit_args *a, const credit_plan_t *p) {
     const DeviceInfo *di = device_info(device);
     if (!di) return CREDIT_ERR_NOT_INITIALIZED;
@@ -1028,6 +1028,11 @@ int32_t credit_max_clusters(const credit_args *args, const credit_plan_t *plan) 
     const DeviceInfo *di = device_info(dev);
     const int P = plan->path == CREDIT_PATH_ONE_CTA ? 1 : plan->cluster_size;
     const int tout = args->op == OP_LSE ? DT_F32 : args->out_dtype;
+    RowWarpsCfg wc;
+    if (plan->retain == CREDIT_RETAIN_WARPS)
+        return warps_plan_config(*di, args, plan, &wc)
+                   ? staged_max_clusters(dev, wc.fn, wc.P, 32 * wc.W, wc.smem, false)
+                   : 0;
     TeamCfg gc;
     if (team_plan_config(*di, args, plan, &gc))
         return staged_max_clusters(dev, team_kernel(args->op, args->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
