@@ -601,7 +601,10 @@ credit_status credit_mlp_load(const char *path);
  * issued the row's last chunk (6, 7 unused).  Tensor-memory retention:
  * 0 reducer row start, 5 its TMEM buffer free, 1 sweep done, 2 warp partial
  * merged and pushed; 6 writer row start, 3 statistics in hand, 4 writes done
- * (7 unused).  device_buf: caller-owned device memory, 8-byte aligned; NULL
+ * (7 unused).  Whole rows and rows over warps: the rows of a CTA's first team
+ * or warp, 0 row start, 5 its groups in shared memory, 3 statistics in hand,
+ * 4 outputs written (1, 2, 6, 7 unused).  The backward ops, the split and the
+ * ragged launches are not traced.  device_buf: caller-owned device memory, 8-byte aligned; NULL
  * turns tracing off.  Not thread-safe against concurrent launches; a
  * debugging aid, off by default.
  */

@@ -36,6 +36,9 @@ def _units():
     for tin in (0, 1, 2):
         for name in ("credit_kernels", "credit_team"):
             units.append((os.path.join(CSRC, name + ".cu"), f"{name}_{tin}.o", [f"-DCREDIT_TIN={tin}"]))
+        units.append((os.path.join(CSRC, "credit_team.cu"), f"credit_team_traced_{tin}.o",
+                      [f"-DCREDIT_TIN={tin}", "-DCREDIT_TRACED=1"]))
+    units.append((os.path.join(CSRC, "credit_warps.cu"), "credit_warps_traced.o", ["-DCREDIT_TRACED=1"]))
     for dt in (0, 1):
         units.append((os.path.join(CSRC, "credit_bwd.cu"), f"credit_bwd_{dt}.o", [f"-DCREDIT_BWD_DT={dt}"]))
     for src in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp"))):

@@ -26,6 +26,9 @@ bool kernels_tin2(int op, int tout, KernelSet *ks);
 const void *team_kernel_tin0(int op, int tout, bool grid, bool aff, bool cluster);
 const void *team_kernel_tin1(int op, int tout, bool grid, bool aff, bool cluster);
 const void *team_kernel_tin2(int op, int tout, bool grid, bool aff, bool cluster);
+const void *team_kernel_traced_tin0(int op, int tout, bool grid, bool aff, bool cluster);
+const void *team_kernel_traced_tin1(int op, int tout, bool grid, bool aff, bool cluster);
+const void *team_kernel_traced_tin2(int op, int tout, bool grid, bool aff, bool cluster);
 }  // namespace credit
 
 using namespace credit;
@@ -67,14 +70,14 @@ bool kernel_set(int op, int tin, int tout, KernelSet *ks) {
     }
 }
 
-const void *team_kernel(int op, int tin, int tout, bool grid, bool aff, bool cluster) {
-    if (op == OP_LSE) tout = DT_F32;
-    switch (tin) {
-    case DT_F32: return team_kernel_tin0(op, tout, grid, aff, cluster);
-    case DT_BF16: return team_kernel_tin1(op, tout, grid, aff, cluster);
-    case DT_E4M3: return team_kernel_tin2(op, tout, grid, aff, cluster);
-    default: return nullptr;
-    }
+// The team kernel of a call; traced: the one that writes the stamps of credit_set_trace.
+const void *team_kernel(const credit_args *a, const TeamCfg &g, bool traced = false) {
+    static const decltype(&team_kernel_tin0) of[2][3] = {
+        {team_kernel_tin0, team_kernel_tin1, team_kernel_tin2},
+        {team_kernel_traced_tin0, team_kernel_traced_tin1, team_kernel_traced_tin2}};
+    if (a->in_dtype < DT_F32 || a->in_dtype > DT_E4M3) return nullptr;
+    return of[traced][a->in_dtype](a->op, a->op == OP_LSE ? DT_F32 : a->out_dtype, g.grid_rows, g.affine_resident != 0,
+                                   g.P > 1);
 }
 
 credit_status cuda_status(cudaError_t e) {
@@ -682,8 +685,7 @@ credit_status check_plan(int device, const credit_args *a, const credit_plan_t *
         }
         TeamCfg gc;
         if (team_plan_config(*di, a, p, &gc))
-            return staged_max_clusters(device, team_kernel(a->op, a->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
-                                       false) > 0
+            return staged_max_clusters(device, team_kernel(a, gc), gc.P, gc.threads * gc.teams, gc.smem, false) > 0
                        ? CREDIT_OK
                        : CREDIT_ERR_UNSUPPORTED;
         RingCfg rc;
@@ -705,6 +707,10 @@ credit_status check_plan(int device, const credit_args *a, const credit_plan_t *
 
 static unsigned long long *g_trace_buf = nullptr;
 static int g_trace_rows = 0;
+unsigned long long *trace_buffer(int *rows) {
+    *rows = g_trace_rows;
+    return g_trace_buf;
+}
 // credit_set_wait_test (test only): the reducers' chunk-wait limit and the
 // extra bytes the first chunk's barrier expects
 static std::atomic<unsigned long long> g_wait_ns{0};
@@ -818,7 +824,7 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
         TeamCfg gc;
         if (team_plan_config(d.info, a, p, &gc)) {
             if (g_test_extra_tx.load() > 0) return CREDIT_ERR_UNSUPPORTED;  // the wait test's ring kernel only
-            const void *fn = team_kernel(a->op, tin, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1);
+            const void *fn = team_kernel(a, gc, base.trace != nullptr);
             if (fn == nullptr) return CREDIT_ERR_UNSUPPORTED;
             const credit_status st = prepare_kernel(d, fn, true);
             if (st != CREDIT_OK) return st;
@@ -1035,8 +1041,7 @@ int32_t credit_max_clusters(const credit_args *args, const credit_plan_t *plan) 
                    : 0;
     TeamCfg gc;
     if (team_plan_config(*di, args, plan, &gc))
-        return staged_max_clusters(dev, team_kernel(args->op, args->in_dtype, tout, gc.grid_rows, gc.affine_resident != 0, gc.P > 1), gc.P, gc.threads * gc.teams, gc.smem,
-                                   false);
+        return staged_max_clusters(dev, team_kernel(args, gc), gc.P, gc.threads * gc.teams, gc.smem, false);
     RingCfg rc;
     if (!ring_config_for(*di, args, dtype_size(args->in_dtype), P, plan, &rc)) return 0;
     return ring_max_clusters(dev, args->op, args->in_dtype, tout, P, rc.threads, rc.smem, rc.tmem != 0);

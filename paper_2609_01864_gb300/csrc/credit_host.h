@@ -70,6 +70,8 @@ struct RowWarpsCfg {
     long long smem;
     const void *fn;
 };
+// The buffer of credit_set_trace (null: none) and its rows per CTA.
+unsigned long long *trace_buffer(int *rows);
 // False where a row does not fit, or the op or types have no such kernel.
 bool row_warps_config(const DeviceInfo &di, int op, int tin, int tout, long long rows, long long cols, int P, int W,
                       RowWarpsCfg *out);

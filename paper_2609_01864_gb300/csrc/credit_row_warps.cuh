@@ -61,6 +61,8 @@ struct WarpArgs {
     long long ld_in, ld_out;  // rows of one width and op: strides (elements), columns, int8 scales
     int cols;
     float *out_scale;
+    unsigned long long *trace;  // as in RowArgs (TR)
+    int trace_rows;
 };
 constexpr int OP_ROWS = -1;  // k_row_warps: the op is the row's
 
@@ -136,7 +138,7 @@ __device__ __forceinline__ void write_segment(const unsigned char *d, unsigned c
     }
 }
 
-template <int OP, int TIN, int W>
+template <int OP, int TIN, int W, bool TR = false>  // TR: with the stamps of credit_set_trace
 __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int isz = Fmt<TIN>::size, V = Fmt<TIN>::V, osz = OP == OP_Q8 ? 1 : isz;
@@ -251,6 +253,11 @@ __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArg
     int was_first = 0;
     Turn turn{};
     enter(turn);
+    auto stamp = [&](int field) {
+        if constexpr (TR) {
+            if (warp == 0 && lane == 0) trace_stamp(a, turn.k, field);
+        }
+    };
     for (int last = 0;;) {
         const int lu = turn.lu, lw = turn.lw, k = turn.k, wl = 1 << (lu - lw), first = warp & ~(wl - 1);
         if (turn.cls != last) {
@@ -262,6 +269,7 @@ __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArg
         }
         was_first = first;
         if (turn.row < turn.row_end) {
+            stamp(0);
             const RRow rw = row_at(turn.row);
             const Seg s = segment(rw, lu, lw);
             const bool sm = OP == OP_ROWS ? rw.op == OP_SOFTMAX : true;  // a maximum (and a sum about it)
@@ -278,6 +286,7 @@ __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArg
                 mbar_wait_bounded(&full[h], phase >> h & 1u, a.err);
                 phase ^= 1u << h;
             }
+            stamp(5);
             float2 v = make_float2(-INFINITY, 0.0f);
             float lo = 0.0f;  // the segment's smallest element (softmax)
             float2 s2 = make_float2(0.0f, 0.0f);
@@ -344,6 +353,7 @@ __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArg
                 ++xchs;
                 v = merge(sm, sl[lane & (P - 1)], P);
             }
+            stamp(3);
             unsigned char *orow = a.out + rw.out_off * (OP == OP_LSE ? 4 : osz);
             Stats st{v.x, v.y};
             if constexpr (OP == OP_LSE) {
@@ -377,6 +387,7 @@ __global__ void __launch_bounds__(32 * W, kWWarps / W) k_row_warps(const WarpArg
                 }
                 if (ie >= 0) store_one<OP == OP_Q8 ? DT_I8 : TIN>(orow + static_cast<long long>(ie) * osz, one(xe));
             }
+            stamp(4);
             __syncwarp();  // the segment is done with: its half takes a later turn's
         }
         load_ahead(k);

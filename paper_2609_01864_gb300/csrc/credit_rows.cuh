@@ -852,7 +852,8 @@ __device__ __forceinline__ void write_chunk_direct(const unsigned char *cb, int 
 // done, [5] producer issued the row's last chunk.
 constexpr int kTraceCtas = 32;
 constexpr int kTraceFields = 8;
-__device__ __forceinline__ void trace_stamp(const RowArgs &a, int rr, int field) {
+template <class Args>
+__device__ __forceinline__ void trace_stamp(const Args &a, int rr, int field) {
     if (a.trace != nullptr && blockIdx.x < kTraceCtas && rr < a.trace_rows)
         a.trace[(static_cast<size_t>(blockIdx.x) * a.trace_rows + rr) * kTraceFields + field] = global_timer_ns();
 }

@@ -1,26 +1,35 @@
 // credit_team.cu -- instantiates the team kernels for one input
-// dtype (compiled with -DCREDIT_TIN=0, 1 and 2, like credit_kernels.cu).
+// dtype (compiled with -DCREDIT_TIN=0, 1 and 2, like credit_kernels.cu; with
+// -DCREDIT_TRACED=1 once more for the kernels that write trace stamps).
 #include "credit_row_team.cuh"
 
 #ifndef CREDIT_TIN
 #error "CREDIT_TIN must be defined (0 = FP32, 1 = BF16, 2 = FP8-E4M3)"
 #endif
 
+#ifndef CREDIT_TRACED
+#define CREDIT_TRACED 0
+#endif
 #define CREDIT_CAT2(a, b) a##b
 #define CREDIT_CAT(a, b) CREDIT_CAT2(a, b)
+#if CREDIT_TRACED
+#define CREDIT_TEAM_KERNEL CREDIT_CAT(team_kernel_traced_tin, CREDIT_TIN)
+#else
+#define CREDIT_TEAM_KERNEL CREDIT_CAT(team_kernel_tin, CREDIT_TIN)
+#endif
 
 namespace credit {
 
 // Clusters: rows at any phase, gamma / beta always in shared memory.
 template <int OP, int TOUT>
 static const void *team_fn(bool grid, bool aff, bool cluster) {
-    constexpr bool N = OP == OP_LN || OP == OP_RMS;
-    if (cluster) return reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, true>);
+    constexpr bool N = OP == OP_LN || OP == OP_RMS, R = CREDIT_TRACED != 0;
+    if (cluster) return reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, true, R>);
     if (N && aff)
-        return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, N, false>)
-                    : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, false>);
-    return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, false, false>)
-                : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, false, false>);
+        return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, N, false, R>)
+                    : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, N, false, R>);
+    return grid ? reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, true, false, false, R>)
+                : reinterpret_cast<const void *>(&k_row_team<OP, CREDIT_TIN, TOUT, false, false, false, R>);
 }
 
 template <int OP>
@@ -33,7 +42,7 @@ static const void *team_out(int tout, bool grid, bool aff, bool cluster) {
     }
 }
 
-const void *CREDIT_CAT(team_kernel_tin, CREDIT_TIN)(int op, int tout, bool grid, bool aff, bool cluster) {
+const void *CREDIT_TEAM_KERNEL(int op, int tout, bool grid, bool aff, bool cluster) {
     switch (op) {
     case OP_SOFTMAX: return team_out<OP_SOFTMAX>(tout, grid, aff, cluster);
     case OP_LSE: return team_fn<OP_LSE, DT_F32>(grid, aff, cluster);

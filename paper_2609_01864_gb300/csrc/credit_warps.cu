@@ -1,5 +1,7 @@
 // credit_warps.cu -- k_row_warps for rows of one width: softmax, log-sum-exp
 // and int8 quantisation of FP32 and BF16 rows (plans with CREDIT_RETAIN_WARPS).
+// Compiled twice: with -DCREDIT_TRACED=1 for the kernels that write trace
+// stamps alone.
 #include <cuda_runtime.h>
 
 #include "../../include/credit.h"
@@ -8,23 +10,30 @@
 
 namespace credit {
 
-template <int W>
+template <int W, bool TR>
 static const void *kernel_of(int op, int tin) {
     const bool f32 = tin == DT_F32;
     switch (op) {
     case OP_SOFTMAX:
-        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_SOFTMAX, DT_F32, W>)
-                   : reinterpret_cast<const void *>(&k_row_warps<OP_SOFTMAX, DT_BF16, W>);
+        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_SOFTMAX, DT_F32, W, TR>)
+                   : reinterpret_cast<const void *>(&k_row_warps<OP_SOFTMAX, DT_BF16, W, TR>);
     case OP_LSE:
-        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_LSE, DT_F32, W>)
-                   : reinterpret_cast<const void *>(&k_row_warps<OP_LSE, DT_BF16, W>);
+        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_LSE, DT_F32, W, TR>)
+                   : reinterpret_cast<const void *>(&k_row_warps<OP_LSE, DT_BF16, W, TR>);
     case OP_Q8:
-        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_Q8, DT_F32, W>)
-                   : reinterpret_cast<const void *>(&k_row_warps<OP_Q8, DT_BF16, W>);
+        return f32 ? reinterpret_cast<const void *>(&k_row_warps<OP_Q8, DT_F32, W, TR>)
+                   : reinterpret_cast<const void *>(&k_row_warps<OP_Q8, DT_BF16, W, TR>);
     default: return nullptr;
     }
 }
 
+const void *row_warps_kernel_traced(int op, int tin, int W);
+
+#if CREDIT_TRACED
+const void *row_warps_kernel_traced(int op, int tin, int W) {
+    return W == kWWarps ? kernel_of<kWWarps, true>(op, tin) : kernel_of<kWWarps / 2, true>(op, tin);
+}
+#else
 bool row_warps_config(const DeviceInfo &di, int op, int tin, int tout, long long rows, long long cols, int P, int W,
                       RowWarpsCfg *out) {
     if (tin != DT_F32 && tin != DT_BF16) return false;
@@ -36,19 +45,21 @@ bool row_warps_config(const DeviceInfo &di, int op, int tin, int tout, long long
     while ((1 << lu) < P) ++lu;
     while (((groups - 1) >> lu) + 1 > 2 * kWHalf)
         if ((1 << ++lu) > P * W) return false;
-    *out = {P, W, lu, warps_smem(W), W == kWWarps ? kernel_of<kWWarps>(op, tin) : kernel_of<kWWarps / 2>(op, tin)};
+    *out = {P, W, lu, warps_smem(W), W == kWWarps ? kernel_of<kWWarps, false>(op, tin) : kernel_of<kWWarps / 2, false>(op, tin)};
     return out->fn != nullptr;
 }
 
 credit_status run_row_warps(int device, const credit_args *a, const RowWarpsCfg &cfg, cudaStream_t s) {
-    credit_status st = prepare_staged_kernel(device, cfg.fn);
+    WarpArgs w{};
+    w.trace = trace_buffer(&w.trace_rows);
+    const void *fn = w.trace != nullptr ? row_warps_kernel_traced(a->op, a->in_dtype, cfg.W) : cfg.fn;
+    credit_status st = prepare_staged_kernel(device, fn);
     if (st != CREDIT_OK) return st;
-    const int most = staged_max_clusters(device, cfg.fn, cfg.P, 32 * cfg.W, cfg.smem, false);
+    const int most = staged_max_clusters(device, fn, cfg.P, 32 * cfg.W, cfg.smem, false);
     if (most <= 0) return CREDIT_ERR_UNSUPPORTED;
     const long long per = static_cast<long long>(cfg.P) * cfg.W >> cfg.lu;  // rows a cluster works on at a time
     const long long want = (a->rows + per - 1) / per;
     const int ncl = static_cast<int>(want < most ? want : most);
-    WarpArgs w{};
     w.in = static_cast<const unsigned char *>(a->in);
     w.out = static_cast<unsigned char *>(a->out);
     w.n_classes = 1;
@@ -62,9 +73,10 @@ credit_status run_row_warps(int device, const credit_args *a, const RowWarpsCfg 
     w.cols = static_cast<int>(a->cols);
     w.out_scale = a->out_scale;
     void *args[] = {&w};
-    const cudaError_t e = launch_kernel(cfg.fn, dim3(static_cast<unsigned>(cfg.P * ncl)), dim3(32 * cfg.W),
+    const cudaError_t e = launch_kernel(fn, dim3(static_cast<unsigned>(cfg.P * ncl)), dim3(32 * cfg.W),
                                         static_cast<size_t>(cfg.smem), cfg.P, s, args);
     return e == cudaSuccess ? CREDIT_OK : CREDIT_ERR_CUDA;
 }
+#endif
 
 }  // namespace credit
