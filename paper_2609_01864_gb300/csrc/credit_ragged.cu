@@ -482,33 +482,47 @@ struct credit_ragged {
     int device = 0;
     int dtype = 0;
     long long n_rows = 0;
-    std::vector<RRow> rows;  // host copy, original order
+    std::vector<RRow> rows;  // host copy, widest first
     const unsigned char *in = nullptr;
     unsigned char *out = nullptr;
-    // chosen launch
-    int P = 0, threads = 0, cap = 0, clusters = 0, vw = 1, kernels = 1;
-    long long n_items = 0, n_narrow = 0, n_wide = 0, n_huge = 0;
-    RRow *d_rows = nullptr;
-    RItem *d_items = nullptr;
+    RRow *d_rows = nullptr;    // the same
+    RItem *d_items = nullptr;  // of the cluster size and capacity last used
     unsigned *d_err = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    // A captured launch of the batch.
+    struct Launch {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        int P = 0, threads = 0, cap = 0, clusters = 0, vw = 1, kernels = 1;
+        long long n_items = 0, n_narrow = 0, n_wide = 0, n_huge = 0;
+        void destroy() {
+            if (exec) cudaGraphExecDestroy(exec);
+            if (graph) cudaGraphDestroy(graph);
+            exec = nullptr;
+            graph = nullptr;
+        }
+    } l;  // the chosen one
     float tuned_us = 0.0f;
 };
 
 namespace {
 
-// Items for launch shape (P, cap): rows sorted widest first; each row gets
+// Items for launch shape (P, cap), rows widest first: each row gets
 // the smallest power-of-two width w <= P whose slices (plus 32 bytes for an
 // unaligned head and tail) fit cap bytes, consecutive rows of one width share
 // an item (P / w of them), and rows that fit no width are huge.
-void build_items(const std::vector<RRow> &rows, int isz, int P, int cap, std::vector<RItem> &items,
-                 std::vector<RRow> &sorted, long long &nn, long long &nw, long long &nh) {
-    sorted = rows;
-    std::stable_sort(sorted.begin(), sorted.end(), [](const RRow &x, const RRow &y) { return x.cols > y.cols; });
+struct ItemList {
+    int P = 0, cap = 0;
+    long long nn = 0, nw = 0, nh = 0;  // items of one CTA, of several, streamed rows
+    std::vector<RItem> items;
+};
+void build_items(const std::vector<RRow> &sorted, int isz, int P, int cap, ItemList &l) {
+    std::vector<RItem> &items = l.items;
+    long long &nn = l.nn, &nw = l.nw, &nh = l.nh;
     items.clear();
     nn = nw = nh = 0;
+    l.P = P;
+    l.cap = cap;
     auto width_of = [&](const RRow &r) -> int {
         const long long groups = r.cols * isz / 16 + 1;
         for (int w = 1; w <= P; w *= 2)
@@ -543,23 +557,25 @@ bool upload(credit_ragged *h, T *dst, const std::vector<T> &src) {
            cudaStreamSynchronize(h->cap_stream) == cudaSuccess;
 }
 
-// Median of three runs of a launch on the handle's stream (15 of a short one), after a warm-up.
+// Median of `n` runs of a launch on the handle's stream (five times as many of a short one), after a warm-up.  A
+// launch whose warm-up takes twice `limit`, or whose first run is 15% above it, is not run again.
 template <class F>
-cudaError_t time_launch(credit_ragged *h, F &&launch, float *us) {
+cudaError_t time_launch(credit_ragged *h, int n, float limit, F &&launch, float *us) {
     cudaEvent_t a0, a1;
     cudaEventCreate(&a0);
     cudaEventCreate(&a1);
     std::vector<float> t;
     cudaError_t e = cudaSuccess;
-    for (int k = 0, n = 3; k <= n && e == cudaSuccess; ++k) {
+    for (int k = 0; k <= n && e == cudaSuccess; ++k) {
         cudaEventRecord(a0, h->cap_stream);
         e = launch();
         cudaEventRecord(a1, h->cap_stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(a1);
         float ms = 0;
         cudaEventElapsedTime(&ms, a0, a1);
-        if (k) t.push_back(ms * 1e3f);
-        if (k == 1 && ms < 0.2f) n = 15;
+        if (k || ms > 2e-3f * limit) t.push_back(ms * 1e3f);
+        if (t.size() == 1 && t[0] > 1.15f * limit) break;
+        if (k == 1 && ms < 0.2f) n *= 5;
     }
     cudaEventDestroy(a0);
     cudaEventDestroy(a1);
@@ -569,13 +585,12 @@ cudaError_t time_launch(credit_ragged *h, F &&launch, float *us) {
     return cudaSuccess;
 }
 
-credit_status upload_and_launch_config(credit_ragged *h, int P, int threads, int cap, int vw, float *us_out) {
-    const int isz = dtype_size(h->dtype);
+// k_ragged over the items on the device: timed (us not null), or captured as *out.
+credit_status items_config(credit_ragged *h, const ItemList &list, int threads, int vw, float limit, float *us_out,
+                           credit_ragged::Launch *out) {
     const DeviceInfo *di = device_info(h->device);
-    std::vector<RItem> items;
-    std::vector<RRow> sorted;
-    long long nn, nw, nh;
-    build_items(h->rows, isz, P, cap, items, sorted, nn, nw, nh);
+    const int P = list.P, cap = list.cap;
+    const std::vector<RItem> &items = list.items;
     const long long smem = kRCtrl + cap;
     if (smem > di->smem_optin) return CREDIT_ERR_UNSUPPORTED;
     const void *fn = ragged_kernel(h->dtype, vw);
@@ -598,7 +613,6 @@ credit_status upload_and_launch_config(credit_ragged *h, int P, int threads, int
         return CREDIT_ERR_UNSUPPORTED;
     }
     const long long ncl = std::min<long long>(maxc, static_cast<long long>(items.size()));
-    if (!upload(h, h->d_rows, sorted) || !upload(h, h->d_items, items)) return CREDIT_ERR_CUDA;
     RaggedArgs ra;
     ra.in = h->in;
     ra.out = h->out;
@@ -612,28 +626,33 @@ credit_status upload_and_launch_config(credit_ragged *h, int P, int threads, int
     cfg.gridDim = dim3(static_cast<unsigned>(P * std::max<long long>(ncl, 1)));
     cfg.stream = h->cap_stream;
     if (us_out != nullptr)
-        return time_launch(h, [&] { return cudaLaunchKernelExC(&cfg, fn, args); }, us_out) == cudaSuccess ? CREDIT_OK
-                                                                                                          : CREDIT_ERR_CUDA;
+        return time_launch(h, 3, limit, [&] { return cudaLaunchKernelExC(&cfg, fn, args); }, us_out) == cudaSuccess
+                   ? CREDIT_OK
+                   : CREDIT_ERR_CUDA;
     if (cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return CREDIT_ERR_CUDA;
     cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
-    cudaGraph_t g = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
-    if (e != cudaSuccess || e2 != cudaSuccess) return CREDIT_ERR_CUDA;
-    if (h->exec) cudaGraphExecDestroy(h->exec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    h->graph = g;
-    if (cudaGraphInstantiate(&h->exec, g, 0) != cudaSuccess) return CREDIT_ERR_CUDA;
-    h->kernels = 1;
-    h->P = P;
-    h->vw = vw;
-    h->threads = threads;
-    h->cap = cap;
-    h->clusters = static_cast<int>(ncl);
-    h->n_items = static_cast<long long>(items.size());
-    h->n_narrow = nn;
-    h->n_wide = nw;
-    h->n_huge = nh;
+    cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &out->graph);
+    if (e != cudaSuccess || e2 != cudaSuccess || cudaGraphInstantiate(&out->exec, out->graph, 0) != cudaSuccess) {
+        out->destroy();
+        return CREDIT_ERR_CUDA;
+    }
+    out->kernels = 1;
+    out->P = P;
+    out->vw = vw;
+    out->threads = threads;
+    out->cap = cap;
+    out->clusters = static_cast<int>(ncl);
+    out->n_items = static_cast<long long>(items.size());
+    out->n_narrow = list.nn;
+    out->n_wide = list.nw;
+    out->n_huge = list.nh;
     return CREDIT_OK;
+}
+
+// The items of (P, cap) in the handle's device list.
+bool use_items(credit_ragged *h, int P, int cap, ItemList &list) {
+    build_items(h->rows, dtype_size(h->dtype), P, cap, list);
+    return upload(h, h->d_items, list.items);
 }
 
 // One launch of k_row_warps: the rows that take clusters of P CTAs.
@@ -654,15 +673,14 @@ struct WarpLaunch {
 struct WarpShape {
     int P, W, q, tight, spread;
 };
-credit_status warps_plan(credit_ragged *h, const WarpShape &w, std::vector<RRow> &sorted, std::vector<WarpLaunch> &out) {
+credit_status warps_plan(credit_ragged *h, const WarpShape &w, std::vector<WarpLaunch> &out) {
+    const std::vector<RRow> &sorted = h->rows;
     const int P = w.P, spread = w.spread, W = w.W;
     const int isz = dtype_size(h->dtype);
     const DeviceInfo *di = device_info(h->device);
     if (warps_smem(kWWarps) > di->smem_optin || P < 0 || P > 16 || (P & (P - 1)) != 0 || spread < 0 || spread > 9 || w.q < 1 ||
         (W != kWWarps && W != kWWarps / 2))
         return CREDIT_ERR_UNSUPPORTED;
-    sorted = h->rows;
-    std::stable_sort(sorted.begin(), sorted.end(), [](const RRow &x, const RRow &y) { return x.cols > y.cols; });
     const long long n = static_cast<long long>(sorted.size());
     const int most = 31 - __builtin_clz(static_cast<unsigned>(P ? W * P : kWWarps * 16));
     if (n > (1LL << 30) || sorted[0].cols > (1LL << 24) || ((sorted[0].cols * isz / 16 + 1) >> most) + 1 > 2 * kWHalf)
@@ -740,16 +758,11 @@ credit_status warps_plan(credit_ragged *h, const WarpShape &w, std::vector<RRow>
 
 // Capture the launches as a graph of parallel kernels, widest rows first (the
 // SMs that clusters leave over, and those that run out of wide rows, take the
-// next launch's), time it (us not null) and keep it as the handle's unless it
-// is slower than *us.  Each kernel after the first adds 1.5 us to the launch of
-// a graph that runs do not hide behind another (107 BF16 rows of 16K to 119K,
-// four kernels: 16.6 us alone against 14.3 for one that timed alike).
-credit_status warps_config(credit_ragged *h, const WarpShape &w, float *us) {
-    std::vector<RRow> sorted;
+// next launch's).
+credit_status warps_config(credit_ragged *h, const WarpShape &w, credit_ragged::Launch *out) {
     std::vector<WarpLaunch> ls;
-    credit_status st = warps_plan(h, w, sorted, ls);
+    credit_status st = warps_plan(h, w, ls);
     if (st != CREDIT_OK) return st;
-    if (!upload(h, h->d_rows, sorted)) return CREDIT_ERR_CUDA;
     int low = 0, high = 0;
     cudaDeviceGetStreamPriorityRange(&low, &high);
     std::vector<cudaStream_t> side(ls.size() - 1, nullptr);
@@ -758,8 +771,6 @@ credit_status warps_config(credit_ragged *h, const WarpShape &w, float *us) {
     auto ok = [&](cudaError_t r) { e = e == cudaSuccess ? r : e; };
     for (auto &q : side) ok(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     for (auto &q : ev) ok(cudaEventCreateWithFlags(&q, cudaEventDisableTiming));
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
     if (e == cudaSuccess) {
         ok(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
         if (e == cudaSuccess) {
@@ -788,40 +799,105 @@ credit_status warps_config(credit_ragged *h, const WarpShape &w, float *us) {
                     ok(cudaStreamWaitEvent(h->cap_stream, ev[i], 0));
                 }
             }
-            ok(cudaStreamEndCapture(h->cap_stream, &graph));
+            ok(cudaStreamEndCapture(h->cap_stream, &out->graph));
         }
-        if (e == cudaSuccess) ok(cudaGraphInstantiate(&exec, graph, 0));
+        if (e == cudaSuccess) ok(cudaGraphInstantiate(&out->exec, out->graph, 0));
     }
     for (auto &q : side)
         if (q) cudaStreamDestroy(q);
     for (auto &q : ev)
         if (q) cudaEventDestroy(q);
-    float t = 0.0f;
-    if (e == cudaSuccess && us != nullptr) e = time_launch(h, [&] { return cudaGraphLaunch(exec, h->cap_stream); }, &t);
-    const float cost = t + 1.5f * static_cast<float>(ls.size() - 1);
-    if (e != cudaSuccess || (us != nullptr && cost >= *us)) {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        return e == cudaSuccess ? CREDIT_OK : CREDIT_ERR_CUDA;
+    if (e != cudaSuccess) {
+        out->destroy();
+        return CREDIT_ERR_CUDA;
     }
-    if (us != nullptr) *us = cost;
-    if (h->exec) cudaGraphExecDestroy(h->exec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    h->exec = exec;
-    h->graph = graph;
-    h->kernels = static_cast<int>(ls.size());
-    h->P = ls[0].P;
-    h->vw = 1;
-    h->threads = 32 * kWWarps;
-    h->cap = kWWarps * 2 * kWHalf * 16;
-    h->n_items = static_cast<long long>(sorted.size());
-    h->n_narrow = h->n_wide = h->n_huge = 0;
-    h->clusters = 0;
+    out->kernels = static_cast<int>(ls.size());
+    out->P = ls[0].P;
+    out->vw = 1;
+    out->threads = 32 * kWWarps;
+    out->cap = kWWarps * 2 * kWHalf * 16;
+    out->n_items = static_cast<long long>(h->rows.size());
+    out->n_narrow = out->n_wide = out->n_huge = 0;
+    out->clusters = 0;
     for (const WarpLaunch &l : ls) {
-        h->clusters += l.ncl;
+        out->clusters += l.ncl;
         for (int j = 0; j < l.args.n_classes; ++j)
-            (l.args.cls[j].lw == 0 ? h->n_narrow : h->n_wide) += l.args.cls[j].row_end - l.args.cls[j].row0;
+            (l.args.cls[j].lw == 0 ? out->n_narrow : out->n_wide) += l.args.cls[j].row_end - l.args.cls[j].row0;
     }
+    return CREDIT_OK;
+}
+
+// Choose the launch by timing shapes on this batch: k_ragged's cluster size x staging capacity x threads x vector
+// width, then rows over warps, each as far as it keeps up with the best so far.  The best four within 4% are captured
+// and timed again, nine runs each, as they will be launched.  Shapes that share the lead stay hard to tell apart: of
+// 20000 BF16 rows of 1K to 1M columns one launch's own runs lie between 2.05 and 2.16 ms.  Making that batch takes
+// 0.6 s (1.1 s with every shape run to the end), 8000 rows of 8K to 40K 107 ms (171).
+credit_status autotune(credit_ragged *h, ItemList &list) {
+    struct Trial {
+        float us;
+        int P, cap, threads, vw;  // threads = 32 kWWarps: `w`
+        WarpShape w;
+    };
+    std::vector<Trial> trials;
+    float best = 1e30f;
+    auto add = [&](const Trial &t) {
+        best = std::min(best, t.us);
+        trials.push_back(t);
+    };
+    for (int P : {4, 8, 16})
+        for (int cap : {3 * kRChunk, 4 * kRChunk, 6 * kRChunk, 13 * kRChunk}) {  // 4, 3, 2, 1 CTAs per SM
+            if (!use_items(h, P, cap, list)) return CREDIT_ERR_CUDA;
+            for (int threads : {128, 256})  // the kernel is built for up to 256 threads, 4 CTAs per SM (64 registers)
+                for (int vw : {1, 2}) {     // 16-byte groups each thread reads before using them
+                    float us = 0.0f;
+                    if (items_config(h, list, threads, vw, best, &us, nullptr) == CREDIT_OK)
+                        add({us, P, cap, threads, vw, {}});
+                }
+        }
+    // Each kernel after the first adds 1.5 us to the launch of a graph that runs do not hide behind another (107 BF16
+    // rows of 16K to 119K, four kernels: 16.6 us alone against 14.3 for one that timed alike).
+    auto more = [](const credit_ragged::Launch &l) { return 1.5f * static_cast<float>(l.kernels - 1); };
+    auto replay = [&](const credit_ragged::Launch &l) { return [&] { return cudaGraphLaunch(l.exec, h->cap_stream); }; };
+    auto try_warps = [&](const WarpShape &w) {
+        credit_ragged::Launch l;
+        float us = 0.0f;
+        if (warps_config(h, w, &l) != CREDIT_OK) return;
+        if (time_launch(h, 3, best, replay(l), &us) == cudaSuccess) add({us + more(l), 0, 0, 32 * kWWarps, 1, w});
+        l.destroy();
+    };
+    for (int W : {kWWarps, kWWarps / 2}) {
+        for (int q : {2, 4, 8, 16}) try_warps({0, W, q, 1, 0});
+        for (int q : {2, 8}) try_warps({0, W, q, 0, 0});
+        for (int spread = 1; spread < 4; ++spread) try_warps({0, W, 8, 0, spread});
+    }
+    for (int P : {1, 2, 4, 8})
+        for (int spread : {0, 2}) try_warps({P, kWWarps, 1, 0, spread});
+
+    std::stable_sort(trials.begin(), trials.end(), [](const Trial &x, const Trial &y) { return x.us < y.us; });
+    float least = 1e30f;
+    for (size_t i = 0; i < trials.size() && i < 4 && trials[i].us <= 1.04f * best; ++i) {
+        const Trial &t = trials[i];
+        credit_ragged::Launch l;
+        const bool warps = t.threads == 32 * kWWarps;
+        const credit_status st = warps ? warps_config(h, t.w, &l)
+                                 : use_items(h, t.P, t.cap, list)
+                                     ? items_config(h, list, t.threads, t.vw, 0.0f, nullptr, &l)
+                                     : CREDIT_ERR_CUDA;
+        float us = 0.0f;
+        if (st != CREDIT_OK) continue;
+        if (time_launch(h, 9, least, replay(l), &us) != cudaSuccess || us + more(l) >= least) {
+            l.destroy();
+            continue;
+        }
+        least = us + more(l);
+        h->l.destroy();
+        h->l = l;
+    }
+    if (h->l.exec == nullptr) return CREDIT_ERR_UNSUPPORTED;
+    h->tuned_us = least;
+    if (h->l.threads != 32 * kWWarps && (list.P != h->l.P || list.cap != h->l.cap) &&
+        !use_items(h, h->l.P, h->l.cap, list))
+        return CREDIT_ERR_CUDA;
     return CREDIT_OK;
 }
 
@@ -855,77 +931,45 @@ credit_status credit_ragged_create(const credit_ragged_row *host_rows, int64_t n
         }
         h->rows[i] = RRow{r.in_off, r.out_off, r.cols, r.op, 0};
     }
+    std::stable_sort(h->rows.begin(), h->rows.end(), [](const RRow &x, const RRow &y) { return x.cols > y.cols; });
     const bool ok = cudaMalloc(&h->d_rows, n * sizeof(RRow)) == cudaSuccess &&
                     cudaMalloc(&h->d_items, n * sizeof(RItem)) == cudaSuccess &&
                     cudaMalloc(&h->d_err, 16) == cudaSuccess &&
-                    cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) == cudaSuccess;
+                    cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
+                    upload(h, h->d_rows, h->rows);
     if (!ok) {
         credit_ragged_destroy(h);
         return CREDIT_ERR_CUDA;
     }
     cudaMemsetAsync(h->d_err, 0, 16, h->cap_stream);
-    // autotune: cluster size x staging capacity x threads x vector width, timed on this batch
-    const int Ps[3] = {4, 8, 16};
-    const int vws[2] = {1, 2};  // 16-byte groups each thread reads before using them
-    const int caps[4] = {3 * kRChunk, 4 * kRChunk, 6 * kRChunk, 13 * kRChunk};  // 4, 3, 2, 1 CTAs per SM
-    const int thr[2] = {128, 256};  // the kernel is built for up to 256 threads, 4 CTAs per SM (64 registers)
-    float best = 1e30f;
-    int bP = 16, bcap = caps[3], bthr = 256, bvw = 1;
-    WarpShape shape{0, kWWarps, 4, 0, 0};
-    if (!tune) {  // fixed launch shape (CREDIT_RAGGED_P / _CHUNKS / _THREADS / _VW override the defaults;
-                  // _THREADS = 512: k_row_warps, with _P = 0 for each row's own, _W, _Q, _TIGHT and _SPREAD)
-        const char *eP = std::getenv("CREDIT_RAGGED_P"), *eC = std::getenv("CREDIT_RAGGED_CHUNKS");
-        const char *eT = std::getenv("CREDIT_RAGGED_THREADS"), *eV = std::getenv("CREDIT_RAGGED_VW");
-        if (eP) bP = std::atoi(eP);
-        if (eC) bcap = std::atoi(eC) * kRChunk;
-        if (eT) bthr = std::atoi(eT);
-        if (eV) bvw = std::atoi(eV);
-        if (const char *eN = std::getenv("CREDIT_RAGGED_W")) shape.W = std::atoi(eN);
-        if (const char *eQ = std::getenv("CREDIT_RAGGED_Q")) shape.q = std::atoi(eQ);
-        if (const char *eF = std::getenv("CREDIT_RAGGED_TIGHT")) shape.tight = std::atoi(eF);
-        if (const char *eS = std::getenv("CREDIT_RAGGED_SPREAD")) shape.spread = std::atoi(eS);
-        shape.P = bP;
-        if (bP < (bthr == 32 * kWWarps ? 0 : 1) || bP > 16 || bcap < kRChunk || bcap > 13 * kRChunk || (bthr != 32 * kWWarps && (bthr < 64 || bthr > 256 || bthr % 32)) ||
-            (bvw != 1 && bvw != 2)) {
-            credit_ragged_destroy(h);
-            return CREDIT_ERR_INVALID_ARG;
-        }
-    } else {
-        for (int P : Ps)
-            for (int cap : caps)
-                for (int t : thr)
-                    for (int vw : vws) {
-                        float us = 0;
-                        if (upload_and_launch_config(h, P, t, cap, vw, &us) == CREDIT_OK && us < best) {
-                            best = us;
-                            bP = P;
-                            bcap = cap;
-                            bthr = t;
-                            bvw = vw;
-                        }
-                    }
-        bool warps = false;
-        auto try_warps = [&](const WarpShape &w) {
-            const float was = best;
-            if (warps_config(h, w, &best) == CREDIT_OK && best < was) warps = true;
+    ItemList list;
+    if (tune) {
+        st = autotune(h, list);
+    } else {  // fixed launch shape (CREDIT_RAGGED_P / _CHUNKS / _THREADS / _VW override the defaults;
+              // _THREADS = 512: k_row_warps, with _P = 0 for each row's own, _W, _Q, _TIGHT and _SPREAD)
+        int P = 16, cap = 13 * kRChunk, threads = 256, vw = 1;
+        WarpShape shape{0, kWWarps, 4, 0, 0};
+        auto env = [](const char *name, int &v, int unit = 1) {
+            if (const char *e = std::getenv(name)) v = std::atoi(e) * unit;
         };
-        for (int W : {kWWarps, kWWarps / 2}) {
-            for (int q : {2, 4, 8, 16}) try_warps({0, W, q, 1, 0});
-            for (int q : {2, 8}) try_warps({0, W, q, 0, 0});
-            for (int spread = 1; spread < 4; ++spread) try_warps({0, W, 8, 0, spread});
-        }
-        for (int P : {1, 2, 4, 8})
-            for (int spread : {0, 2}) try_warps({P, kWWarps, 1, 0, spread});
-        if (warps) bthr = 32 * kWWarps;
-        if (best >= 1e30f) {
-            credit_ragged_destroy(h);
-            return CREDIT_ERR_UNSUPPORTED;
-        }
+        env("CREDIT_RAGGED_P", P);
+        env("CREDIT_RAGGED_CHUNKS", cap, kRChunk);
+        env("CREDIT_RAGGED_THREADS", threads);
+        env("CREDIT_RAGGED_VW", vw);
+        env("CREDIT_RAGGED_W", shape.W);
+        env("CREDIT_RAGGED_Q", shape.q);
+        env("CREDIT_RAGGED_TIGHT", shape.tight);
+        env("CREDIT_RAGGED_SPREAD", shape.spread);
+        shape.P = P;
+        const bool warps = threads == 32 * kWWarps;
+        if (P < (warps ? 0 : 1) || P > 16 || cap < kRChunk || cap > 13 * kRChunk ||
+            (!warps && (threads < 64 || threads > 256 || threads % 32)) || (vw != 1 && vw != 2))
+            st = CREDIT_ERR_INVALID_ARG;
+        else if (warps)
+            st = warps_config(h, shape, &h->l);
+        else
+            st = use_items(h, P, cap, list) ? items_config(h, list, threads, vw, 0.0f, nullptr, &h->l) : CREDIT_ERR_CUDA;
     }
-    h->tuned_us = tune ? best : 0.0f;
-    if (bthr != 32 * kWWarps) st = upload_and_launch_config(h, bP, bthr, bcap, bvw, nullptr);
-    else if (!tune) st = warps_config(h, shape, nullptr);
-    else st = CREDIT_OK;  // captured when it was timed
     if (st != CREDIT_OK) {
         credit_ragged_destroy(h);
         return st;
@@ -936,31 +980,30 @@ credit_status credit_ragged_create(const credit_ragged_row *host_rows, int64_t n
 }
 
 credit_status credit_ragged_run(credit_ragged *h, cudaStream_t stream) {
-    if (!h || !h->exec) return CREDIT_ERR_INVALID_ARG;
-    if (cudaGraphLaunch(h->exec, stream) != cudaSuccess) return CREDIT_ERR_CUDA;
-    g_launch_count.fetch_add(h->kernels);
+    if (!h || !h->l.exec) return CREDIT_ERR_INVALID_ARG;
+    if (cudaGraphLaunch(h->l.exec, stream) != cudaSuccess) return CREDIT_ERR_CUDA;
+    g_launch_count.fetch_add(h->l.kernels);
     return CREDIT_OK;
 }
 
 credit_status credit_ragged_info(const credit_ragged *h, credit_ragged_info_t *out) {
     if (!h || !out) return CREDIT_ERR_INVALID_ARG;
-    out->cluster_size = h->P;
-    out->threads = h->threads;
-    out->staging_bytes = h->cap;
-    out->clusters = h->clusters;
-    out->items = h->n_items;
-    out->narrow_items = h->n_narrow;
-    out->wide_items = h->n_wide;
-    out->huge_items = h->n_huge;
+    out->cluster_size = h->l.P;
+    out->threads = h->l.threads;
+    out->staging_bytes = h->l.cap;
+    out->clusters = h->l.clusters;
+    out->items = h->l.n_items;
+    out->narrow_items = h->l.n_narrow;
+    out->wide_items = h->l.n_wide;
+    out->huge_items = h->l.n_huge;
     out->tuned_us = h->tuned_us;
-    out->vector_groups = h->vw;
+    out->vector_groups = h->l.vw;
     return CREDIT_OK;
 }
 
 void credit_ragged_destroy(credit_ragged *h) {
     if (!h) return;
-    if (h->exec) cudaGraphExecDestroy(h->exec);
-    if (h->graph) cudaGraphDestroy(h->graph);
+    h->l.destroy();
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     cudaFree(h->d_rows);
     cudaFree(h->d_items);

@@ -39,3 +39,36 @@ def test_run_on_another_stream_right_after_making(monkeypatch, threads):
             want[k] = y
         else:
             assert torch.equal(y, want[k % 3])
+
+
+@pytest.mark.parametrize("rows,lo,hi", [(3000, 20000, 500000)])
+def test_autotuning_costs_a_bounded_number_of_runs(rows, lo, hi):
+    """Shapes that fall behind are not run to the end: 74 shapes in fewer than 330 runs' time of the chosen one."""
+    import math
+    import random
+    import time
+    rng = random.Random(7)
+    table, off = [], 0
+    for _ in range(rows):
+        w = int(lo * 2 ** (rng.random() * math.log2(hi / lo)))
+        table.append((off, off, w, C.SOFTMAX if rng.random() < 0.5 else C.RMSNORM))
+        off += w
+    x = torch.randn(off, device="cuda").bfloat16()
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    C.Ragged(table[:50], C.BF16, x, y).close()  # kernels loaded
+    t0 = time.perf_counter()
+    R = C.Ragged(table, C.BF16, x, y)
+    made = time.perf_counter() - t0
+    for _ in range(3):
+        R.run()
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record()
+    for _ in range(10):
+        R.run()
+    b.record()
+    torch.cuda.synchronize()
+    one = a.elapsed_time(b) / 10 * 1e-3
+    R.close()
+    assert made < 330 * one, (made, one)
