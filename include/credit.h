@@ -429,8 +429,10 @@ credit_status credit_bwd_plan_check(const credit_bwd_args *args, const credit_pl
  * exchanging partials over DSMEM (w = 1: the one-CTA path, w = P: the cluster
  * path).  Rows beyond the capacity at w = P stream twice within the cluster.
  * Batches whose rows all fit a cluster's shared memory may instead run with
- * every row over 1, 2, 4, ... 256 warps (threads = 512; an item is then a row,
- * clusters those of all its launches, one per cluster size).
+ * every row over 1, 2, 4, ... 256 warps, one launch per cluster size: threads =
+ * 512 stands for this kind, in CTAs of 16 or 8 warps; cluster_size and
+ * staging_bytes (of a CTA) are those of the widest rows' launch, clusters those
+ * of all launches, and an item is a row.
  * Info: narrow_items counts the items of one CTA, wide_items those of several,
  * huge_items the streamed rows.  The project's addition; the paper runs
  * one shape per launch.
@@ -444,7 +446,7 @@ typedef struct credit_ragged credit_ragged;
 typedef struct {
     int32_t cluster_size, threads, staging_bytes, clusters;
     int64_t items, narrow_items, wide_items, huge_items;
-    float tuned_us;  /* autotuner's best time for the batch (0 if not tuned) */
+    float tuned_us;  /* the chosen launch's median time when the batch was made (0 if not tuned) */
     int32_t vector_groups;  /* vector width: 16-byte groups a thread reads per step (1 or 2) */
 } credit_ragged_info_t;
 /* Build the work list, autotune (tune != 0: cluster size 4/8/16 x staging

@@ -815,7 +815,7 @@ credit_status warps_config(credit_ragged *h, const WarpShape &w, credit_ragged::
     out->P = ls[0].P;
     out->vw = 1;
     out->threads = 32 * kWWarps;
-    out->cap = kWWarps * 2 * kWHalf * 16;
+    out->cap = ls[0].W * 2 * kWHalf * 16;
     out->n_items = static_cast<long long>(h->rows.size());
     out->n_narrow = out->n_wide = out->n_huge = 0;
     out->clusters = 0;
@@ -890,11 +890,11 @@ credit_status autotune(credit_ragged *h, ItemList &list) {
             continue;
         }
         least = us + more(l);
+        h->tuned_us = us;
         h->l.destroy();
         h->l = l;
     }
     if (h->l.exec == nullptr) return CREDIT_ERR_UNSUPPORTED;
-    h->tuned_us = least;
     if (h->l.threads != 32 * kWWarps && (list.P != h->l.P || list.cap != h->l.cap) &&
         !use_items(h, h->l.P, h->l.cap, list))
         return CREDIT_ERR_CUDA;

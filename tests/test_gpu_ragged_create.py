@@ -72,3 +72,15 @@ def test_autotuning_costs_a_bounded_number_of_runs(rows, lo, hi):
     one = a.elapsed_time(b) / 10 * 1e-3
     R.close()
     assert made < 330 * one, (made, one)
+
+
+@pytest.mark.parametrize("W", [8, 16])
+def test_info_of_rows_over_warps(monkeypatch, W):
+    """threads = 512 marks the kind; staging_bytes are those of the launch's own CTAs, of W buffers of 14080 bytes."""
+    for k, v in dict(THREADS=512, P=0, W=W).items():
+        monkeypatch.setenv("CREDIT_RAGGED_" + k, str(v))
+    x = torch.zeros(9000, device="cuda")
+    R = C.Ragged([(0, 0, 9000, C.RMSNORM)], C.F32, x, x, tune=False)
+    info = R.info()
+    R.close()
+    assert (info["threads"], info["staging_bytes"], info["tuned_us"]) == (512, W * 14080, 0.0)
