@@ -289,6 +289,15 @@ credit_status credit_run_host(const credit_args *args, const credit_plan_t *plan
 int32_t credit_max_clusters(const credit_args *args, const credit_plan_t *plan);
 
 /*
+ * credit_plan_kernel -- the kernel that `plan` runs for these arguments
+ * ("k_row_team", "k_row_warps", "k_ring", "k_ring_tm", "k_tp_fused",
+ * "k_tp_stats" for a split row; of a plan with a fill its cluster kernel), ""
+ * where credit_plan_check refuses it.  Tells a RETAIN_ROW plan whose rows do
+ * not fit (and so means AUTO) from one that runs as whole rows.
+ */
+const char *credit_plan_kernel(const credit_args *args, const credit_plan_t *plan);
+
+/*
  * credit_plan_check -- CREDIT_OK if `plan` is legal for `args` on the current
  * device (Eq. 3 capacity, cluster size, scheduling), CREDIT_ERR_UNSUPPORTED
  * if not, CREDIT_ERR_INVALID_ARG for bad arguments.  Launches nothing.
@@ -417,6 +426,10 @@ credit_status credit_plan_bwd(int32_t op, int64_t rows, int64_t cols, credit_dty
 
 /* CREDIT_OK if `plan` is legal for `args` (see credit_run_bwd), else its error; launches nothing. */
 credit_status credit_bwd_plan_check(const credit_bwd_args *args, const credit_plan_t *plan);
+
+/* The kernel that `plan` runs for `args` ("k_bwd_team", "k_bwd_staged", "k_bwd_tp_fused", "k_bwd_tp_stats" for a split
+ * row), "" where credit_bwd_plan_check refuses it. */
+const char *credit_bwd_plan_kernel(const credit_bwd_args *args, const credit_plan_t *plan);
 
 /* ------------------------------------------------------------------ ragged batches
  * Rows of uneven width and mixed op in one persistent cluster launch captured

@@ -109,6 +109,10 @@ def lib() -> ctypes.CDLL:
             L.credit_plan_check.argtypes = [ctypes.POINTER(ArgsT), ctypes.POINTER(PlanT)]
             L.credit_max_clusters.restype = i32
             L.credit_max_clusters.argtypes = [ctypes.POINTER(ArgsT), ctypes.POINTER(PlanT)]
+            L.credit_plan_kernel.restype = ctypes.c_char_p
+            L.credit_plan_kernel.argtypes = [ctypes.POINTER(ArgsT), ctypes.POINTER(PlanT)]
+            L.credit_bwd_plan_kernel.restype = ctypes.c_char_p
+            L.credit_bwd_plan_kernel.argtypes = [ctypes.POINTER(BwdArgsT), ctypes.POINTER(PlanT)]
             L.credit_device_error.restype = i32
             L.credit_device_error.argtypes = [vp]
             L.credit_slice_capacity.restype = i64
@@ -344,6 +348,12 @@ def max_clusters(op: int, x, out, plan: PlanT, **kw) -> int:
     return int(lib().credit_max_clusters(ctypes.byref(a), ctypes.byref(plan)))
 
 
+def plan_kernel(op: int, x, out, plan: PlanT, **kw) -> str:
+    """credit_plan_kernel: name of the kernel a plan runs for these arguments; empty if illegal."""
+    a = make_args(op, x, out, **kw)
+    return lib().credit_plan_kernel(ctypes.byref(a), ctypes.byref(plan)).decode()
+
+
 def run_ex(op: int, x, out, *, plan: PlanT | None = None, stream=None, **kw) -> int:
     """credit_run_ex.  x / out: tensors or raw device addresses; keyword
     arguments as make_args.  Returns the status (raises CreditError on a
@@ -409,6 +419,12 @@ def plan_bwd(op: int, rows: int, cols: int, dtype: int) -> PlanT:
 def bwd_plan_check(op: int, a, dy, dx, plan: PlanT, **kw) -> int:
     r = make_bwd_args(op, a, dy, dx, **kw)
     return lib().credit_bwd_plan_check(ctypes.byref(r), ctypes.byref(plan))
+
+
+def bwd_plan_kernel(op: int, a, dy, dx, plan: PlanT, **kw) -> str:
+    """credit_bwd_plan_kernel: name of the kernel a backward plan runs for these arguments; empty if illegal."""
+    r = make_bwd_args(op, a, dy, dx, **kw)
+    return lib().credit_bwd_plan_kernel(ctypes.byref(r), ctypes.byref(plan)).decode()
 
 
 def run_ex_status(*args, **kw) -> int:

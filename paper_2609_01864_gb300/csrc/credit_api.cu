@@ -1047,6 +1047,22 @@ int32_t credit_max_clusters(const credit_args *args, const credit_plan_t *plan) 
     return ring_max_clusters(dev, args->op, args->in_dtype, tout, P, rc.threads, rc.smem, rc.tmem != 0);
 }
 
+const char *credit_plan_kernel(const credit_args *args, const credit_plan_t *plan) {
+    int dev = 0;
+    if (!plan || validate_args(args) != CREDIT_OK || ensure_init(&dev, nullptr) != CREDIT_OK ||
+        check_plan(dev, args, plan) != CREDIT_OK)
+        return "";
+    if (plan->path == CREDIT_PATH_TWO_PASS) return plan->ctas_per_row == 1 ? "k_tp_fused" : "k_tp_stats";
+    if (plan->retain == CREDIT_RETAIN_WARPS) return "k_row_warps";
+    const DeviceInfo *di = device_info(dev);
+    TeamCfg gc;
+    if (team_plan_config(*di, args, plan, &gc)) return "k_row_team";
+    RingCfg rc;
+    const int P = plan->path == CREDIT_PATH_ONE_CTA ? 1 : plan->cluster_size;
+    if (!ring_config_for(*di, args, dtype_size(args->in_dtype), P, plan, &rc)) return "";
+    return rc.tmem ? "k_ring_tm" : "k_ring";
+}
+
 credit_status credit_plan_check(const credit_args *args, const credit_plan_t *plan) {
     credit_status st = validate_args(args);
     if (st != CREDIT_OK) return st;

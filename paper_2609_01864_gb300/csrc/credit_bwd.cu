@@ -1679,6 +1679,13 @@ bool phases_agree(const credit_bwd_args *a) {
     return ((ua ^ ud) & 15u) == 0 && ua % dtype_size(a->dtype) == 0;
 }
 
+// Does k_bwd_team run a (legal) plan: one CTA per row, or rows split over clusters?
+bool runs_team(const DeviceInfo &di, const credit_bwd_args *a, const credit_plan_t *p, BwdTeamCfg *tc) {
+    const int P = p->retain == CREDIT_RETAIN_ROW ? p->cluster_size
+                  : p->path == CREDIT_PATH_TWO_PASS && p->ctas_per_row == 1 ? 1 : 0;
+    return P > 0 && phases_agree(a) && bwd_team_config(di, a->op, a->dtype, a->rows, a->cols, P, tc);
+}
+
 // gamma is staged in shared memory by the norms when present and 16-byte aligned.
 bool stage_gamma(int op, const float *gamma) {
     return (op == BOP_LN || op == BOP_RMS) && gamma != nullptr && (reinterpret_cast<uintptr_t>(gamma) & 15u) == 0;
@@ -1830,6 +1837,18 @@ credit_status credit_bwd_plan_check(const credit_bwd_args *args, const credit_pl
     return check_bwd_plan(dev, args, plan, &cfg, &maxc);
 }
 
+const char *credit_bwd_plan_kernel(const credit_bwd_args *args, const credit_plan_t *plan) {
+    int dev = 0, maxc = 0;
+    BwdCfg cfg;
+    if (validate_bwd(args) != CREDIT_OK || plan == nullptr || ensure_init(&dev, nullptr) != CREDIT_OK ||
+        check_bwd_plan(dev, args, plan, &cfg, &maxc) != CREDIT_OK)
+        return "";
+    BwdTeamCfg tc;
+    if (runs_team(*device_info(dev), args, plan, &tc)) return "k_bwd_team";
+    if (plan->path != CREDIT_PATH_TWO_PASS) return "k_bwd_staged";
+    return plan->ctas_per_row == 1 ? "k_bwd_tp_fused" : "k_bwd_tp_stats";
+}
+
 credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *plan, cudaStream_t stream) {
     credit_status st = validate_bwd(args);
     if (st != CREDIT_OK) return st;
@@ -1867,12 +1886,9 @@ credit_status credit_run_bwd(const credit_bwd_args *args, const credit_plan_t *p
     const long long rows = args->rows;
     cudaError_t e;
 
-    // k_bwd_team: one CTA per row, or (tP > 1) rows split over clusters
-    const int tP = chosen.retain == CREDIT_RETAIN_ROW ? chosen.cluster_size
-                   : chosen.path == CREDIT_PATH_TWO_PASS && chosen.ctas_per_row == 1 ? 1 : 0;
     BwdTeamCfg tc;
-    if (tP > 0 && phases_agree(args) &&
-        bwd_team_config(*device_info(dev), args->op, args->dtype, rows, args->cols, tP, &tc)) {
+    if (runs_team(*device_info(dev), args, &chosen, &tc)) {
+        const int tP = tc.P;
         const bool grid_rows = rows_aligned(args) && args->cols % (16 / dtype_size(args->dtype)) == 0;
         const void *fn = tP > 1 ? k.team_cl : k.team[grid_rows][tc.gamma_smem];
         if ((st = prepare_staged_kernel(dev, fn)) != CREDIT_OK) return st;
