@@ -97,6 +97,9 @@ int two_pass_split(int sm_count, long long rows, long long cols, int isz) {
     return static_cast<int>(G < 1 ? 1 : G);
 }
 
+// Widest rows that row_plan gives to one CTA's teams, and to a cluster's.
+constexpr long long kTeamRowBytes = 96 << 10, kTeamClusterBytes = 1 << 20;
+
 // Rows (or slices of rows) of one CTA's teams that fit shared memory beside the op's gamma / beta.
 static long long team_room(const DeviceInfo &di, long long cols, int isz, int nab, int P) {
     const long long V = 16 / isz, groups = (cols / V + P - 1) / P;
@@ -143,7 +146,7 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
     const bool grid = cols * isz % 16 == 0, fp8 = tin == 2 || tout == 2, sm8 = op == CREDIT_OP_SOFTMAX && tin == 2;
     const long long bytes = cols * isz;
     const bool many = rows >= 4LL * di.sm_count;
-    long long limit = 96 << 10;
+    long long limit = kTeamRowBytes;
     if (op == CREDIT_OP_LOGSUMEXP) limit = tin == 0 ? limit : tin == 1 ? 32 << 10 : 8 << 10;
     else if (sm8) limit = 24 << 10;
     else if (nab && !fp8 && grid) limit = 48 << 10;
@@ -154,7 +157,7 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
                                                               (nab > 1 || rows >= di.sm_count))
                                                      : true;
     const bool split = op != CREDIT_OP_LOGSUMEXP && !sm8 && pays && (!grid || (nab && fp8)) &&
-                       bytes <= (grid ? 450 << 10 : 1 << 20);
+                       bytes <= (grid ? 450LL << 10 : kTeamClusterBytes);
     if (split && (P == 0 || (nab && (many || (tin == 2 && !(op == CREDIT_OP_RMSNORM && grid && bytes <= 64 << 10)))))) {
         int q = nab || P ? 1 : 4;
         while (q <= 16 && team_room(di, cols, isz, nab, q) < 3) q *= 2;
@@ -173,46 +176,61 @@ static bool row_plan(const DeviceInfo &di, int op, long long rows, long long col
 }
 
 // Rows over warps (k_row_warps), for softmax, log-sum-exp and int8 of FP32 and
-// BF16 rows.  u is the number of warps whose buffers hold a row.  Clusters of
-// CTAs of 8 warps, two to an SM, of which a row takes four warps each (rows of
-// 128 KiB 104 us, 107 with its 16 warps in one CTA), eight of 8 CTAs from u =
-// 64 (512 KiB 408, over 16 CTAs 436), and eight CTAs of 16 warps at u = 128;
-// one CTA while that holds the row (but for many rows of 96 KiB, 2600 FP32 94
-// us against 80 over four), or there is hardly a row per SM (150 rows of 128 KiB
-// 11 against 13).  Measured (2400 rows, 600 from 768 KiB on, the
-// plan before -> this): BF16 softmax 128 KiB 122 -> 106, 192 KiB 204 -> 151,
-// 256 KiB 235 -> 208, 384 KiB 384 -> 300, 768 KiB 225 -> 169, 1.5 MiB 430 ->
-// 361; FP32 128 KiB 116 -> 104, 384 KiB 294 -> 288, 768 KiB 191 -> 160; int8
-// BF16 192 KiB 153 -> 121, 384 KiB 308 -> 239, FP32 off the grid 512 KiB 397 ->
-// 287; log-sum-exp FP32 192 KiB 84 -> 74, BF16 96 KiB 48 -> 43.  Outside the
-// ranges below the other paths are level or ahead: FP32 softmax of 128 KiB with
-// few rows (300 rows 15.6 against 17.3), 192 KiB (149 against 153), 256 KiB
-// (600 rows 58 against 61), 448 KiB (355 against 404) or above 900 KiB, BF16
-// int8 of 96 KiB (61 against 66), int8 of 1 MiB, which eight CTAs' tensor
-// memory holds (600 rows 176 against 198), log-sum-exp FP32 128 KiB with few
-// rows (600 rows 15 against 18) and 256 KiB (103 against 107), BF16 128 KiB
-// (600 rows 16 against 18), rows of 2 MiB (BF16 softmax 500 against 587).
+// BF16 rows.  u is the number of warps whose buffers of 880 16-byte groups hold
+// a row, fill the part of them that it fills.  Clusters of CTAs of 8 warps, two
+// to an SM, of which a row takes four warps each (rows of 128 KiB 104 us, 107
+// with its 16 warps in one CTA), eight of 8 CTAs from u = 64 (512 KiB 408, over
+// 16 CTAs 436), and eight CTAs of 16 warps at u = 128; one CTA while that holds
+// the row (but for many rows of u = 8, 2600 FP32 of 96 KiB 94 us against 80
+// over four), or there is hardly a row per SM (150 rows of 128 KiB 11 against
+// 13).
+// Where it pays, the other plans' time over this one's for 200, 400, 600, 1300
+// and 2600 rows (u = 8 .. 128 at six fills and 24 widths in whole KiB, on and
+// off the 16-byte grid):
+//   - half-full buffers keep half the bytes in flight.  FP32 softmax u = 32 and
+//     64 above fill 0.6 1.02-1.46, at 0.5-0.58 0.86-1.18 (448 KiB 0.87, 512 KiB
+//     0.92); u = 128 0.81-1.2 at all.  BF16 softmax, whose other path reads the
+//     row twice, 1.05-1.53 from u = 16 on, u = 128 0.95-1.16.
+//   - u = 8 (55 to 110 KiB) competes with whole rows in one CTA up to 96 KiB
+//     (kTeamRowBytes): beyond, FP32 softmax 1.0-1.26, BF16 1.02-1.43, int8
+//     1.9-2.7 (0.88-1.45 off the grid); within, BF16 softmax off the grid
+//     1.0-1.31, on it 0.97-1.2, but with more than 8 rows per SM 0.90-0.95 from
+//     fill 0.65 on; FP32 softmax and int8 0.78-1.0, log-sum-exp 0.95-1.35.
+//   - u = 16: FP32 softmax above two rows per SM 0.96-1.42, below 0.91-1.09;
+//     BF16 int8 off the grid below two rows per SM 0.72-1.01.  Int8 from u = 16
+//     on 1.0-2.9 else; FP32 u = 128 behind eight CTAs' rings of whole 16 KiB
+//     chunks (896 and 1024 KiB 0.86-0.95), 1.5-1.7 at other widths of that fill.
+//   - log-sum-exp, with no output to save a second look for: u = 8 0.95-1.53,
+//     BF16 u = 4 from fill 0.72 1.0-1.41; FP32 u = 16 above 8 rows per SM
+//     1.13-1.3, below 0.83-1.16; wider 0.54-1.25.
 static bool warps_plan(const DeviceInfo &di, int op, long long rows, long long cols, int tin, int tout,
                        credit_plan_t *p) {
-    const int isz = dtype_size(tin);
-    const long long kib = cols * isz / 1024;
-    const bool f32 = tin == 0;
-    bool pays = false;
     if (tin > 1) return false;
-    if (op == CREDIT_OP_SOFTMAX)
-        pays = f32 ? (kib >= 90 && kib <= 160 && rows >= 3LL * di.sm_count) || (kib >= 300 && kib <= 400) ||
-                         (kib > 640 && kib <= 900)
-                   : kib >= 60 && kib <= 1700;
-    else if (op == CREDIT_OP_QUANT_INT8)
-        pays = kib >= (cols * isz % 16 == 0 ? 101 : 96) && kib <= 1700 && !(kib > 900 && kib <= 1024);
-    else if (op == CREDIT_OP_LOGSUMEXP)
-        pays = f32 ? kib >= 60 && kib <= (rows >= 8LL * di.sm_count ? 220 : 110) : kib >= 40 && kib <= 110;
-    if (!pays) return false;
     RowWarpsCfg c;
     if (!row_warps_config(di, op, tin, tout, rows, cols, 1, 16, &c) &&
         !row_warps_config(di, op, tin, tout, rows, cols, 16, 16, &c))
         return false;
+    const long long bytes = cols * dtype_size(tin);
+    const bool f32 = tin == 0, grid = bytes % 16 == 0, many = rows >= 8LL * di.sm_count, two = rows > 2LL * di.sm_count;
     const int u = 1 << c.lu;
+    const float fill = static_cast<float>(bytes / 16) / static_cast<float>(880 * u);
+    bool pays = false;
+    if (op == CREDIT_OP_SOFTMAX) {
+        if (u == 8)
+            pays = bytes > kTeamRowBytes || (!f32 && fill > 0.54f && (!grid || !many || fill < 0.65f));
+        else if (u == 16)
+            pays = !f32 || two;
+        else
+            pays = f32 ? (u == 32 || u == 64) && fill > 0.6f : u >= 32;
+    } else if (op == CREDIT_OP_QUANT_INT8) {
+        const bool ring8 = bytes / 16 * 16 % (8 * 16384) == 0 && (grid || bytes > kTeamClusterBytes);
+        pays = u == 8    ? bytes > kTeamRowBytes
+               : u == 16 ? f32 || grid || two
+                         : u > 16 && !(f32 && u == 128 && fill < 0.6f && ring8);
+    } else if (op == CREDIT_OP_LOGSUMEXP) {
+        pays = f32 ? (u == 8 && fill > 0.54f) || (u == 16 && many) : u == 8 || (u == 4 && fill > 0.72f);
+    }
+    if (!pays) return false;
     int P = u < 8 ? 1 : u <= 8 ? (op != CREDIT_OP_LOGSUMEXP && rows >= 8LL * di.sm_count ? 4 : 1) : u <= 32 ? u / 4 : 8;
     int W = u <= 64 ? 8 : 16;
     if (u == 16 && rows < 2LL * di.sm_count) {

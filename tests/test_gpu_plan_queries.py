@@ -119,3 +119,21 @@ def test_kernels_of_other_plans():
                        (C.make_plan(C.PATH_TWO_PASS, ctas_per_row=4), "k_tp_stats"),
                        (C.make_plan(C.PATH_CLUSTER, 3, retain=C.RETAIN_WARPS), "")):
         assert C.plan_kernel(C.SOFTMAX, x, x, plan) == want
+
+
+@pytest.mark.parametrize("op,dt,rows,nbytes,warps", [
+    (C.SOFTMAX, C.F32, 600, 98 << 10, True), (C.SOFTMAX, C.F32, 400, 128 << 10, True), (C.SOFTMAX, C.F32, 304, 128 << 10, False),
+    (C.SOFTMAX, C.F32, 600, 288 << 10, True), (C.SOFTMAX, C.F32, 600, 448 << 10, False), (C.SOFTMAX, C.F32, 600, 560 << 10, True),
+    (C.SOFTMAX, C.F32, 600, 1024 << 10, False), (C.SOFTMAX, C.BF16, 2600, 88 << 10, False),
+    (C.SOFTMAX, C.BF16, 2600, (88 << 10) + 2, True), (C.SOFTMAX, C.BF16, 600, 88 << 10, True),
+    (C.SOFTMAX, C.BF16, 600, 1024 << 10, True), (C.SOFTMAX, C.BF16, 600, 1740 << 10, True),
+    (C.QUANT_INT8, C.F32, 600, 98 << 10, True), (C.QUANT_INT8, C.F32, 600, 896 << 10, False),
+    (C.QUANT_INT8, C.F32, 600, 1000 << 10, True), (C.QUANT_INT8, C.F32, 600, 1024 << 10, False),
+    (C.QUANT_INT8, C.BF16, 200, (160 << 10) + 2, False), (C.QUANT_INT8, C.BF16, 400, (160 << 10) + 2, True),
+    (C.LOGSUMEXP, C.F32, 600, 128 << 10, False), (C.LOGSUMEXP, C.F32, 1300, 128 << 10, True),
+    (C.LOGSUMEXP, C.BF16, 600, 36 << 10, False), (C.LOGSUMEXP, C.BF16, 600, 48 << 10, True),
+    (C.LOGSUMEXP, C.BF16, 600, 57 << 10, True), (C.LOGSUMEXP, C.F32, 600, 57 << 10, False)])
+def test_rows_over_warps_are_planned_by_their_buffers(op, dt, rows, nbytes, warps):
+    """Both sides of the planner's lines: how many warps' buffers a row takes, and how full they are."""
+    p = C.plan(op, rows, nbytes // SIZE[dt], dt, C.INT8 if op == C.QUANT_INT8 else None)
+    assert (p.retain == C.RETAIN_WARPS) == warps
