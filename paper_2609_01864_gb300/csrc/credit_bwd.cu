@@ -1578,42 +1578,6 @@ bool bwd_config(const DeviceInfo &di, long long N, int isz, int P, int req_nbuf,
     return false;
 }
 
-// CTAs per row of a cluster team plan (CLUSTER, retain ROW), 0 where the other
-// paths are the better ones.  Logits ops: the smallest cluster of which a CTA
-// holds two rows' slices at a time.  Measured (GB300, 1200 rows, staged or
-// two-pass -> this): BF16 on the 16-byte grid 96 KiB per array 87 -> 71 us,
-// 140 KiB 150 -> 120, 200 KiB 182 -> 152, 300 KiB 276 -> 271, 420 KiB 382 ->
-// 339; FP32 300 KiB 273 -> 236, 420 KiB 377 -> 295, off the grid 96 KiB 71 ->
-// 65, 200 KiB 187 -> 135, 420 KiB 383 -> 298; 100 FP32 rows of 300 KiB 60 ->
-// 30.  Behind stay FP32 rows on the grid within the staged kernel's four
-// slices of 64 KiB (1300 x 200 KiB 147 against 153), BF16 rows a little wider
-// than those (1300 x 264 KiB 276 against 290), few rows on the grid (150 x 100
-// KiB BF16 15 against 18) or narrow off it (100 x 96 KiB FP32 9 against 14),
-// and single slices (1000 KiB 883 against 1201).  Softmax from its output, off
-// the grid only (on it the staged kernel is at the copy rate), not few rows
-// (300 x 100 KiB FP32 19 against 24): clusters of 16 while four slices fit,
-// 140 KiB BF16 122 -> 101, 256 KiB 226 -> 187, 420 KiB 370 -> 347; three
-// slices lose (600 KiB 530 against 677), smaller clusters gain less.  The
-// norms, with gamma beside the slices, and the pair ops lose or stay level at
-// most widths.
-int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, bool grid) {
-    const long long bytes = cols * dtype_size(dtype);
-    const bool logits = op == BOP_SMLOGITS || op == BOP_XENT, many = rows >= 4LL * di.sm_count;
-    bool pays = false;
-    if (logits && grid)
-        pays = bytes > (dtype == CREDIT_F32 ? 256 << 10 : 300 << 10) ||
-               (dtype == CREDIT_BF16 && many && bytes > 64 << 10 && bytes <= 256 << 10);
-    else if (logits)
-        pays = bytes > (many ? 64 << 10 : 128 << 10);
-    else if (op == BOP_SOFTMAX && !grid)
-        pays = many && bytes > kBwdTeamMaxBytes;
-    if (!pays) return 0;
-    const long long room = di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16, true);
-    for (int P = logits ? 2 : 16; team_cluster(di, P); P *= 2)
-        if (room / ((bytes / 16 + P - 1) / P * 32) >= (logits ? 2 : 4)) return P;
-    return 0;
-}
-
 credit_plan_t bwd_row_plan(int P) {
     credit_plan_t p;
     std::memset(&p, 0, sizeof(p));
@@ -1671,6 +1635,66 @@ bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, lo
     r.grid_rows = false;
     *out = r;
     return true;
+}
+
+// CTAs per row of a cluster team plan (CLUSTER, retain ROW), 0 where the other
+// paths are the better ones.  Logits ops: the smallest cluster of which a CTA
+// holds two rows' slices at a time.  What decides is the part of shared memory
+// that its teams' stages fill: P goes up in twos, so rows just too wide for one
+// P leave half of the next one's empty (112, 224 and 448 KiB per array: one
+// stage of two teams, fill 0.5).  Measured (GB300, 24 widths of 56 to 1000 KiB
+// per array, 150 to 2600 rows; the other plans' time over this one's for the
+// cross entropy, softmax from logits alike or a little ahead):
+//   - BF16 on the 16-byte grid, from four rows per SM on: fill 0.55 and up, and
+//     rows of which the staged kernel holds one at a time, 0.99-1.24; fill 0.49
+//     beside two rows of the staged kernel (112 KiB; 114, beside one, 1.14-1.2)
+//     0.80-0.95; with fewer rows behind the staged kernel (0.85-1.19) up to its
+//     four slices of 64 KiB.  Wider rows from fill 0.65 on 0.96-1.27 (264 KiB,
+//     0.58, 0.89-0.99), with fewer rows 0.95-1.43.
+//   - BF16 off the grid, beyond the one-CTA rows of 96 KiB: two teams from fill
+//     0.52 on 0.91-1.18 (0.49: over four CTAs 0.99-1.05, eight 0.90-1.0), one
+//     from 0.7 on 0.91-1.28 (264 to 300 KiB, below it, 0.79-1.02, 600 KiB
+//     0.87-0.98); with fewer than four rows per SM above 256 KiB from 0.7 on
+//     0.95-1.25, two per SM of narrower ones from 0.8 on 1.06 (0.90-0.93 below).
+//   - FP32 on the grid beyond the staged kernel's reach 0.99-1.63, within it
+//     0.69-1.14; off the grid from four rows per SM on 1.0-1.46, with two per SM
+//     above 128 KiB 0.99-1.21, with one per SM only above 256 KiB 1.0-1.39 (160
+//     KiB 0.72).
+// Rows of which no cluster holds two slices take the two-pass path (1000 KiB
+// 883 us against 1201).  Softmax from its output, off the grid only (on it the
+// staged kernel is at the copy rate), not few rows (300 x 100 KiB FP32 19
+// against 24): clusters of 16 while four slices fit, 140 KiB BF16 122 -> 101,
+// 256 KiB 226 -> 187, 420 KiB 370 -> 347; three slices lose (600 KiB 530 against
+// 677), smaller clusters gain less.  The norms, with gamma beside the slices, and
+// the pair ops lose or stay level at most widths.
+int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, bool grid) {
+    const long long bytes = cols * dtype_size(dtype), kStagedMax = 4 * 65536;  // plan_bwd_for: P <= 4, 64 KiB slices
+    const bool logits = op == BOP_SMLOGITS || op == BOP_XENT, f32 = dtype == CREDIT_F32, many = rows >= 4LL * di.sm_count;
+    if (bytes <= (grid ? bwd_team_bytes(op) : f32 ? 65536 : kBwdTeamMaxBytes) || (!logits && (op != BOP_SOFTMAX || grid)))
+        return 0;
+    const long long room = di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16, true);
+    int P = logits ? 2 : 16;
+    while (team_cluster(di, P) && room / ((bytes / 16 + P - 1) / P * 32) < (logits ? 2 : 4)) P *= 2;
+    BwdTeamCfg c;
+    if (!team_cluster(di, P) || !bwd_team_config(di, op, dtype, 64LL * di.sm_count, cols, P, &c)) return 0;
+    if (!logits) return many && bytes > kBwdTeamMaxBytes ? P : 0;
+    const float fill = static_cast<float>(c.stages * c.teams * ((cols * dtype_size(dtype) / 16 + P - 1) / P) * 32) /
+                       static_cast<float>(di.smem_optin);
+    const bool wide = bytes > kStagedMax, two = 2 * rows >= 3LL * di.sm_count;
+    bool pays;
+    if (f32)
+        pays = grid ? wide : many || wide || (two && bytes > 131072);
+    else if (grid && wide)
+        pays = fill > (many ? 0.65f : c.teams == 1 ? 0.6f : 0.0f);
+    else if (grid) {
+        BwdCfg staged;  // its two row buffers, over the CTAs that plan_bwd_for takes
+        pays = many && (fill > 0.55f || !bwd_config(di, cols, dtype_size(dtype), bytes <= 131072 ? 2 : 4, 2, false, &staged));
+    }
+    else
+        pays = fill > (many   ? (c.teams == 1 ? 0.7f : P <= 4 ? 0.45f : 0.51f)
+                       : wide ? 0.7f
+                              : two && bytes > 131072 ? 0.8f : 1.0f);
+    return pays ? P : 0;
 }
 
 // a and dy at one phase of the 16-byte grid (k_bwd_team cuts both arrays alike)

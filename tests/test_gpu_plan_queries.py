@@ -137,3 +137,14 @@ def test_rows_over_warps_are_planned_by_their_buffers(op, dt, rows, nbytes, warp
     """Both sides of the planner's lines: how many warps' buffers a row takes, and how full they are."""
     p = C.plan(op, rows, nbytes // SIZE[dt], dt, C.INT8 if op == C.QUANT_INT8 else None)
     assert (p.retain == C.RETAIN_WARPS) == warps
+
+
+@pytest.mark.parametrize("dt,rows,nbytes,P", [
+    (C.BF16, 1300, 66 << 10, 2), (C.BF16, 1300, 112 << 10, 0), (C.BF16, 1300, 116 << 10, 4), (C.BF16, 1300, 192 << 10, 4),
+    (C.BF16, 1300, 224 << 10, 0), (C.BF16, 1300, 256 << 10, 8), (C.BF16, 1300, 264 << 10, 0), (C.BF16, 1300, 300 << 10, 8),
+    (C.BF16, 300, 192 << 10, 0), (C.BF16, 300, 300 << 10, 8), (C.F32, 1300, 256 << 10, 0), (C.F32, 1300, 264 << 10, 8),
+    (C.F32, 300, 420 << 10, 16), (C.F32, 1300, 1000 << 10, 0)])
+def test_logits_rows_over_clusters_are_planned_by_their_slices(dt, rows, nbytes, P):
+    """Both sides of the backward planner's lines: how much of shared memory the slices in flight fill."""
+    p = C.plan_bwd(C.XENT_BWD, rows, nbytes // SIZE[dt], dt)
+    assert (p.cluster_size if p.retain == C.RETAIN_ROW else 0) == P
