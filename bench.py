@@ -189,8 +189,8 @@ def time_events(fn, reps, warm=1):
 
 
 def candidates(C, op, x, y, g=None, b=None, fills=True, **kw):
-    """Every legal plan of one call: one-CTA / cluster P = 2..16 in both retention tiers, fills of cluster
-    plans that leave SMs idle, two-pass G = 1, 2, 4, 8."""
+    """Every legal plan of one call: one-CTA / cluster P = 2..16 in both retention tiers, as whole rows and over
+    warps, fills of cluster plans that leave SMs idle, two-pass G = 1, 2, 4, 8."""
     import torch
     sm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     kw = dict(kw, gamma=g, beta=b)
@@ -203,6 +203,14 @@ def candidates(C, op, x, y, g=None, b=None, fills=True, **kw):
                 name = f"{'one_cta' if P == 1 else 'cluster'}{'' if P == 1 else P}{tag}"
                 out.append((name, p))
                 legal.append((name, retain, p))
+        path, base = (C.PATH_ONE_CTA, "one_cta") if P == 1 else (C.PATH_CLUSTER, f"cluster{P}")
+        p = C.make_plan(path, P, retain=C.RETAIN_ROW)  # rows that do not fit would run as AUTO
+        if C.plan_kernel(op, x, y, p, **kw) == "k_row_team":
+            out.append((f"{base}_row", p))
+        for W in (8, 16):
+            p = C.make_plan(path, P, retain=C.RETAIN_WARPS, threads=32 * W)
+            if C.plan_check(op, x, y, p, **kw) == C.OK:
+                out.append((f"{base}_w{W}", p))
         if fills and P > 1 and legal:  # fills of a cluster plan that leaves SMs idle
             name, retain, p = legal[-1]
             if sm - P * C.max_clusters(op, x, y, p, **kw) >= 16:
@@ -516,7 +524,8 @@ def run_ours(args):
             os.environ["CREDIT_MODEL"] = "analytic"
             ap_ = C.plan(j["op"], ROWS, j["cols"], C.F32)
             os.environ.pop("CREDIT_MODEL", None)
-            cl = [v for n, v in times.items() if n.startswith("cluster") and not n.endswith("_tm")]
+            cl = [v for n, v in times.items()
+                  if n.startswith("cluster") and not n.endswith(("_tm", "_row", "_w8", "_w16"))]
             pick_rows.append({"op": j["name"], "cols": j["cols"], "chosen_ms": chosen,
                               "best": min(times, key=times.get), "best_ms": round(best_all, 4),
                               "best_non_dsmem_ms": round(best_non, 4), "hit": hit,
@@ -632,6 +641,7 @@ def run_bwd_bench(C, torch, dev, synth):
             cands = [(f"two_pass_g{G}", C.make_plan(C.PATH_TWO_PASS, ctas_per_row=G)) for G in (1, 2, 4, 8)]
             cands.append(("one_cta", C.make_plan(C.PATH_ONE_CTA)))
             cands += [(f"cluster{P}", C.make_plan(C.PATH_CLUSTER, P)) for P in (2, 4, 8, 16)]
+            cands += [(f"cluster{P}_row", C.make_plan(C.PATH_CLUSTER, P, retain=C.RETAIN_ROW)) for P in (2, 4, 8, 16)]
             times = {}
             for cname, p in cands:
                 if C.bwd_plan_check(op, a_, dy_, dx, p, **kw) != C.OK:
@@ -643,11 +653,8 @@ def run_bwd_bench(C, torch, dev, synth):
             non = {k: v for k, v in times.items() if k.startswith("two_pass")}
             staged = {k: v for k, v in times.items() if not k.startswith("two_pass")}
             best_non = min(non.values())
-            pname = (PATH_NAMES_SHORT[chosen_plan.path] +
-                     (str(chosen_plan.cluster_size) if chosen_plan.path == C.PATH_CLUSTER else
-                      (f"_g{chosen_plan.ctas_per_row}" if chosen_plan.path == C.PATH_TWO_PASS else "")))
             out["shapes"].append({
-                "op": name, "cols": cols, "bytes_per_elem": nbytes // (ROWS * cols), "chosen": pname,
+                "op": name, "cols": cols, "bytes_per_elem": nbytes // (ROWS * cols), "chosen": plan_name(C, chosen_plan),
                 "chosen_ms": round(chosen, 4),
                 "chosen_GBps": round(nbytes / chosen / 1e6, 1), "frac": round(nbytes / chosen / 1e6 / peak, 4),
                 "best": min(times, key=times.get), "best_ms": round(min(times.values()), 4),
@@ -672,7 +679,7 @@ def plan_name(C, p):
     if p.path == C.PATH_TWO_PASS:
         return f"two_pass_g{p.ctas_per_row}"
     base = "one_cta" if p.path == C.PATH_ONE_CTA else f"cluster{p.cluster_size}"
-    tag = "_tm" if p.retain == C.RETAIN_TMEM else ""
+    tag = {C.RETAIN_TMEM: "_tm", C.RETAIN_ROW: "_row", C.RETAIN_WARPS: f"_w{(p.threads or 512) // 32}"}.get(p.retain, "")
     return base + tag + (f"_f{round(p.fill_share, 2)}" if p.fill_share > 0 else "")
 
 
@@ -905,9 +912,6 @@ def run_controls_bench(C, torch, dev, synth):
     out["peak_GBps"], out["peak_source"] = peak, peak_kind
     assert C.device_error() == C.OK
     return out
-
-
-PATH_NAMES_SHORT = {0: "one_cta", 1: "two_pass", 2: "cluster"}
 
 
 def profitability(pick_rows):
