@@ -28,8 +28,10 @@ x {16K, 64K, 128K, 256K} FP32; `quant_int8`: row-wise int8 quantisation of
 rows against the oracle; `ragged`: 20000 BF16 rows of log-uniform width in one
 graph-replayed persistent launch; `controls`: the screen's negative controls
 (row scan, row stencil) planned and timed on the global path.  In every table each candidate plan is
-timed beside the planner's pick (outside the timed step).  `summary`, last on
-the line, repeats each table's headline figures.
+timed beside the planner's pick (outside the timed step).  The line on stdout
+carries each table's headline figures (`summary`, last on it), so that it stays
+a few KiB long; the tables themselves (`picks`, `backward`, `quant_int8`,
+`precision`, `ragged`, `controls`) are one JSON line on stderr.
 
 --impl reference  times the FP64 CPU oracle (the reference arm of this
            project) on a bounded sample of the same workload.
@@ -570,13 +572,9 @@ def run_ours(args):
         "profitability": profitability(pick_rows) if pick_rows else None,
         "pick_rule": "chosen plan within 5% of the fastest measured candidate (median of 5)",
         "per_job": per_job,
-        "picks": pick_rows,
-        "backward": bwd,
-        "quant_int8": quant,
-        "precision": prec,
-        "ragged": ragged,
-        "controls": controls,
     }
+    tables = {"picks": pick_rows, "backward": bwd, "quant_int8": quant, "precision": prec, "ragged": ragged,
+              "controls": controls}
     # the headline figures of every table, last on the line
     line["summary"] = {
         "forward": {"GBps": round(value, 1), "frac": round(value / roofline["peak"], 4),
@@ -595,8 +593,14 @@ def run_ours(args):
         "controls": None if controls is None else {
             "screen": controls["screen"], "GBps": {f"{r['op']}_{r['cols']}": r["GBps"] for r in controls["shapes"]}},
         "e2e_frac_of_link": None if e2e is None else e2e["frac_of_link_both"]}
-    print(json.dumps(line), flush=True)
+    emit(line, tables)
     return 0
+
+
+def emit(line, tables):
+    """The result line on stdout (short enough to be read from the end of a log), the tables on stderr."""
+    print(json.dumps({"tables": tables}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
 
 
 BWD_WIDTHS = [16384, 65536, 131072, 262144]

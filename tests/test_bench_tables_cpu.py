@@ -47,3 +47,12 @@ def test_whole_rows_in_one_cta_are_no_dsmem_plans():
     r = bench.table_row("softmax", 4096, 1e9, {"one_cta_row": 1.0, "one_cta_w16": 1.5, "cluster4_row": 0.9, "two_pass_g1": 2.0},
                         1.0, "one_cta_row", 6800.0)
     assert r["best_non_dsmem_ms"] == 1.0 and r["speedup_vs_best_non_dsmem"] == 1.0 and r["best"] == "cluster4_row"
+
+
+def test_tables_stay_off_the_result_line(capsys):
+    import json
+    tables = {"backward": {"shapes": [{"candidates": {f"c{i}": 0.1234 for i in range(30)}} for _ in range(28)]}}
+    bench.emit({"metric": "m", "value": 1.0}, tables)
+    out, err = capsys.readouterr()
+    assert json.loads(out) == {"metric": "m", "value": 1.0} and out.count("\n") == 1
+    assert json.loads(err)["tables"] == tables
