@@ -836,7 +836,6 @@ credit_status run_with_plan(int device, const credit_args *a, const credit_plan_
             }
             RowArgs r = base;
             r.ring = gc.stages;
-            r.affine_resident = gc.affine_resident;
             void *args[] = {&r};
             const cudaError_t e = launch(fn, dim3(static_cast<unsigned>(grid * P)), dim3(gc.threads, gc.teams),
                                          static_cast<size_t>(gc.smem), P, s, args);

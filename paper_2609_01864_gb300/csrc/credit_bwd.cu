@@ -1089,6 +1089,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
     const int T = blockDim.x, t = threadIdx.x, team = threadIdx.y, teams = blockDim.y, S = p.nbuf;
     const int N = static_cast<int>(p.cols);
     const int P = CL ? static_cast<int>(cluster_nctarank()) : 1, c = CL ? static_cast<int>(cluster_ctarank()) : 0;
+    static_assert(!CL || kLogits<OP> || OP == BOP_SOFTMAX, "over a cluster the plain sums exchange one");
     const int lp = CL ? 31 - __clz(P) : 0;   // P is a power of two
     const int gmax = (N / V + P - 1) >> lp;  // groups of a row's slice are at most this many
     uint64_t *full = reinterpret_cast<uint64_t *>(smem) + team * kTeamMaxStages;
@@ -1592,7 +1593,7 @@ credit_plan_t bwd_row_plan(int P) {
 // different phases of the 16-byte grid, or no room for a row of both arrays.
 struct BwdTeamCfg {
     int P, threads, teams, stages, grid;
-    bool grid_rows, gamma_smem;
+    bool gamma_smem;
     long long smem;
 };
 bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, int P, BwdTeamCfg *out) {
@@ -1632,7 +1633,6 @@ bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, lo
     r.smem = ctrl + (r.gamma_smem ? aff : 0) + r.stages * stage;
     const long long ctas = (rows + r.teams - 1) / r.teams;
     r.grid = static_cast<int>(ctas < walkers ? ctas : walkers);
-    r.grid_rows = false;
     *out = r;
     return true;
 }

@@ -1,9 +1,11 @@
-// credit_row_team.cuh -- the one-CTA staged path for rows of up to ~100 KiB, several rows per SM at once.
+// credit_row_team.cuh -- whole rows in shared memory, several per SM at once: rows of one CTA (up to ~100 KiB), or the
+// slices of rows split over a cluster (up to 1 MiB as planned).
 //
-// k_row_team is the staged method (one HBM read and one write, Eq. 4) with
-// whole rows in shared memory and no roles: one persistent CTA of up to 1024
-// threads per SM is split into teams of T threads (about four 16-byte groups
-// of the row per thread); a team walks rows g, g + teams, ...
+// k_row_team is the staged method (one HBM read and one write, Eq. 4) without
+// roles: one persistent CTA of up to 1024 threads per SM is split into teams of
+// T threads (four to eight 16-byte groups of the row per thread); a team walks
+// rows g, g + teams, ...  Over a cluster the teams of one number hold a row's
+// slices and exchange their partials over DSMEM (Eq. 5).
 //
 //   - bulk-async copies bring rows into the team's S shared-memory stages;
 //     a stage takes its next row as soon as the team is done with it (at the
@@ -18,9 +20,13 @@
 // and k_tp_fused waits for its loads once per CTA and row.
 //
 // gamma / beta sit in shared memory once per SM when they fit beside the
-// stages (any row phase: they are indexed by column).  Rows off the 16-byte
-// grid are cut as everywhere (Eq. 2 with P = 1); their head and tail elements
-// are held one per thread and loaded one row ahead.
+// stages (any row phase: they are indexed by column; a cluster's CTA holds its
+// slice's).  Rows off the 16-byte grid are cut as everywhere (Eq. 2); their
+// head and tail elements are held one per thread and loaded one row ahead.  A
+// row without a whole group asks for no copy and waits for none, while the
+// stages' phases go on with the rows: rows of one team all have a group or all
+// have none, since rows that short make 32 teams wherever a team has a second
+// row, and a team's rows then lie a multiple of 32 apart, at one phase.
 //
 // A second look at the row is a shared-memory read, so the statistics take two
 // local steps: softmax the maximum first and then each exponential, LayerNorm

@@ -224,9 +224,8 @@ __device__ __forceinline__ void load_affine(const float *p, long long i0, bool v
 }
 
 // V floats from i0 on of an array of N in global memory (L1 / L2; a null array
-// is all dflt), as
-// aligned vectors shifted by their phase: no vector that reaches outside it is read (such a group loads its
-// elements one by one).
+// is all dflt), as aligned vectors shifted by their phase: no vector that
+// reaches outside it is read (such a group loads its elements one by one).
 template <int V>
 __device__ __forceinline__ void ldg_shift(const float *p, long long i0, long long N, float dflt, float (&v)[V]) {
     if (p == nullptr) {
