@@ -58,3 +58,52 @@ def test_eager_and_captured_calls_overlap(op, tin, tout, rows, cols):
     assert C.device_error() == C.OK
     for (_, outs), w in zip(cs, want):
         assert all(torch.equal(a, b) for a, b in zip(outs, w))
+
+
+MANY = r"""
+import ctypes, sys, torch
+from paper_2609_01864_gb300 import credit as C
+C.init()
+x = torch.randn(8, 120001, device="cuda") * 3
+want, y = torch.empty_like(x), torch.empty_like(x)
+split = C.make_plan(C.PATH_TWO_PASS, ctas_per_row=3)
+C.run_ex(C.SOFTMAX, x, want, plan=split)
+whole = torch.empty_like(x)
+C.run_ex(C.SOFTMAX, x, whole, plan=C.make_plan(C.PATH_TWO_PASS))
+torch.cuda.synchronize()
+rt = ctypes.CDLL(next(l.split()[-1] for l in open("/proc/self/maps") if "libcudart" in l))
+for k in range(560):  # more streams than workspaces: the one used longest ago goes to the new one
+    s = ctypes.c_void_p()
+    assert rt.cudaStreamCreateWithFlags(ctypes.byref(s), 1) == 0
+    y.zero_()
+    torch.cuda.synchronize()
+    C.run_ex(C.SOFTMAX, x, y, plan=split, stream=s.value)
+    assert rt.cudaStreamSynchronize(s) == 0 and rt.cudaStreamDestroy(s) == 0
+    assert torch.equal(y, want), k
+n = torch.randn(40, 300001, device="cuda").bfloat16()
+g = torch.ones(300001, device="cuda")
+p = C.plan(C.LAYERNORM, 40, 300001, C.BF16)
+assert p.path == C.PATH_TWO_PASS and p.ctas_per_row > 1
+ref = torch.layer_norm(n.double(), (300001,)).float()
+z = torch.empty_like(n)
+for k in range(530):  # more captures than workspaces: a planned call then runs one CTA per row
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        C.run_ex(C.LAYERNORM, n, z, gamma=g)
+    if k % 40 == 0 or k > 505:
+        z.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert (z.float() - ref).abs().max().item() <= 2.0 ** -6 * ref.abs().max().item(), k
+assert C.device_error() == C.OK
+print("ok")
+"""
+
+
+def test_more_streams_and_captures_than_workspaces():
+    """In a process of its own: captured calls keep their workspaces for good."""
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", MANY], capture_output=True, text=True, timeout=300,
+                       cwd=__import__("pathlib").Path(C.__file__).resolve().parents[1])
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
