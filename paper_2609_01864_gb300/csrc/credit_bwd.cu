@@ -1657,9 +1657,10 @@ bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, lo
 //     0.87-0.98); with fewer than four rows per SM above 256 KiB from 0.7 on
 //     0.95-1.25, two per SM of narrower ones from 0.8 on 1.06 (0.90-0.93 below).
 //   - FP32 on the grid beyond the staged kernel's reach 0.99-1.63, within it
-//     0.69-1.14; off the grid from four rows per SM on 1.0-1.46, with two per SM
-//     above 128 KiB 0.99-1.21, with one per SM only above 256 KiB 1.0-1.39 (160
-//     KiB 0.72).
+//     0.69-1.14; off the grid from four rows per SM on 1.0-1.46, with fewer above
+//     128 KiB 0.99-1.39 from two per SM on, 0.72-0.96 with one per SM up to 256
+//     KiB, where its sums about the row's maximum err half as much as the split
+//     path's online states (160 and 224 KiB, 8e-8 of dx against 1.1e-7 to 1.5e-7).
 // Rows of which no cluster holds two slices take the two-pass path (1000 KiB
 // 883 us against 1201).  Softmax from its output, off the grid only (on it the
 // staged kernel is at the copy rate), not few rows (300 x 100 KiB FP32 19
@@ -1669,9 +1670,10 @@ bool bwd_team_config(const DeviceInfo &di, int op, int dtype, long long rows, lo
 // the pair ops lose or stay level at most widths.
 int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, long long cols, bool grid) {
     const long long bytes = cols * dtype_size(dtype), kStagedMax = 4 * 65536;  // plan_bwd_for: P <= 4, 64 KiB slices
-    const bool logits = op == BOP_SMLOGITS || op == BOP_XENT, f32 = dtype == CREDIT_F32, many = rows >= 4LL * di.sm_count;
-    if (bytes <= (grid ? bwd_team_bytes(op) : f32 ? 65536 : kBwdTeamMaxBytes) || (!logits && (op != BOP_SOFTMAX || grid)))
-        return 0;
+    const bool logits = op == BOP_SMLOGITS || op == BOP_XENT, f32 = dtype == CREDIT_F32;
+    const bool many = rows >= 4LL * di.sm_count;
+    if (!logits && (op != BOP_SOFTMAX || grid)) return 0;
+    if (bytes <= (grid ? bwd_team_bytes(op) : f32 ? 65536 : kBwdTeamMaxBytes)) return 0;
     const long long room = di.smem_optin - bwd_team_ctrl(kTeamMaxThreads / 16, 16, true);
     int P = logits ? 2 : 16;
     while (team_cluster(di, P) && room / ((bytes / 16 + P - 1) / P * 32) < (logits ? 2 : 4)) P *= 2;
@@ -1683,14 +1685,14 @@ int bwd_row_cluster(const DeviceInfo &di, int op, int dtype, long long rows, lon
     const bool wide = bytes > kStagedMax, two = 2 * rows >= 3LL * di.sm_count;
     bool pays;
     if (f32)
-        pays = grid ? wide : many || wide || (two && bytes > 131072);
+        pays = grid ? wide : many || bytes > 131072;
     else if (grid && wide)
         pays = fill > (many ? 0.65f : c.teams == 1 ? 0.6f : 0.0f);
     else if (grid) {
         BwdCfg staged;  // its two row buffers, over the CTAs that plan_bwd_for takes
-        pays = many && (fill > 0.55f || !bwd_config(di, cols, dtype_size(dtype), bytes <= 131072 ? 2 : 4, 2, false, &staged));
-    }
-    else
+        pays = many &&
+               (fill > 0.55f || !bwd_config(di, cols, dtype_size(dtype), bytes <= 131072 ? 2 : 4, 2, false, &staged));
+    } else
         pays = fill > (many   ? (c.teams == 1 ? 0.7f : P <= 4 ? 0.45f : 0.51f)
                        : wide ? 0.7f
                               : two && bytes > 131072 ? 0.8f : 1.0f);
