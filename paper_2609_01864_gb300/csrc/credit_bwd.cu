@@ -1057,8 +1057,9 @@ __device__ __forceinline__ void team_sums(float (&v)[K], float *red, int bar, in
 
 // Does an element of the warp lie so far below the row's maximum that its exponential is no normal number?  d: the
 // smallest element of each lane less the maximum.  ex2.ftz gives 0 for those; such warps take exp_fast, which the
-// other backward paths use throughout (its range handling costs three instructions per element).  Looking for them
-// costs 2% (4096 x 131072 BF16 cross entropy 784 -> 798 us); exponentials raised by 2^24 for all elements, as in the
+// other backward paths use throughout (its range handling costs three instructions per element), in loops of their own
+// that the compiler lays out of the way (in line 798 us for the case below).  Looking for them costs 1% (4096 x 131072
+// BF16 cross entropy 782 -> 791 us); exponentials raised by 2^24 for all elements, as in the
 // forward softmax, would cost less but round the exponents near 0 three times as coarsely.
 __device__ __forceinline__ bool reaches_subnormal(float d) {
     return __any_sync(0xffffffffu, d * kLog2e < -126.0f) != 0;
@@ -1239,10 +1240,19 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         };
 
         Coef kc;
+        // norms: rows of an ordinary scale sum (x - mean) g and apply rstd^2 to it; in others a sum or rstd^2 could
+        // leave FP32, and x-hat is formed first, as on the other paths (a multiply per element and look, 4% of the
+        // time off the grid if all rows paid it, and a rounding more)
+        const bool ordinary = !kNorm<OP> || (R.rstd > 0x1p-16f && R.rstd < 0x1p16f);
         float lo = 0.0f;  // logits: the smallest of this thread's elements and 0 (edges apart)
         if constexpr (!kLogits<OP> && !kPair<OP>) {
             float2 s0 = f2(0.0f), s1 = f2(0.0f);
-            each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+            if (__builtin_expect(!ordinary, 0)) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+                times_gamma(gi, fd);
+#pragma unroll
+                for (int v = 0; v < V; ++v) R.acc(fa[v], fd[v], 1.0f, s0.x, s1.x);
+            });
+            else each([&](int gi, float (&fa)[V], float (&fd)[V]) {
                 times_gamma(gi, fd);
 #pragma unroll
                 for (int v = 0; v < V; v += 2) {
@@ -1252,14 +1262,13 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                         x = __fadd2_rn(x, f2(-R.mean));
                         s0 = __fadd2_rn(s0, d);
                     }
-                    if constexpr (kNorm<OP>) x = __fmul2_rn(x, f2(R.rstd));  // xh: in range whatever the row's scale
                     s1 = __ffma2_rn(x, d, s1);
                 }
             });
             float v[2] = {s1.x + s1.y, s0.x + s0.y};
             if (edge) {
                 const float d = ed * eg;
-                v[0] = fmaf((OP == BOP_LN ? ea - R.mean : ea) * R.rstd, d, v[0]);  // softmax: rstd 1
+                v[0] = fmaf((OP == BOP_LN ? ea - R.mean : ea) * (ordinary ? 1.0f : R.rstd), d, v[0]);
                 v[1] += d;
             }
             if constexpr (OP == BOP_LN) {
@@ -1270,7 +1279,7 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                 v[0] = v1[0];
             }
             if constexpr (CL) v[0] = warp_sum(exchange(make_float4(v[0], 0.0f, 0.0f, 0.0f)).x);
-            kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], v[0], N);
+            kc = OP == BOP_SOFTMAX ? row_coeffs<OP>(v[0], 0.0f, N) : row_coeffs<OP>(v[1], ordinary ? v[0] * R.rstd : v[0], N);
         } else if constexpr (kLogits<OP>) {
             GroupMax<DT, false> gm;
             LowestBits<DT> gl;
@@ -1289,16 +1298,15 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
             float2 sS = f2(0.0f), sT = f2(0.0f);
             // a term below the normal numbers counts in T beside a large dy (in S it does not)
             const bool low = OP == BOP_SMLOGITS && reaches_subnormal(lo - mz);
-            each([&](int, float (&fa)[V], float (&fd)[V]) {
-                if (low) {
+            if (__builtin_expect(low, 0)) each([&](int, float (&fa)[V], float (&fd)[V]) {
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        const float e = exp_fast(fa[v] - mz);
-                        sS.x += e;
-                        sT.x = fmaf(e, fd[v], sT.x);
-                    }
-                    return;
+                for (int v = 0; v < V; ++v) {
+                    const float e = exp_fast(fa[v] - mz);
+                    sS.x += e;
+                    sT.x = fmaf(e, fd[v], sT.x);
                 }
+            });
+            else each([&](int, float (&fa)[V], float (&fd)[V]) {
 #pragma unroll
                 for (int v = 0; v < V; v += 2) {
                     const float2 x = __fmul2_rn(__fadd2_rn(make_float2(fa[v], fa[v + 1]), f2(-mz)), f2(kLog2e));
@@ -1388,19 +1396,20 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
         if constexpr (!kLogits<OP> && !kPair<OP>) refill();
 
         // ---- gradients
-        const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
+        const float k0 = -R.rstd * kc.c0, k1 = -R.rstd * R.rstd * kc.c1;  // norms: rstd (g - c0 - xh c1)
         const size_t at = off + g.h0 * isz + g.lo * 16;
         unsigned char *xr = p.dx + at;
         unsigned char *xr2 = kPair<OP> ? p.dx2 + at : nullptr;
         const bool vec = GRID || ((reinterpret_cast<uintptr_t>(xr) | reinterpret_cast<uintptr_t>(xr2)) & 15u) == 0;
-        const bool low = kLogits<OP> && reaches_subnormal(lo - kc.c0);
-        if (low) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+        const bool general = kLogits<OP> ? reaches_subnormal(lo - kc.c0) : !ordinary;
+        if (__builtin_expect(general, 0)) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
             float y[V];
+            times_gamma(gi, fd);
 #pragma unroll
-            for (int v = 0; v < V; ++v) y[v] = kLogits<OP> ? R.dx(fa[v], fd[v], 1.0f, kc) : 0.0f;
+            for (int v = 0; v < V; ++v) y[v] = kPair<OP> ? 0.0f : R.dx(fa[v], fd[v], 1.0f, kc);
             store_group<DT, V>(xr + 16 * gi, y, vec);
         });
-        if (!low) each([&](int gi, float (&fa)[V], float (&fd)[V]) {
+        else each([&](int gi, float (&fa)[V], float (&fd)[V]) {
             float y[V];
             if constexpr (kPair<OP>) {
                 float y2[V];
@@ -1424,8 +1433,8 @@ __global__ void __launch_bounds__(kTeamMaxThreads, 1) k_bwd_team(const BwdArgs p
                             r = __fmul2_rn(f2(R.w), __ffma2_rn(e, f2(kc.c1), make_float2(-d.x, -d.y)));
                         }
                     } else {
-                        const float2 xh = __fmul2_rn(OP == BOP_LN ? __fadd2_rn(x, f2(-R.mean)) : x, f2(R.rstd));
-                        r = __ffma2_rn(d, f2(R.rstd), __ffma2_rn(xh, f2(k1), f2(k0)));
+                        const float2 xm = OP == BOP_LN ? __fadd2_rn(x, f2(-R.mean)) : x;
+                        r = __ffma2_rn(d, f2(R.rstd), __ffma2_rn(xm, f2(k1), f2(k0)));
                     }
                     y[v] = r.x;
                     y[v + 1] = r.y;
